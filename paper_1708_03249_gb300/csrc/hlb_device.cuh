@@ -339,42 +339,48 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// WENO-5 face value from a stencil already divided by the population's
-// weight (values O(1) wherever the population matters), without epsilon
-// (Sec. IV.C.2), face between c and d of the upwind-ordered stencil a..e:
-// - the candidates relative to c, q_k = c + R_k / 6, with R_1 = 2a - 7b + 5c,
-//   R_2 = 2d - b - c, R_3 = 5d - 4c - e, and the indicators' t_k, s_k, all from
-//   the differences of neighbouring stencil values;
-// - the indicators scaled by 12/13, B_k = t_k^2 + (3/13) s_k^2 (a common factor
-//   leaves the weights unchanged), with an additive floor of 1e-30, below which
-//   FP32 cannot resolve them anyway;
-// - the nonlinear weights from the ratios u_k = min_j B_j / B_k in (0, 1], so
-//   nothing overflows, and a zero B_k takes the limit of Tab. "weno" (the
-//   zero-indicator stencils share the weight in proportion to d_k);
-// - face = c + (v_1 R_1 + 6 v_2 R_2 + 3 v_3 R_3) / (6 (v_1 + 6 v_2 + 3 v_3)) with
-//   v_k = u_k^2: the linear weights (0.1, 0.6, 0.3) scaled by 10, so the
-//   denominator is at least 1.
-// The packed form below needs six constants (f32x2 instructions take no
-// immediates).  The scalar form performs the same roundings in the same
-// order (explicit _rn operations, no contraction), so a face gives the same
-// bits in either form: the wall kernel's incident flux is the stage kernels'.
+// WENO-5 face values from stencils already divided by the population's weight
+// (values O(1) wherever the population matters), without epsilon (Sec.
+// IV.C.2), face between c and d of the upwind-ordered stencil a..e, in terms
+// of the first differences d1 = b - a .. d4 = e - d and the second differences
+// s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3:
+// - the candidates relative to c, q_k = c + R_k / 6: R_1 = 2 s1 + 3 d2,
+//   R_2 = 2 s2 + 3 d2, R_3 = 3 d3 - s3;
+// - the indicators times 3/4 (a common factor leaves the weights unchanged):
+//   IS = 13/12 s^2 + 1/4 (s +- 2 d)^2 = 4/3 [(s +- 3/8 d)^2 + 39/64 d^2], so
+//   B_1 = (s1 + 3/8 d2)^2 + m(d2), B_2 = (s2 + 3/8 d2)^2 + m(d2), B_3 =
+//   (s3 - 3/8 d3)^2 + m(d3) with m(d) = 39/64 d^2 plus a floor, below which
+//   FP32 cannot resolve an indicator anyway (a zero B_k takes the limit of
+//   Tab. "weno");
+// - the nonlinear weights relative to the second one's, r_k = B_2 / B_k.
+//   B_2 <= C (B_1 + B_3) (a, b, c and c, d, e both smooth leave b, c, d
+//   smooth), so at most one of r_1, r_3 is large; 2^-60 B_2 added to B_1 and
+//   B_3 keeps its square in range and changes no weight that FP32 resolves;
+// - face = c + (w_1 R_1 + R_2 + w_3 R_3) / (6 (w_1 + 1 + w_3)), w_1 = r_1^2 / 6
+//   and w_3 = r_3^2 / 2 the linear weights' ratios folded into r.
+// What the form saves is issue slots, which bound the marching kernels: two
+// reciprocals and no minimum instead of three and two per face, ten packed
+// operations for the indicators instead of fifteen, and what consecutive
+// faces share (d, s, m) is formed once: 29 packed operations and 6 reciprocals
+// per packed face in a row of three instead of 38 and 8.  (The third-difference
+// form R_1 - R_2 saves two more but cancels R_2 beside a jump.)
+// The scalar form performs the same roundings in the same order (explicit _rn
+// operations, no contraction), so a face gives the same bits in either form:
+// the wall kernel's incident flux is the stage kernels'.
+constexpr float kWenoK = 39.0f / 64.0f, kWenoFloor = 8.125e-31f, kWenoEps = 8.673617379884035e-19f,   // 2^-60
+                kWenoR1 = 0.408248290463863f;                                                         // 1 / sqrt(6)
 __device__ __forceinline__ float weno5_scaled(float a, float b, float c, float d, float e) {
-    const float dmm = __fsub_rn(a, b), dm = __fsub_rn(c, b), dp = __fsub_rn(d, c), dpp = __fsub_rn(e, d);
-    const float t1 = __fadd_rn(dm, dmm), s1 = __fmaf_rn(3.0f, dm, dmm);
-    const float t2 = __fsub_rn(dp, dm), s2 = __fadd_rn(dm, dp);
-    const float t3 = __fsub_rn(dpp, dp), s3 = __fmaf_rn(-3.0f, dp, dpp);
-    const float R1 = __fadd_rn(__fadd_rn(t1, s1), dm), R2 = __fadd_rn(s2, dp), R3 = __fsub_rn(dp, s3);
-    constexpr float k = 3.0f / 13.0f, fl = 1e-30f;
-    const float B1 = __fmaf_rn(t1, t1, __fmaf_rn(__fmul_rn(k, s1), s1, fl));
-    const float B2 = __fmaf_rn(t2, t2, __fmaf_rn(__fmul_rn(k, s2), s2, fl));
-    const float B3 = __fmaf_rn(t3, t3, __fmaf_rn(__fmul_rn(k, s3), s3, fl));
-    const float m = fminf(B1, fminf(B2, B3));
-    const float u1 = __fmul_rn(m, rcp_approx(B1)), u2 = __fmul_rn(m, rcp_approx(B2)), u3 = __fmul_rn(m, rcp_approx(B3));
-    const float v1 = __fmul_rn(u1, u1);
-    const float V2 = __fmul_rn(6.0f, __fmul_rn(u2, u2)), V3 = __fmul_rn(3.0f, __fmul_rn(u3, u3));
-    const float den = __fadd_rn(__fadd_rn(v1, V2), V3);
-    const float num = __fmaf_rn(V3, R3, __fmaf_rn(V2, R2, __fmul_rn(v1, R1)));
-    return __fmaf_rn(__fmul_rn(num, 1.0f / 6.0f), rcp_approx(den), c);
+    const float d1 = __fsub_rn(b, a), d2 = __fsub_rn(c, b), d3 = __fsub_rn(d, c), d4 = __fsub_rn(e, d);
+    const float s1 = __fsub_rn(d2, d1), s2 = __fsub_rn(d3, d2), ns3 = __fsub_rn(d3, d4);
+    const float m2 = __fmaf_rn(__fmul_rn(kWenoK, d2), d2, kWenoFloor), m3 = __fmaf_rn(__fmul_rn(kWenoK, d3), d3, kWenoFloor);
+    const float u1 = __fmaf_rn(0.375f, d2, s1), u2 = __fmaf_rn(0.375f, d2, s2), u3 = __fmaf_rn(0.375f, d3, ns3);
+    const float B1 = __fmaf_rn(u1, u1, m2), B2 = __fmaf_rn(u2, u2, m2), B3 = __fmaf_rn(u3, u3, m3);
+    const float r1 = __fmul_rn(__fmul_rn(kWenoR1, B2), rcp_approx(__fmaf_rn(kWenoEps, B2, B1)));
+    const float r3 = __fmul_rn(__fmul_rn(0.5f, B2), rcp_approx(__fmaf_rn(kWenoEps, B2, B3)));
+    const float w1 = __fmul_rn(r1, r1), v3 = __fmul_rn(r3, r3);        // v3 = w_3 / 2
+    const float den = __fmaf_rn(3.0f, w1, __fmaf_rn(6.0f, v3, 3.0f));
+    const float num = __fmaf_rn(v3, __fmaf_rn(3.0f, d3, ns3), __fmaf_rn(w1, __fmaf_rn(1.5f, d2, s1), __fmaf_rn(1.5f, d2, s2)));
+    return __fmaf_rn(num, rcp_approx(den), c);
 }
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
@@ -390,27 +396,36 @@ __device__ __forceinline__ float2 fsub2(float2 a, float2 b) {
     return d;
 }
 
-// Two independent faces at once in the packed FP32 pipe (f32x2 on sm_100+);
-// the arithmetic of weno5_scaled, lane by lane.
-__device__ __forceinline__ float2 weno5_scaled2(float2 a, float2 b, float2 c, float2 d, float2 e) {
-    const float2 dmm = fsub2(a, b), dm = fsub2(c, b), dp = fsub2(d, c), dpp = fsub2(e, d);
-    const float2 t1 = __fadd2_rn(dm, dmm), s1 = __ffma2_rn(f2(3.0f), dm, dmm);
-    const float2 t2 = fsub2(dp, dm), s2 = __fadd2_rn(dm, dp);
-    const float2 t3 = fsub2(dpp, dp), s3 = __ffma2_rn(f2(-3.0f), dp, dpp);
-    const float2 R1 = __fadd2_rn(__fadd2_rn(t1, s1), dm), R2 = __fadd2_rn(s2, dp), R3 = fsub2(dp, s3);
-    const float2 k = f2(3.0f / 13.0f), fl = f2(1e-30f);
-    const float2 B1 = __ffma2_rn(t1, t1, __ffma2_rn(__fmul2_rn(k, s1), s1, fl));
-    const float2 B2 = __ffma2_rn(t2, t2, __ffma2_rn(__fmul2_rn(k, s2), s2, fl));
-    const float2 B3 = __ffma2_rn(t3, t3, __ffma2_rn(__fmul2_rn(k, s3), s3, fl));
-    const float2 m = make_float2(fminf(B1.x, fminf(B2.x, B3.x)), fminf(B1.y, fminf(B2.y, B3.y)));
-    const float2 u1 = __fmul2_rn(m, make_float2(rcp_approx(B1.x), rcp_approx(B1.y)));
-    const float2 u2 = __fmul2_rn(m, make_float2(rcp_approx(B2.x), rcp_approx(B2.y)));
-    const float2 u3 = __fmul2_rn(m, make_float2(rcp_approx(B3.x), rcp_approx(B3.y)));
-    const float2 v1 = __fmul2_rn(u1, u1);
-    const float2 V2 = __fmul2_rn(f2(6.0f), __fmul2_rn(u2, u2)), V3 = __fmul2_rn(f2(3.0f), __fmul2_rn(u3, u3));
-    const float2 den = __fadd2_rn(__fadd2_rn(v1, V2), V3);
-    const float2 num = __ffma2_rn(V3, R3, __ffma2_rn(V2, R2, __fmul2_rn(v1, R1)));
-    return __ffma2_rn(__fmul2_rn(num, f2(1.0f / 6.0f)), make_float2(rcp_approx(den.x), rcp_approx(den.y)), c);
+// NF consecutive faces, two independent rows (or columns) at once in the
+// packed FP32 pipe (f32x2 on sm_100+), the arithmetic of weno5_scaled lane by
+// lane: face f lies between c[f + 2] and c[f + 3] of the upwind-ordered values.
+template <int NF>
+__device__ __forceinline__ void weno5_faces2(const float2 (&c)[NF + 4], float2 (&F)[NF]) {
+    const float2 k = f2(kWenoK), fl = f2(kWenoFloor), eps = f2(kWenoEps);
+    float2 d2 = fsub2(c[2], c[1]), d3 = fsub2(c[3], c[2]);
+    float2 s1 = fsub2(d2, fsub2(c[1], c[0]));
+    float2 m2 = __ffma2_rn(__fmul2_rn(k, d2), d2, fl);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const float2 d4 = fsub2(c[f + 4], c[f + 3]);
+        const float2 s2 = fsub2(d3, d2), ns3 = fsub2(d3, d4);
+        const float2 m3 = __ffma2_rn(__fmul2_rn(k, d3), d3, fl);
+        const float2 u1 = __ffma2_rn(f2(0.375f), d2, s1), u2 = __ffma2_rn(f2(0.375f), d2, s2),
+                     u3 = __ffma2_rn(f2(0.375f), d3, ns3);
+        const float2 B1 = __ffma2_rn(u1, u1, m2), B2 = __ffma2_rn(u2, u2, m2), B3 = __ffma2_rn(u3, u3, m3);
+        const float2 g1 = __ffma2_rn(eps, B2, B1), g3 = __ffma2_rn(eps, B2, B3);
+        const float2 r1 = __fmul2_rn(__fmul2_rn(f2(kWenoR1), B2), make_float2(rcp_approx(g1.x), rcp_approx(g1.y)));
+        const float2 r3 = __fmul2_rn(__fmul2_rn(f2(0.5f), B2), make_float2(rcp_approx(g3.x), rcp_approx(g3.y)));
+        const float2 w1 = __fmul2_rn(r1, r1), v3 = __fmul2_rn(r3, r3);
+        const float2 den = __ffma2_rn(f2(3.0f), w1, __ffma2_rn(f2(6.0f), v3, f2(3.0f)));
+        const float2 num = __ffma2_rn(v3, __ffma2_rn(f2(3.0f), d3, ns3),
+                                      __ffma2_rn(w1, __ffma2_rn(f2(1.5f), d2, s1), __ffma2_rn(f2(1.5f), d2, s2)));
+        F[f] = __ffma2_rn(num, make_float2(rcp_approx(den.x), rcp_approx(den.y)), c[f + 2]);
+        s1 = s2;
+        d2 = d3;
+        d3 = d4;
+        m2 = m3;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -511,6 +526,33 @@ __device__ __forceinline__ uint32_t sr_key(const void* p) {
 
 __device__ __forceinline__ float2 upwind2_face2(float2 b, float2 c) {
     return __ffma2_rn(f2(1.5f), c, __fmul2_rn(f2(-0.5f), b));
+}
+
+// Fluxes per unit velocity at NF consecutive faces, two independent rows at
+// once: face f lies between c[f + 2] and c[f + 3] of c[0 .. NF + 4] (cells in
+// ascending order), upwind for a positive (pos) or negative velocity.
+template <int ADV, int NF>
+__device__ __forceinline__ void packed_faces(bool pos, const float2* c, float2* F) {
+    if (ADV == HLB_WENO5_) {
+        float2 u[NF + 4], r[NF];           // in upwind order
+        if (pos) {
+#pragma unroll
+            for (int j = 0; j < NF + 4; ++j) u[j] = c[j];
+            weno5_faces2<NF>(u, r);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) F[f] = r[f];
+        } else {
+#pragma unroll
+            for (int j = 0; j < NF + 4; ++j) u[j] = c[NF + 4 - j];
+            weno5_faces2<NF>(u, r);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) F[f] = r[NF - 1 - f];
+        }
+    } else {
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+            F[f] = pos ? upwind2_face2(c[f + 1], c[f + 2]) : upwind2_face2(c[f + 4], c[f + 3]);
+    }
 }
 
 __device__ __forceinline__ int find_slot(const int* start, int n, int key) {

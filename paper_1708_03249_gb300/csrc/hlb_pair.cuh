@@ -269,14 +269,6 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         for (int j = 0; j < 6; ++j) w[j] = make_float2(wr[0][j], wr[1][j]);
         w[6] = w[7] = f2(0.0f);
     }
-    // flux per unit velocity at the face between c[2] and c[3] of c[0..5]
-    auto face = [&](bool pos, const float2* c) -> float2 {
-        if (ADV == HLB_WENO5_) {
-            if (pos) return weno5_scaled2(c[0], c[1], c[2], c[3], c[4]);
-            return weno5_scaled2(c[5], c[4], c[3], c[2], c[1]);
-        }
-        return pos ? upwind2_face2(c[1], c[2]) : upwind2_face2(c[4], c[3]);
-    };
     // a cell entering the window at position e (head row pair hd; right-wall
     // ghosts from the cells nx-1, nx-2, nx-3 already in the window)
     auto enter = [&](int h, const float* hd0, const float* hd1, float2 m1, float2 m2, float2 m3,
@@ -287,7 +279,9 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         if (h == nx + 1) return __ffma2_rn(f2(6.0f), m2, __ffma2_rn(f2(-8.0f), m3, __fmul2_rn(f2(3.0f), m4)));
         return f2(0.0f);                                                        // never read by v > 0
     };
-    float2 Fm = __fmul2_rn(vxs, face(xpos, w));
+    float2 Fm;
+    packed_faces<ADV, 1>(xpos, w, &Fm);
+    Fm = __fmul2_rn(vxs, Fm);
 
     // Per pair: wait for its copies; write the centre values to sF[b] and
     // arrive on xch[b]; evaluate the faces (the other warps catch up
@@ -317,8 +311,9 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         __syncwarp();
         if (lane == 0) mbar_arrive(&xch[b]);
         // x faces x0+1/2, x0+3/2 (rows packed); x0-1/2 carried
-        const float2 Fp0 = __fmul2_rn(vxs, face(xpos, w + 1));
-        const float2 Fp1 = __fmul2_rn(vxs, face(xpos, w + 2));
+        float2 Fx[2];
+        packed_faces<ADV, 2>(xpos, w + 1, Fx);
+        const float2 Fp0 = __fmul2_rn(vxs, Fx[0]), Fp1 = __fmul2_rn(vxs, Fx[1]);
         const float2 divx0 = __fmul2_rn(fsub2(Fp0, Fm), f2(invdx[x0]));
         const float2 divx1 = __fmul2_rn(fsub2(Fp1, Fp0), f2(two ? invdx[x0 + 1] : 0.0f));
         Fm = Fp1;
@@ -338,9 +333,10 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         col[4] = make_float2(w[3].y, w[4].y);
 #pragma unroll
         for (int k = 0; k < 3; ++k) col[5 + k] = __fmul2_rn(make_float2(B.halo[0][3 + k][vl], B.halo[1][3 + k][vl]), sv2);
-        const float2 G0 = face(ypos, col), G1 = face(ypos, col + 1), G2 = face(ypos, col + 2);
-        const float2 dy0 = __fmul2_rn(vys, fsub2(G1, G0));   // row y0, cells x0, x0+1
-        const float2 dy1 = __fmul2_rn(vys, fsub2(G2, G1));   // row y0+1
+        float2 Gy[3];
+        packed_faces<ADV, 3>(ypos, col, Gy);
+        const float2 dy0 = __fmul2_rn(vys, fsub2(Gy[1], Gy[0]));   // row y0, cells x0, x0+1
+        const float2 dy1 = __fmul2_rn(vys, fsub2(Gy[2], Gy[1]));   // row y0+1
         // shift the window by two cells
 #pragma unroll
         for (int j = 0; j < 6; ++j) w[j] = w[j + 2];

@@ -331,17 +331,6 @@ __device__ HLB_MARCH_ITEM_ATTR uint32_t march_item(const GroupDev& g, const Pers
 #pragma unroll
         for (int j = 6; j < 10; ++j) w[j] = 0.0f;
     }
-    auto faces2 = [&](const float* c) -> float2 {
-        if (ADV == HLB_WENO5_) {
-            if (xpos)
-                return weno5_scaled2(make_float2(c[0], c[1]), make_float2(c[1], c[2]), make_float2(c[2], c[3]),
-                                     make_float2(c[3], c[4]), make_float2(c[4], c[5]));
-            return weno5_scaled2(make_float2(c[5], c[6]), make_float2(c[4], c[5]), make_float2(c[3], c[4]),
-                                 make_float2(c[2], c[3]), make_float2(c[1], c[2]));
-        }
-        return xpos ? upwind2_face2(make_float2(c[1], c[2]), make_float2(c[2], c[3]))
-                    : upwind2_face2(make_float2(c[4], c[5]), make_float2(c[3], c[4]));
-    };
     auto face1 = [&](const float* c) -> float {
         if (ADV == HLB_WENO5_)
             return xpos ? weno5_scaled(c[0], c[1], c[2], c[3], c[4]) : weno5_scaled(c[5], c[4], c[3], c[2], c[1]);
@@ -371,81 +360,85 @@ __device__ HLB_MARCH_ITEM_ATTR uint32_t march_item(const GroupDev& g, const Pers
         const int b = Pg & 1;
 #pragma unroll
         for (int k = 0; k < 4; ++k) w[6 + k] = enter(x0 + 3 + k, B.head[k], w[5 + k], w[4 + k], w[3 + k], w[2 + k]);
-        const float2 fc01 = __fmul2_rn(make_float2(w[3], w[4]), isv2);
-        const float2 fc23 = __fmul2_rn(make_float2(w[5], w[6]), isv2);
-        sF[(b * VY + jy) * SP + ix] = make_float4(fc01.x, fc01.y, fc23.x, fc23.y);
+        float2 q[7];                                     // cells two apart share a packed register
+#pragma unroll
+        for (int j = 0; j < 7; ++j) q[j] = make_float2(w[j + 1], w[j + 3]);
+        const float2 fcA = __fmul2_rn(q[2], isv2);      // cells x0, x0+2
+        const float2 fcB = __fmul2_rn(q[3], isv2);      // cells x0+1, x0+3
+        sF[(b * VY + jy) * SP + ix] = make_float4(fcA.x, fcA.y, fcB.x, fcB.y);
         __syncwarp();
         if (lane == 0) mbar_arrive(&xch[b]);
-        const float2 Fp01 = __fmul2_rn(vxs, faces2(w + 1));
-        const float2 Fp23 = __fmul2_rn(vxs, faces2(w + 3));
+        float2 Fx[2];
+        packed_faces<ADV, 2>(xpos, q, Fx);
+        const float2 FA = __fmul2_rn(vxs, Fx[0]), FB = __fmul2_rn(vxs, Fx[1]);
         float idx[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) idx[k] = k < n4 ? invdx[x0 + k] : 0.0f;
-        const float2 divx01 = __fmul2_rn(fsub2(Fp01, make_float2(Fm, Fp01.x)), make_float2(idx[0], idx[1]));
-        const float2 divx23 = __fmul2_rn(fsub2(Fp23, make_float2(Fp01.y, Fp23.x)), make_float2(idx[2], idx[3]));
-        Fm = Fp23.y;
+        const float2 divxA = __fmul2_rn(fsub2(FA, make_float2(Fm, FB.x)), make_float2(idx[0], idx[2]));
+        const float2 divxB = __fmul2_rn(fsub2(FB, FA), make_float2(idx[1], idx[3]));
+        Fm = FB.y;
 #pragma unroll
         for (int j = 0; j < 6; ++j) w[j] = w[j + 4];
         if (!mbar_wait(&xch[b], (Pg >> 1) & 1, g.err, g.wait_ns)) *sAbort = 1;
         if (*sAbort) break;
         issue(p + kPDepth - 1);
         const float4* fr = sF + b * VY * SP;
-        float2 fk01 = f2(0.0f), fk23 = f2(0.0f);
+        float2 fkA = f2(0.0f), fkB = f2(0.0f);
         if constexpr (kMMA) {
             mma.run(fr, sKx, sKy);
             __syncwarp();
             if (lane == 0) mbar_arrive(xch2);
             if (!mbar_wait(xch2, Pg & 1, g.err, g.wait_ns)) *sAbort = 1;
             const float4 ex = sKx[jy * SP + ix], ey = sKy[jy * SP + ix];
-            fk01 = __fadd2_rn(make_float2(ex.x, ex.y), make_float2(ey.x, ey.y));
-            fk23 = __fadd2_rn(make_float2(ex.z, ex.w), make_float2(ey.z, ey.w));
+            fkA = __fadd2_rn(make_float2(ex.x, ex.y), make_float2(ey.x, ey.y));
+            fkB = __fadd2_rn(make_float2(ex.z, ex.w), make_float2(ey.z, ey.w));
         } else {
             const float4* kxr = reinterpret_cast<const float4*>(sKd + ix * KXR);
             const float4* kyr = reinterpret_cast<const float4*>(sKd + QX2 * KXR + jy * KYR);
 #pragma unroll
             for (int i = 0; i < QX2; i += 2) {
                 const float4 kk = kxr[i >> 1], fa = fr[jy * SP + i], fb = fr[jy * SP + i + 1];
-                fk01 = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.x, fa.y), fk01);
-                fk23 = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.z, fa.w), fk23);
-                fk01 = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.x, fb.y), fk01);
-                fk23 = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.z, fb.w), fk23);
+                fkA = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.x, fa.y), fkA);
+                fkB = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.z, fa.w), fkB);
+                fkA = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.x, fb.y), fkA);
+                fkB = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.z, fb.w), fkB);
             }
             if (VY > 1) {
 #pragma unroll
                 for (int j = 0; j < VY; j += 2) {
                     const float4 kk = kyr[j >> 1], fa = fr[j * SP + ix], fb = fr[(j + 1) * SP + ix];
-                    fk01 = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.x, fa.y), fk01);
-                    fk23 = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.z, fa.w), fk23);
-                    fk01 = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.x, fb.y), fk01);
-                    fk23 = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.z, fb.w), fk23);
+                    fkA = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.x, fa.y), fkA);
+                    fkB = __ffma2_rn(make_float2(kk.x, kk.y), make_float2(fa.z, fa.w), fkB);
+                    fkA = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.x, fb.y), fkA);
+                    fkB = __ffma2_rn(make_float2(kk.z, kk.w), make_float2(fb.z, fb.w), fkB);
                 }
             }
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {                       // cells x0+2q, x0+2q+1
-            if (2 * q >= n4) break;
-            const float* c0 = B.coef + (2 * q) * NCP;
-            const float* c1 = c0 + NCP;                     // stale beyond n4: its results are not stored
+        for (int h = 0; h < 2; ++h) {                       // cells x0+h, x0+h+2
+            if (h >= n4) break;
+            const float* c0 = B.coef + h * NCP;
+            const float* c1 = c0 + 2 * NCP;                     // stale beyond n4: its results are not stored
             const float2 feq = __fmul2_rn(make_float2(c0[ix], c1[ix]), make_float2(c0[QX2 + jy], c1[QX2 + jy]));
             const float2 itau = make_float2(c0[csrc_t], c1[csrc_t]);
-            const float2 fc = q ? fc23 : fc01;
-            const float2 Lv = __ffma2_rn(fsub2(fc, feq), itau, __fadd2_rn(q ? divx23 : divx01, q ? fk23 : fk01));
+            const float2 fc = h ? fcB : fcA;
+            const float2 Lv = __ffma2_rn(fsub2(fc, feq), itau, __fadd2_rn(h ? divxB : divxA, h ? fkB : fkA));
             float2 out;
             if (g.sround) {      // stochastic rounding of the stage output (hlb_device.cuh)
-                const float2 fo_n = stage > 0 ? make_float2(B.fnr[2 * q][vl], B.fnr[2 * q + 1][vl]) : f2(0.0f);
-                out = rk3_out_sr2(stage, fc, __fmul2_rn(dt2, Lv), fo_n, sr_key(fov + (x0 + 2 * q) * V));
+                const float2 fo_n = stage > 0 ? make_float2(B.fnr[h][vl], B.fnr[h + 2][vl]) : f2(0.0f);
+                out = rk3_out_sr2(stage, fc, __fmul2_rn(dt2, Lv), fo_n, sr_key(fov + (x0 + h) * V));
             } else if (stage == 0) {
                 out = fsub2(fc, __fmul2_rn(dt2, Lv));
             } else {
-                const float2 fo_n = make_float2(B.fnr[2 * q][vl], B.fnr[2 * q + 1][vl]);
+                const float2 fo_n = make_float2(B.fnr[h][vl], B.fnr[h + 2][vl]);
                 // c f^n + (1 - c) f' as f' + c (f^n - f'): the weights sum
                 // to 1 exactly whatever the rounding of c (with 1/3 and 2/3
                 // each rounded, FP32 gains mass 2^-25 per step)
                 const float2 fp = fsub2(fc, __fmul2_rn(dt2, Lv));
                 out = __ffma2_rn(f2(stage == 1 ? 0.75f : 1.0f / 3.0f), fsub2(fo_n, fp), fp);
             }
-            fov[(x0 + 2 * q) * V] = out.x;
-            if (2 * q + 1 < n4) fov[(x0 + 2 * q + 1) * V] = out.y;
+            fov[(x0 + h) * V] = out.x;
+            if (h + 2 < n4) fov[(x0 + h + 2) * V] = out.y;
         }
     }
     if (*sAbort && t == 0) {
