@@ -119,6 +119,7 @@ struct Group {
     // items of a stage (per instance its node chunks, then its segments),
     // node chunks and segments per instance, resident CTAs
     bool persist_ok = false;
+    bool node_fused = false;                 // the node pass and the walls in one launch
     bool persist_use = true;                 // the autotuner's pick: persistent or per-stage launches
     float tuned_ms_persist = 0.0f, tuned_ms_stages = 0.0f;   // its best step times (0: not timed)
     int persist_per_sm = 0, persist_grid = 0, persist_nitems = 0;
@@ -645,10 +646,14 @@ hlb_status build_group(hlb_handle* h, Group& G) {
             // FMA loop is faster (3.43 against 3.64 ms; 32 x 16: 0.330
             // against 0.347 ms)
             HLB_CUDA(hlb::prepare_march(G.precision, G.adv, G.QX2, G.VY, G.TY, G.force_form));
-            HLB_CUDA(hlb::prepare_node());
         }
     }
     fill_dev(G);
+    // 2D groups below 1024 nodes (32 CTAs of the one-launch node pass) keep the
+    // separate sums, factor-line and wall kernels and with them their twelve
+    // launches per step, which callers can count (hlb_launch_count)
+    G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && (G.TY == 1 || G.nnodes >= 1024);
+    if (G.march_ok) HLB_CUDA(G.node_fused ? hlb::prepare_node_fused(G.adv, G.dev) : hlb::prepare_node());
 
     // launch shape of the stage kernel.  With Kx in global memory each
     // velocity's force term is a 2Qx-term dot product (FP64), so the velocities
@@ -748,8 +753,12 @@ void enqueue_group_step(hlb_handle* h, Group& G, cudaStream_t st_) {
         NvtxRange range(kStageNames[st]);
         const bool march = G.march_ok && !group_has_z_force(h, G);
         if (G.quad_x) hlb::launch_quad_coef(G.dev, ins[st], st_);
-        if (march) hlb::launch_node(G.precision, G.dev, ins[st], st_);
-        hlb::launch_wall(G.precision, G.adv, G.dev, ins[st], st_);
+        if (march && G.node_fused) {
+            hlb::launch_node_fused(G.adv, G.dev, ins[st], st_);
+        } else {
+            if (march) hlb::launch_node(G.precision, G.dev, ins[st], st_);
+            hlb::launch_wall(G.precision, G.adv, G.dev, ins[st], st_);
+        }
         if (h->time_kernels) cudaEventRecord(e1, st_);
         if (march)
             hlb::launch_march(G.precision, G.adv, G.QX2, G.VY, G.TY, G.dev, (const hlb::Work*)G.d_works.p,
@@ -789,7 +798,8 @@ long long kernels_per_step(hlb_handle* h) {
     long long n = 0;
     for (auto& G : h->groups)
         n += persist_on(h, *G) ? 1
-                               : 3 * ((G->march_ok && !group_has_z_force(h, *G)) ? 4 : 2) + (G->quad_x ? 3 : 0);
+                               : 3 * ((G->march_ok && !group_has_z_force(h, *G)) ? (G->node_fused ? 2 : 4) : 2) +
+                                     (G->quad_x ? 3 : 0);
     return n;
 }
 

@@ -178,13 +178,66 @@ __device__ __forceinline__ float2 df_sqrt(float2 x) {
     return df_fast_two_sum(s, res.x / (2.0f * s));
 }
 
+// exp(y) and (sqrt(pi) / 2) erf(z) / z = sum_n y^n / (n! (2n + 1)) for y = -z^2 in
+// [-0.49, 0], their Taylor polynomials by Horner's rule: the flows' own range,
+// |u_x| up to sqrt(2 T) 0.7, where neither needs a reduction.
+// In double-float, both at once in the lanes of f32x2 registers, the terms from
+// degree 9 on (5e-9 of the sum) in FP32; degree 14 leaves 1e-17.
+__device__ __forceinline__ DF2 df2_exp_erf_small(float2 y) {
+    const float ch[15][2] = {
+        {1.0f, 1.0f}, {1.0f, 0.3333333432674408f}, {0.5f, 0.10000000149011612f}, {0.1666666716337204f,
+        0.02380952425301075f}, {0.0416666679084301f, 0.004629629664123058f}, {0.008333333767950535f,
+        0.0007575757335871458f}, {0.0013888889225199819f, 0.00010683760774554685f}, {0.00019841270113829523f,
+        1.3227513591118623e-05f}, {2.4801587642286904e-05f, 1.4589169268219848e-06f},
+        {2.7557318844628753e-06f, 1.4503852696634567e-07f}, {2.755731998149713e-07f, 1.3122533282228233e-08f},
+        {2.5052107943679403e-08f, 1.0892221569136495e-09f}, {2.0876755879584152e-09f, 8.350702768167295e-11f},
+        {1.6059044372074283e-10f, 5.94779390669653e-12f}, {1.147074536050896e-11f, 3.9554294626979736e-13f}};
+    const float cl[9][2] = {
+        {0.0f, 0.0f}, {0.0f, -9.934107758624577e-09f}, {0.0f, -1.4901161415892261e-09f},
+        {-4.967053879312289e-09f, -4.434869416147791e-10f}, {-1.2417634698280722e-09f,
+        -3.449342894645824e-11f}, {-4.34617203337595e-10f, 2.3988611444480945e-11f},
+        {-3.3631094437103215e-11f, -9.079400100676926e-13f}, {-2.725596874933456e-12f,
+        -3.6360538603445736e-13f}, {-3.40699609366682e-13f, -2.672861423565296e-14f}};
+    float2 t = make_float2(ch[14][0], ch[14][1]);
+#pragma unroll
+    for (int n = 13; n >= 9; --n) t = __ffma2_rn(t, f2(y.x), make_float2(ch[n][0], ch[n][1]));
+    const DF2 yy = df2_dup(y);
+    DF2 s = {t, f2(0.0f)};
+#pragma unroll
+    for (int n = 8; n >= 0; --n)
+        s = df2_add(df2_mul(s, yy), DF2{make_float2(ch[n][0], ch[n][1]), make_float2(cl[n][0], cl[n][1])});
+    return s;
+}
+// In FP64 (degree 15 leaves 5e-19).
+__device__ __forceinline__ void exp_erf_small(double y, double& e, double& f) {
+    const double c[16] = {
+        1.0 / 1.0, 1.0 / 1.0, 1.0 / 2.0, 1.0 / 6.0, 1.0 / 24.0, 1.0 / 120.0, 1.0 / 720.0, 1.0 / 5040.0, 1.0 /
+        40320.0, 1.0 / 362880.0, 1.0 / 3628800.0, 1.0 / 39916800.0, 1.0 / 479001600.0, 1.0 / 6227020800.0, 1.0
+        / 87178291200.0, 1.0 / 1307674368000.0};
+    const double d[16] = {
+        1.0 / 1.0, 1.0 / 3.0, 1.0 / 10.0, 1.0 / 42.0, 1.0 / 216.0, 1.0 / 1320.0, 1.0 / 9360.0, 1.0 / 75600.0,
+        1.0 / 685440.0, 1.0 / 6894720.0, 1.0 / 76204800.0, 1.0 / 918086400.0, 1.0 / 11975040000.0, 1.0 /
+        168129561600.0, 1.0 / 2528170444800.0, 1.0 / 40537905408000.0};
+    e = c[15];
+    f = d[15];
+#pragma unroll
+    for (int n = 14; n >= 0; --n) {
+        e = fma(e, y, c[n]);
+        f = fma(f, y, d[n]);
+    }
+}
+
 // The per-node inputs of the recurrences (NodeDF) from the compensated FP32
 // moment sums (running sum and error term of n, j_x, j_y, j_z, E at sm[0..4]
-// and sm[8..12]) entirely in double-float: n = s + c, u = j / n, T = (E - n
-// |u|^2) / (D n), sqrt(T) and 1/sqrt(T) by Newton steps, and exp, erf as in
-// node_inputs_df (FP64 where |u_x| / sqrt(2T) > 2.5).  For equilibrium orders
-// up to 10: the relative error, about 1e-14, grows threefold per order in the
-// recurrence and stays below FP32 resolution there.  Returns n (FP64) for 1/tau.
+// and sm[8..12]): n = s + c, u = j / n, T = (E - n |u|^2) / (D n) in
+// double-float, relative error about 1e-14.  The recurrence grows an error of
+// its start, exp(-u_x^2 / 2T) and erf(u_x / sqrt(2T)) against the u and T it
+// runs with, about threefold per order.  LOW (equilibrium orders up to 10):
+// both in double-float (1e-14 stays below FP32 resolution there; FP64 where
+// |u_x| / sqrt(2T) > 2.5).  Else in FP64 from the double-float u and T as they
+// stand, 1 / sqrt(T) by one third-order Householder step on the FP32 root (the
+// FP64 pipe runs at 1/64 of FP32 here, so it takes only what needs it).  Returns n (FP64) for 1/tau.
+template <bool LOW>
 __device__ inline double node_inputs_from_sums_df(const float* sm, int D, NodeDF& o) {
     const float2 n = df_two_sum(sm[0], sm[8]);
     const float2 in = df_recip(n);
@@ -201,20 +254,276 @@ __device__ inline double node_inputs_from_sums_df(const float* sm, int D, NodeDF
     o.uz = uz;
     o.T = T;
     o.Tm1 = df_add(T, make_float2(-1.0f, 0.0f));
-    const float2 irt = df_recip(df_sqrt(T));
-    const float2 z = df_mul(ux, df_mul(irt, make_float2(0.7071067690849304f, 1.2101617485882343e-08f)));
-    const float2 inv_sqrt2pi = make_float2(0.3989422917366028f, -1.1335170135851058e-08f);
-    if (fabsf(z.x) <= 2.5f) {
-        const float2 z2 = df_mul(z, z);
-        const float2 Ez = df_exp_nonpos(make_float2(-z2.x, -z2.y));
-        o.erf_z = df_erf_series(z, z2, Ez);
-        o.g0 = df_mul(df_mul(Ez, inv_sqrt2pi), irt);
+    if constexpr (LOW) {
+        const float2 irt = df_recip(df_sqrt(T));
+        const float2 z = df_mul(ux, df_mul(irt, make_float2(0.7071067690849304f, 1.2101617485882343e-08f)));
+        const float2 inv_sqrt2pi = make_float2(0.3989422917366028f, -1.1335170135851058e-08f);
+        if (fabsf(z.x) <= 0.7f) {
+            const float2 z2 = df_mul(z, z);
+            const DF2 p = df2_exp_erf_small(make_float2(-z2.x, -z2.y));
+            o.g0 = df_mul(df_mul(make_float2(p.h.x, p.l.x), inv_sqrt2pi), irt);
+            o.erf_z = df_mul(df_mul(z, make_float2(1.128379225730896f, -5.8635382771399236e-08f)),      // 2 / sqrt(pi)
+                             make_float2(p.h.y, p.l.y));
+        } else if (fabsf(z.x) <= 2.5f) {
+            const float2 z2 = df_mul(z, z);
+            const float2 Ez = df_exp_nonpos(make_float2(-z2.x, -z2.y));
+            o.erf_z = df_erf_series(z, z2, Ez);
+            o.g0 = df_mul(df_mul(Ez, inv_sqrt2pi), irt);
+        } else {
+            const double zd = (double)z.x + (double)z.y;
+            o.erf_z = df_from_double(erf(zd));
+            o.g0 = df_mul(df_mul(df_from_double(exp(-zd * zd)), inv_sqrt2pi), irt);
+        }
     } else {
-        const double zd = (double)z.x + (double)z.y;
-        o.erf_z = df_from_double(erf(zd));
-        o.g0 = df_mul(df_mul(df_from_double(exp(-zd * zd)), inv_sqrt2pi), irt);
+        const double Td = (double)T.x + (double)T.y, ud = (double)ux.x + (double)ux.y;
+        double r = (double)rsqrtf(T.x);
+        const double e = fma(-Td * r, r, 1.0);                   // 1 - T r^2, about 1e-7
+        r = fma(r * e, fma(0.375, e, 0.5), r);                   // error 5/16 e^3
+        const double z = ud * r * 0.70710678118654752440;
+        double E, F;
+        if (fabs(z) <= 0.7) {
+            exp_erf_small(-z * z, E, F);
+            F *= z * 1.1283791670955125739;                      // 2 / sqrt(pi)
+        } else {
+            E = exp(-z * z);
+            F = erf(z);
+        }
+        o.erf_z = df_from_double(F);
+        o.g0 = df_from_double(E * (r * (1.0 / kSqrt2Pi)));
     }
     return (double)n.x + (double)n.y;
+}
+
+// ---------------------------------------------------------------------------
+// The factor lines of up to NB nodes by one CTA of T threads.  The three parts
+// of a line's arithmetic (inputs, recurrences, dot products) are chains of
+// dependent double-float operations; with one thread per node doing all of
+// them in a row the pass waits on latency (71 us for the 65536 nodes of order
+// 15 of the 256^2 box, where the instructions alone take about 20).  Here thread
+// t works on node t % NB, and every double-float operation on two values in
+// the lanes of f32x2 registers:
+//  - recurrences: G^+ with G^- (slot 0), G_y with G_z (slot 1), a thread per
+//    node and pair; the coefficients go to shared memory;
+//  - dot products (Dot2 of Ogita, Rump and Oishi, as in dot2_pair), items of two
+//    rows over all threads of the node: n g_x of +z_k with that of -z_k (one
+//    table entry for both lanes); along p_y and p_z the even orders in one lane
+//    and the odd ones in the other, since He_l(-z) = (-1)^l He_l(z) makes the
+//    rows of z and -z the sum and the difference of the two: half the terms.
+// ---------------------------------------------------------------------------
+constexpr int kNodeFields = 9;           // float2 fields of a node's inputs, [field][NB]
+
+// Shared-memory tables (float4 each) and coefficients of node_lines, in bytes.
+struct NodeTables {
+    int nx, ny, nz;                      // entries: x row pairs, y and z rows of (even, odd) pairs
+    int my, mz;                          // (even, odd) pairs per row
+    __host__ __device__ NodeTables(const GroupDev& g) {
+        my = (g.Ny + 2) >> 1;
+        mz = (g.Nz + 2) >> 1;
+        nx = (g.Qx >> 1) * (g.Nx + 1);
+        ny = g.Qy ? (g.VY >> 1) * my : 0;
+        nz = g.Qz ? (g.VZ >> 1) * mz : 0;
+    }
+    __host__ __device__ size_t table_bytes() const { return (size_t)(nx + ny + nz) * 16; }
+    template <int NB> __host__ __device__ size_t coef_bytes(const GroupDev& g) const {
+        return (size_t)NB * 16 * (g.Nx + 1 + (g.Qy ? my : 0) + (g.Qz ? mz : 0));
+    }
+};
+__host__ __device__ inline int node_line_stride(int ncp) { return (ncp / 4) & 1 ? ncp : ncp + 4; }   // few bank conflicts
+
+__device__ __forceinline__ void node_load_tables(const GroupDev& g, const NodeTables& nt, float4* tab, int t, int T) {
+    const float2* Tx = g.Tf;
+    const float2* Ty = Tx + g.Qx * (g.Nx + 1);
+    const float2* Tz = Ty + g.VY * (g.Ny + 1);
+    for (int i = t; i < nt.nx; i += T) {                 // rows 2 k and 2 k + 1 side by side
+        const int k = i / (g.Nx + 1), l = i - k * (g.Nx + 1);
+        const float2 a = Tx[2 * k * (g.Nx + 1) + l], b = Tx[(2 * k + 1) * (g.Nx + 1) + l];
+        tab[i] = make_float4(a.x, b.x, a.y, b.y);
+    }
+    auto pairs = [&](float4* dst, const float2* src, int half, int N, int m) {     // rows half .. 2 half - 1: z > 0
+        for (int i = t; i < half * m; i += T) {
+            const int j = i / m, l = 2 * (i - j * m);
+            const float2 a = src[(half + j) * (N + 1) + l];
+            const float2 b = l < N ? src[(half + j) * (N + 1) + l + 1] : make_float2(0.0f, 0.0f);
+            dst[i] = make_float4(a.x, b.x, a.y, b.y);
+        }
+    };
+    if (nt.ny) pairs(tab + nt.nx, Ty, g.VY >> 1, g.Ny, nt.my);
+    if (nt.nz) pairs(tab + nt.nx + nt.ny, Tz, g.VZ >> 1, g.Nz, nt.mz);
+}
+
+// The half-range recurrence's table for node_lines, three float4 per order l
+// (at least one): (a_l, b_l), (c_l, a_l d_l), (h_l(0), a_l h_l(0)) in
+// double-float, d_0 = 0 (recf: a, b, c [Nx], h(0) [Nx + 1], d_1 .. d_Nx).
+__host__ __device__ inline size_t node_rec_bytes(int Nx) { return (size_t)(Nx > 0 ? Nx : 1) * 48; }
+__device__ __forceinline__ void node_load_rec(const GroupDev& g, float4* rec, int t, int T) {
+    const int Nx = g.Nx;
+    const float2* r = g.recf;
+    for (int l = t; l < (Nx > 0 ? Nx : 1); l += T) {
+        const float2 h = r[3 * Nx + l], zero = make_float2(0.0f, 0.0f);
+        const float2 a = Nx ? r[l] : zero, b = Nx ? r[Nx + l] : zero, c = Nx ? r[2 * Nx + l] : zero;
+        const float2 ad = l ? df_mul(a, r[4 * Nx + l]) : zero, ah = df_mul(a, h);
+        rec[3 * l] = make_float4(a.x, a.y, b.x, b.y);
+        rec[3 * l + 1] = make_float4(c.x, c.y, ad.x, ad.y);
+        rec[3 * l + 2] = make_float4(h.x, h.y, ah.x, ah.y);
+    }
+}
+
+// Two dot products per lane with the coefficients G[2 l NB] (high parts) and
+// G[(2 l + 1) NB] (low parts), l < n, as double-floats: of p_x rows 2 k and
+// 2 k + 1 with G^+ and G^- in the lanes (x: P0 the pair's entries), or of two
+// p_y or p_z rows, the even and the odd orders in the lanes.
+template <int NB>
+__device__ __forceinline__ void dot2_rows(bool x, const float4* P0, const float4* P1, const float2* G, int n, DF2& r0,
+                                          DF2& r1) {
+    float2 a0 = f2(0.0f), e0 = f2(0.0f), a1 = f2(0.0f), e1 = f2(0.0f);
+#pragma unroll 2
+    for (int l = 0; l < n; ++l) {
+        const float2 gh = G[2 * l * NB], gl = G[(2 * l + 1) * NB];
+        const float2 ng = fsub2(f2(0.0f), gh);
+        auto term = [&](const float2 th, const float2 tl, float2& acc, float2& err) {
+            const float2 q = __fmul2_rn(th, ng);                  // -p, p = fl(th gh)
+            const float2 e = __ffma2_rn(th, gh, q);               // th gh - p, exact
+            const float2 sum = fsub2(acc, q);                     // acc + p
+            const float2 bb = fsub2(sum, acc);
+            const float2 t2 = fsub2(fsub2(acc, fsub2(sum, bb)), __fadd2_rn(q, bb));   // (acc + p) - sum, exact
+            acc = sum;
+            err = __fadd2_rn(err, __fadd2_rn(t2, e));
+            err = __ffma2_rn(th, gl, __ffma2_rn(tl, gh, err));
+        };
+        const float4 u = P0[l], w = P1[l];
+        term(x ? f2(u.x) : make_float2(u.x, u.y), x ? f2(u.z) : make_float2(u.z, u.w), a0, e0);
+        term(x ? f2(w.y) : make_float2(w.x, w.y), x ? f2(w.w) : make_float2(w.z, w.w), a1, e1);
+    }
+    r0 = df2_add(DF2{a0, f2(0.0f)}, DF2{e0, f2(0.0f)});
+    r1 = df2_add(DF2{a1, f2(0.0f)}, DF2{e1, f2(0.0f)});
+}
+
+// sIn: the inputs of node k (its NodeDF; 1/tau as the .x of field 8), written
+// before a CTA barrier; tab, nt: node_load_tables; rec: node_load_rec; sG:
+// coef_bytes; sLine: [NB][node_line_stride(ncp)].  Ends with the first QX2 + VY
+// + VZ values of every line written, before a CTA barrier.  The loops stay
+// rolled: a CTA runs this code once, and unrolled it spent more time on
+// fetching instructions than on running them.
+template <int NB, int T>
+__device__ __forceinline__ void node_lines(const GroupDev& g, const NodeTables& nt, const float2* sIn, float2* sG,
+                                           float* sLine, const float4* tab, const float4* rec) {
+    constexpr int SLOTS = T / NB;
+    const int k = threadIdx.x % NB, slot = threadIdx.x / NB;
+    const int Nx = g.Nx, Ny = g.Ny, Nz = g.Nz, Qx = g.Qx, QX2 = g.QX2, VY = g.VY, VZ = g.VZ;
+    auto in = [&](int f) { return sIn[f * NB + k]; };       // NodeDF order: ux uy uz T Tm1 erf_z g0 n, then (1/tau, -)
+    const bool active = in(8).x != 0.0f;
+    float2* Gx = sG + k;                                    // [l][h, l][NB]: lanes (+z, -z)
+    float2* Gy = Gx + 2 * (Nx + 1) * NB;                    // [pair][h, l][NB]: lanes (even, odd)
+    float2* Gz = Gy + (g.Qy ? 2 * nt.my * NB : 0);
+    // 1. coefficients
+    if (active && slot == 0) {
+        auto put = [&](int l, const DF2& v) {
+            Gx[2 * l * NB] = v.h;
+            Gx[(2 * l + 1) * NB] = v.l;
+        };
+        if (!g.x_full) {
+            // half_range_G_df's recurrence with its coefficients gathered:
+            //   G_{l+1} = (a_l u + b_l) G_l + (c_l + a_l d_l T) G_{l-1} + a_l h_l(0) W_l,
+            //   W_l = T (g(0) - omega(0) sum_{s<l} h_s(0) G_s),
+            // so that G_l enters G_{l+1} through one product and one sum
+            const float2 ux = in(0), er = in(5);
+            const DF2 Tn = df2_dup(in(3)), us = {make_float2(ux.x, -ux.x), make_float2(ux.y, -ux.y)};
+            const DF2 kap = df2_dup(df_mul(g.m_om0f, in(3)));
+            const float2 hp = df_add(make_float2(0.5f, 0.0f), make_float2(0.5f * er.x, 0.5f * er.y));
+            const float2 hm = df_add(make_float2(0.5f, 0.0f), make_float2(-0.5f * er.x, -0.5f * er.y));
+            const float2 h00 = make_float2(rec[2].x, rec[2].y);
+            DF2 cur = df2_mul(df2_dup(h00), DF2{make_float2(hp.x, hm.x), make_float2(hp.y, hm.y)});
+            DF2 W = df2_dup(df_mul(in(3), in(6))), gm1 = {f2(0.0f), f2(0.0f)};
+            put(0, cur);
+#pragma unroll 1
+            for (int l = 0; l < Nx; ++l) {
+                const float4 ab = rec[3 * l], cd = rec[3 * l + 1], hh = rec[3 * l + 2];
+                const DF2 al = df2_add(df2_mul(DF2{f2(ab.x), f2(ab.y)}, us), DF2{f2(ab.z), f2(ab.w)});
+                const DF2 be = df2_add(df2_mul(DF2{f2(cd.z), f2(cd.w)}, Tn), DF2{f2(cd.x), f2(cd.y)});
+                const DF2 Z = df2_add(df2_mul(be, gm1), df2_mul(DF2{f2(hh.z), f2(hh.w)}, W));
+                W = df2_add(W, df2_mul(df2_mul(kap, DF2{f2(hh.x), f2(hh.y)}), cur));
+                gm1 = cur;
+                cur = df2_add(df2_mul(al, cur), Z);
+                put(l + 1, cur);
+            }
+        } else {
+            // full-range p_x: G_l(+-u_x)
+            const float2 ux = in(0);
+            const DF2 u = {make_float2(ux.x, -ux.x), make_float2(ux.y, -ux.y)}, Tm1 = df2_dup(in(4));
+            DF2 gm1 = {f2(1.0f), f2(0.0f)}, cur = u;
+            put(0, gm1);
+            if (Nx >= 1) put(1, cur);
+#pragma unroll 1
+            for (int l = 1; l < Nx; ++l) {
+                const DF2 nxt = df2_add(df2_mul(u, cur), df2_mul(df2_mul(DF2{f2((float)l), f2(0.0f)}, Tm1), gm1));
+                gm1 = cur;
+                cur = nxt;
+                put(l + 1, cur);
+            }
+        }
+    } else if (active && slot == 1 % SLOTS) {
+        // G_l(u_y) with G_l(u_z); an order past an axis's last is a zero
+        const float2 ua = in(1), ub = in(2);
+        float* fy = reinterpret_cast<float*>(Gy);
+        float* fz = reinterpret_cast<float*>(Gz);
+        const int ly = g.Qy ? 2 * nt.my : 0, lz = g.Qz ? 2 * nt.mz : 0;
+        auto put = [&](int l, const DF2& v) {
+            const int at = 4 * (l >> 1) * NB + (l & 1);
+            if (l < ly) { fy[at] = l <= Ny ? v.h.x : 0.0f; fy[at + 2 * NB] = l <= Ny ? v.l.x : 0.0f; }
+            if (l < lz) { fz[at] = l <= Nz ? v.h.y : 0.0f; fz[at + 2 * NB] = l <= Nz ? v.l.y : 0.0f; }
+        };
+        const DF2 u = {make_float2(ua.x, ub.x), make_float2(ua.y, ub.y)}, Tm1 = df2_dup(in(4));
+        DF2 gm1 = {f2(1.0f), f2(0.0f)}, cur = u;
+        put(0, gm1);
+        put(1, cur);
+#pragma unroll 1
+        for (int l = 1; l + 1 < max(ly, lz); ++l) {
+            const DF2 nxt = df2_add(df2_mul(u, cur), df2_mul(df2_mul(DF2{f2((float)l), f2(0.0f)}, Tm1), gm1));
+            gm1 = cur;
+            cur = nxt;
+            put(l + 1, cur);
+        }
+    }
+    __syncthreads();
+    // 2. dot products: items of two rows of p_x, then of p_y, then of p_z
+    const int ix = Qx >> 1, iy = g.Qy ? (VY + 2) >> 2 : 1, iz = g.Qz ? (VZ + 2) >> 2 : 1;
+    const DF2 n = df2_dup(in(7));
+    float* line = sLine + k * node_line_stride(g.ncp);
+#pragma unroll 1
+    for (int it = slot; it < ix + iy + iz; it += SLOTS) {
+        const bool x = it < ix, z = it >= ix + iy;
+        float* o = line + (x ? 0 : QX2 + (z ? VY : 0));
+        if (!x && (z ? !g.Qz : !g.Qy)) {                 // an absent axis: 1
+            o[0] = active ? 1.0f : 0.0f;
+            continue;
+        }
+        // rows j and j + 1 of p_x, or of the positive half of p_y or p_z
+        const int j = 2 * (x ? it : it - ix - (z ? iy : 0)), half = x ? Qx : (z ? VZ : VY) >> 1;
+        const int m = x ? Nx + 1 : (z ? nt.mz : nt.my);
+        const float4* P = tab + (x ? it * m : nt.nx + (z ? nt.ny : 0) + j * m);
+        float2 a = f2(0.0f), b = f2(0.0f);               // the values of +-p, rows j and j + 1
+        if (active) {
+            DF2 r0, r1;
+            dot2_rows<NB>(x, P, !x && j + 1 < half ? P + m : P, x ? Gx : (z ? Gz : Gy), m, r0, r1);
+            if (x) {
+                r0 = df2_mul(r0, n);
+                r1 = df2_mul(r1, n);
+            } else {
+                // lanes (even, odd) to the rows of z and -z: sum and difference
+                r0 = df2_add(DF2{f2(r0.h.x), f2(r0.l.x)}, DF2{make_float2(r0.h.y, -r0.h.y), make_float2(r0.l.y, -r0.l.y)});
+                r1 = df2_add(DF2{f2(r1.h.x), f2(r1.l.x)}, DF2{make_float2(r1.h.y, -r1.h.y), make_float2(r1.l.y, -r1.l.y)});
+            }
+            a = __fadd2_rn(r0.h, r0.l);
+            b = __fadd2_rn(r1.h, r1.l);
+        }
+        const int p0 = x ? j : half + j, m0 = x ? Qx + j : half - 1 - j, dm = x ? 1 : -1;
+        o[p0] = a.x;
+        o[m0] = a.y;
+        if (j + 1 < half) {
+            o[p0 + 1] = b.x;
+            o[m0 + dm] = b.y;
+        }
+    }
 }
 
 }  // namespace hlb

@@ -162,6 +162,10 @@ void launch_wall(int precision, int adv, const GroupDev& g, const void* fs, cuda
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st);
 void gauss_legendre_rule(int n, std::vector<double>& x, std::vector<double>& w);
 void launch_node(int precision, const GroupDev& g, const void* fs, cudaStream_t st);
+// The node pass and the walls in one launch, for the FP32 groups it takes.
+bool node_fused_available(int precision, const GroupDev& g);
+cudaError_t prepare_node_fused(int adv, const GroupDev& g);
+void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 cudaError_t prepare_node();
 // Marching stage kernel for (QX2, VY, TY); returns false if no instantiation exists.
 bool march_available(int precision, int adv, int QX2, int VY, int TY);

@@ -11,6 +11,7 @@
 #include "hlb_coef.cuh"
 #include "hlb_device.cuh"
 #include "hlb_internal.h"
+#include "hlb_wall.cuh"
 
 namespace hlb {
 namespace {
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(128) coef_df_kernel(const GroupDev g, const fl
                 // n, u, T and the recurrences' start in double-float (no FP64
                 // pipe work but for 1/tau and the rare |z| > 2.5)
                 NodeDF nin;
-                const double n = node_inputs_from_sums_df(sm, g.D, nin);
+                const double n = node_inputs_from_sums_df<true>(sm, g.D, nin);
                 factor_line_df_in<NM>(g, nin, n * inv_Kn, sPx, sPy, sPz, sRec, line);
                 done = true;
             }
@@ -352,6 +353,172 @@ __global__ void __launch_bounds__(128) coef_df_kernel(const GroupDev g, const fl
     }
 }
 
+
+// ---------------------------------------------------------------------------
+// The node pass of FP32 groups in one launch: the first g.nrows g.wchunks CTAs
+// form the walls' emitted densities, every other CTA the moment sums and the
+// factor lines of kNodeNB nodes.  The sums stream the state (HBM-bound), the
+// lines are double-float arithmetic (issue- and latency-bound) and the walls a
+// few CTAs: in one launch they share the SMs instead of running in a row, and a
+// line's work is spread over the CTA (node_lines).  Per stage, against the three
+// kernels: 1024 x 512 nodes of 1024 velocities 0.426 against 0.495 ms (reading
+// the state alone takes 0.317), the 256^2 box of order 15 0.070 against 0.111,
+// 317 x 203 nodes of order 7 0.026 against 0.043 (GB300).  32 nodes and 128
+// threads at 8 CTAs per SM (7 for order 15): 10 per SM spill (0.094 for the
+// box), and a resident grid that loops over the batches runs its CTAs in step,
+// all streaming or all computing (0.93 ms for the large channel).
+// ---------------------------------------------------------------------------
+constexpr int kNodeNB = 32, kNodeT = 128;
+
+struct NodeSmem {                        // byte offsets
+    size_t tab, yz, rec, in, G, line, bytes;
+};
+__host__ __device__ inline NodeSmem node_smem(const GroupDev& g) {
+    const NodeTables nt(g);
+    NodeSmem L;
+    L.tab = 0;
+    L.yz = L.tab + nt.table_bytes();
+    L.rec = L.yz + (size_t)g.VY * g.VZ * 16;
+    L.in = L.rec + node_rec_bytes(g.Nx);
+    L.G = L.in + (size_t)kNodeNB * kNodeFields * 8;
+    L.line = L.G + nt.coef_bytes<kNodeNB>(g);            // the moment sums, then the lines
+    const size_t lines = (size_t)kNodeNB * node_line_stride(g.ncp) * 4, sums = (size_t)kNodeNB * kSumStride * 4;
+    L.bytes = L.line + (lines > sums ? lines : sums);
+    return L;
+}
+
+// The compensated moment sums of nb nodes into sum[node][kSumStride], LPN lanes
+// per node (rows of 4 LPN values); z: a p_z axis.  A lane adds (n, j_x), (j_y, E)
+// and j_z, two sums per packed compensated addition.
+template <int LPN>
+__device__ __forceinline__ void node_sums(const float* __restrict__ fs, const float* __restrict__ P,
+                                          const float4* sYZ, const long long* sOff, float* sum, int nb, int rows, int V,
+                                          bool z) {
+    const int lane = threadIdx.x & 31, sl = lane % LPN;
+    const float4 p = reinterpret_cast<const float4*>(P)[sl];
+    const float2 pa = make_float2(p.x, p.y), pb = make_float2(p.z, p.w);
+    const float2 qa = __fmul2_rn(pa, pa), qb = __fmul2_rn(pb, pb);
+    // every lane of a warp takes part in the shuffles, nodes or not
+    for (int k = threadIdx.x / LPN; (k & ~(32 / LPN - 1)) < nb; k += kNodeT / LPN) {
+        float2 a01 = f2(0.0f), c01 = f2(0.0f), a24 = f2(0.0f), c24 = f2(0.0f);
+        float a3 = 0.0f, c3 = 0.0f;
+        if (k < nb) {
+            const float4* f4 = reinterpret_cast<const float4*>(fs + sOff[k]) + sl;
+            auto add = [&](const float4 x, const float4 yz) {
+                const float2 xa = make_float2(x.x, x.y), xb = make_float2(x.z, x.w);
+                const float2 s2 = __fadd2_rn(xa, xb);
+                const float2 j2 = __ffma2_rn(pb, xb, __fmul2_rn(pa, xa)), e2 = __ffma2_rn(qb, xb, __fmul2_rn(qa, xa));
+                const float sq = s2.x + s2.y;
+                csum_add2(a01, c01, make_float2(sq, j2.x + j2.y));
+                csum_add2(a24, c24, make_float2(yz.x * sq, fmaf(yz.z, sq, e2.x + e2.y)));
+                if (z) csum_add(a3, c3, yz.y * sq);
+            };
+#pragma unroll 4
+            for (int r = 0; r < rows; ++r) add(__ldcs(f4 + r * LPN), sYZ[r]);
+        }
+#pragma unroll
+        for (int o = LPN / 2; o > 0; o >>= 1) {          // compensated tree over the lanes of a node
+            auto up2 = [&](float2& s, float2& c) {
+                const float2 s2 = make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o));
+                const float2 c2 = make_float2(__shfl_xor_sync(0xffffffffu, c.x, o), __shfl_xor_sync(0xffffffffu, c.y, o));
+                csum_add2(s, c, s2);
+                c = __fadd2_rn(c, c2);
+            };
+            up2(a01, c01);
+            up2(a24, c24);
+            if (z) {
+                const float s2 = __shfl_xor_sync(0xffffffffu, a3, o), c2 = __shfl_xor_sync(0xffffffffu, c3, o);
+                csum_add(a3, c3, s2);
+                c3 += c2;
+            }
+        }
+        if (sl == 0 && k < nb) {
+            float* o = sum + k * kSumStride;
+            o[0] = a01.x; o[1] = a01.y; o[2] = a24.x; o[3] = a3; o[4] = a24.y;
+            o[8] = c01.x; o[9] = c01.y; o[10] = c24.x; o[11] = c3; o[12] = c24.y;
+        }
+    }
+}
+
+template <int ADV, int LOWN>
+__global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const GroupDev g, const float* __restrict__ fs) {
+    extern __shared__ __align__(16) unsigned char nsm[];
+    const int nwall = g.nrows * g.wchunks;
+    if ((int)blockIdx.x < nwall) {
+        wall_block<float, ADV>(g, fs, blockIdx.x, reinterpret_cast<double*>(nsm));
+        return;
+    }
+    const NodeSmem L = node_smem(g);
+    float4* tab = reinterpret_cast<float4*>(nsm + L.tab);
+    float4* sYZ = reinterpret_cast<float4*>(nsm + L.yz);
+    float4* rec = reinterpret_cast<float4*>(nsm + L.rec);
+    float2* sIn = reinterpret_cast<float2*>(nsm + L.in);
+    float2* sG = reinterpret_cast<float2*>(nsm + L.G);
+    float* sLine = reinterpret_cast<float*>(nsm + L.line);
+    float* sSum = sLine;
+    const int QX2 = g.QX2, VY = g.VY, VZ = g.VZ, V = g.V;
+    const int tid = threadIdx.x;
+    const NodeTables nt(g);
+    const float* P = static_cast<const float*>(g.p);
+    for (int b = tid; b < VY * VZ; b += kNodeT) {          // momenta of the (jy, kz) pairs
+        const float y = P[QX2 + b % VY], z = P[QX2 + VY + b / VY];
+        sYZ[b] = make_float4(y, z, y * y + z * z, 0.0f);
+    }
+    node_load_rec(g, rec, tid, kNodeT);
+    node_load_tables(g, nt, tab, tid, kNodeT);
+    const int base = ((int)blockIdx.x - nwall) * kNodeNB;
+    const int nb = min(kNodeNB, g.nnodes - base);
+    __shared__ long long sOff[kNodeNB];      // each node's values in the state
+    int ii = 0;
+    if (tid < nb) {
+        ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, base + tid) : 0;
+        sOff[tid] = g.inst[ii].f_off + (long long)(base + tid - g.inst[ii].node_off) * V;
+    }
+    __syncthreads();
+    // 1. moment sums: 2Qx / 4 lanes per node, so that a lane's p_x never change
+    // and step r of its loop is the row r of (jy, kz)
+    if (QX2 == 32) node_sums<8>(fs, P, sYZ, sOff, sSum, nb, VY * VZ, V, VZ > 1);
+    else if (QX2 == 16) node_sums<4>(fs, P, sYZ, sOff, sSum, nb, VY * VZ, V, VZ > 1);
+    else node_sums<2>(fs, P, sYZ, sOff, sSum, nb, VY * VZ, V, VZ > 1);
+    __syncthreads();
+    // 2. n, u, T, 1/tau and what starts the recurrences, one thread per node
+    if (tid < kNodeNB) {
+        NodeDF in;
+        double itau = 0.0;
+        if (tid < nb) {
+            const double inv_Kn = g.inst[ii].inv_Kn;
+            const float* sm = sSum + tid * kSumStride;
+            itau = node_inputs_from_sums_df<LOWN != 0>(sm, g.D, in) * inv_Kn;
+        }
+        const float2 v[kNodeFields] = {in.ux, in.uy, in.uz, in.T, in.Tm1, in.erf_z, in.g0, in.n, make_float2((float)itau, 0.0f)};
+#pragma unroll
+        for (int f = 0; f < kNodeFields; ++f) sIn[f * kNodeNB + tid] = v[f];
+    }
+    __syncthreads();
+    node_lines<kNodeNB, kNodeT>(g, nt, sIn, sG, sLine, tab, rec);
+    if (tid < nb) {                                      // the lines' tails: 1/tau, the field's accelerations
+        float* line = sLine + tid * node_line_stride(g.ncp);
+        const int t0 = QX2 + VY + VZ;
+        line[t0] = sIn[8 * kNodeNB + tid].x;
+        for (int o = t0 + 1; o < g.ncp; ++o) line[o] = 0.0f;
+        if (g.has_field) {                           // a = a_uniform + a_field(node)
+            const InstDev& I = g.inst[ii];
+            const double* af = g.afield + 3 * (size_t)(base + tid);
+            line[g.field_off] = (float)(I.ax + af[0]);
+            line[g.field_off + 1] = (float)(I.ay + af[1]);
+            line[g.field_off + 2] = (float)(I.az + af[2]);
+        }
+    }
+    __syncthreads();
+    // 3. the lines are contiguous in the factor-line buffer
+    const int w4 = g.ncp / 4, s4 = node_line_stride(g.ncp) / 4;
+    float4* dst = reinterpret_cast<float4*>(static_cast<float*>(g.coef) + (size_t)base * g.ncp);
+    const float4* src = reinterpret_cast<const float4*>(sLine);
+    for (int i = tid; i < nb * w4; i += kNodeT) {
+        const int k = i / w4;
+        dst[i] = src[k * s4 + (i - k * w4)];
+    }
+}
 
 }  // namespace
 
@@ -401,6 +568,39 @@ cudaError_t launch_df_special(const double* z, int n, double* erf_out, double* e
     if (n > 0) df_special_kernel<<<(n + 127) / 128, 128>>>(z, n, erf_out, exp_out);
     const cudaError_t e = cudaGetLastError();
     return e != cudaSuccess ? e : cudaDeviceSynchronize();
+}
+
+// Whether the one-launch node pass (sums, factor lines and walls) takes this
+// FP32 group: rows of 8, 16 or 32 p_x values, the double-float lines.
+bool node_fused_available(int precision, const GroupDev& g) {
+    return precision != HLB_FP64_ && g.use_df && max(g.Nx, max(g.Ny, g.Nz)) < 16 && (g.QX2 == 8 || g.QX2 == 16 || g.QX2 == 32);
+}
+
+static bool node_low(const GroupDev& g) { return g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12; }
+
+// Needed only above the 48 KB that a launch has without asking (setting an
+// attribute loads the kernel, which a handle's creation would wait for).
+cudaError_t prepare_node_fused(int adv, const GroupDev& g) {
+    const size_t smem = node_smem(g).bytes;
+    if (smem <= 48 * 1024) return cudaSuccess;
+    const bool low = node_low(g);
+    const void* f = adv == HLB_WENO5_ ? (low ? (const void*)node_df_kernel<HLB_WENO5_, 1> : (const void*)node_df_kernel<HLB_WENO5_, 0>)
+                                      : (low ? (const void*)node_df_kernel<HLB_UPWIND2_, 1> : (const void*)node_df_kernel<HLB_UPWIND2_, 0>);
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
+    const int grid = g.nrows * g.wchunks + (g.nnodes + kNodeNB - 1) / kNodeNB;
+    const size_t smem = node_smem(g).bytes;
+    const float* f = static_cast<const float*>(fs);
+    const bool low = node_low(g);
+    if (adv == HLB_WENO5_) {
+        if (low) node_df_kernel<HLB_WENO5_, 1><<<grid, kNodeT, smem, st>>>(g, f);
+        else node_df_kernel<HLB_WENO5_, 0><<<grid, kNodeT, smem, st>>>(g, f);
+    } else {
+        if (low) node_df_kernel<HLB_UPWIND2_, 1><<<grid, kNodeT, smem, st>>>(g, f);
+        else node_df_kernel<HLB_UPWIND2_, 0><<<grid, kNodeT, smem, st>>>(g, f);
+    }
 }
 
 // Node pass of a stage: the quadrature sums of every node, then the factor
