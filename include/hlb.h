@@ -260,7 +260,7 @@ hlb_status hlb_set_state_dev(hlb_handle* h, const void* f_dev, size_t bytes);
 
 /* Autotuner of the marching kernels' launch shape: for every velocity-set
  * group that runs them, times the three stage launches of one step for x-
- * segment lengths from a quarter to four times the built-in heuristic's (CUDA
+ * segment lengths from half to four times the built-in heuristic's (CUDA
  * events on the handle's stream, one untimed round, three timed) and keeps the
  * fastest; for groups on the persistent kernel, whole persistent steps for
  * segment lengths (cells per work item) of 24 to 264 cells times one or half
@@ -324,10 +324,12 @@ hlb_status hlb_axis(int Q, int half, double* p, double* w, double* K);
  * at most 31; HLB_EINVAL otherwise. */
 hlb_status hlb_equilibrium_x(int Qx, int Nx_eq, double u, double T, double* g);
 
-/* Persistent batched kernel on (1, the default) or off (0).  Velocity-set
- * groups of 1D FP32 instances without a p_z axis (2 Qx x Qy slabs of 8 x 4,
- * 16 x 8, 32 x 16 with the default force-term form, or 32 x 1; equilibrium
- * orders up to 15) step with one persistent launch per RK-3 step: the CTAs
+/* Persistent batched kernel on (1) or off (0) for the groups that can take it;
+ * a handle on which this was never called uses it for such groups of several
+ * instances and at most 1024 nodes, where hlb_autotune has not measured better.
+ * Velocity-set groups of 1D FP32 instances without a p_z axis (2 Qx x Qy slabs
+ * of 8 x 4, 16 x 8, 32 x 16 with the default force-term form, or 32 x 1;
+ * equilibrium orders up to 15) can step with one persistent launch per RK-3 step: the CTAs
  * take work items from a queue in stage-major order, per instance first its
  * node chunks (moment sums, equilibrium factors, the emitted densities of the
  * walls they hold), then its x-segments (the marching update), and each item

@@ -120,6 +120,7 @@ struct Group {
     // node chunks and segments per instance, resident CTAs
     bool persist_ok = false;
     bool node_fused = false;                 // the node pass and the walls in one launch
+    bool persist_auto = false;               // steps with it unless told otherwise (hlb_set_persistent)
     bool persist_use = true;                 // the autotuner's pick: persistent or per-stage launches
     float tuned_ms_persist = 0.0f, tuned_ms_stages = 0.0f;   // its best step times (0: not timed)
     int persist_per_sm = 0, persist_grid = 0, persist_nitems = 0;
@@ -178,7 +179,7 @@ struct hlb_handle {
     std::vector<cudaStream_t> group_stream;
     std::vector<cudaEvent_t> group_done;
     cudaEvent_t step_fork = nullptr;
-    bool persistent = true;                  // eligible groups step with the persistent kernel
+    int persistent = -1;                     // hlb_set_persistent: 1 on, 0 off, -1 not called (by group size)
     // device-to-device state copies between the caller's layout and the
     // groups' buffers (commit of a staged state, the _dev state I/O): chunks
     // of at most kRegroupChunk bytes, group by group, copied by one launch per
@@ -604,12 +605,26 @@ hlb_status build_group(hlb_handle* h, Group& G) {
         }
         G.march_ok = !small_ny && !big && hlb::march_available(G.precision, G.adv, G.QX2, G.VY, G.TY);
         if (G.march_ok) {
-            // segment length: about 4096 CTAs in 2D (strips of two rows), about
-            // 1216 (8 per SM) over the rows of 1D instances; at least 24 cells
-            // so that a CTA's window and table set-up is amortised, at most 512
-            const long long rows = xwork / std::max(1LL, (long long)G.TY);
-            long long sx = rows / (two_d ? 4096 : 1216);
-            sx = std::max(24LL, std::min(512LL, (sx + 5) / 6 * 6));
+            // Segment length from N = cells per resident CTA (strips of TY
+            // rows; CTAs per SM as compiled).  Small problems: one wave of the
+            // shortest segments that fill it, down to one iteration of the line
+            // kernel (4 cells), since a segment is a serial chain of about 1.2 us
+            // per iteration; large ones: a quarter of N within [48, 132] cells (1D)
+            // or [32, 132] (2D), several waves that even out, long enough to
+            // amortise a segment's window and table set-up.  us per step (GB300)
+            // against segments of at least 24 cells sized for 1216 (1D) or 4096
+            // (2D) CTAs: 512 cells of 128 velocities 38.8 against 56.0, 512 of 512
+            // velocities 62.5 against 98.9, 60 x 40 of 128 54 against 93, 317 x 203
+            // 267 against 278, the 256^2 box 1106 against 1142, 131072 cells of 512
+            // velocities 1542 (the same).
+            int dev = 0, nsm = 1;
+            HLB_CUDA(cudaGetDevice(&dev));
+            HLB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+            const long long resident = (long long)nsm * hlb::march_ctas_per_sm(G.precision, G.QX2 * G.VY, G.TY);
+            const long long strips = xwork / std::max(1LL, (long long)G.TY);        // cells of all strips
+            const long long N = (strips + resident - 1) / resident;
+            long long sx = std::min(N, std::max(two_d ? 32LL : 48LL, std::min(132LL, N / 4)));
+            sx = std::max(4LL, two_d ? (sx + 1) / 2 * 2 : (sx + 3) / 4 * 4);
             // the force term's form (below) decides the persistent kernel's
             // eligibility, and that the segment bound: resolve the form first
             G.force_form = 0;
@@ -624,10 +639,17 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                 hlb::persist_available(G.QX2, G.VY, G.force_form, std::max(G.Nx, G.Ny))) {
                 int per = 0;
                 if (hlb::prepare_persist(G.adv, G.QX2, G.VY, G.force_form, &per) == cudaSuccess && per > 0) {
-                    int dev = 0, nsm = 1;
-                    HLB_CUDA(cudaGetDevice(&dev));
-                    HLB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
                     G.persist_ok = true;
+                    // By default the persistent kernel steps groups of several
+                    // instances and at most 1024 nodes (one launch per step);
+                    // larger groups and single instances take the per-stage
+                    // launches.  us per step, persistent against per-stage
+                    // (GB300): 512 cells of 128 velocities 170 against 39, 131072
+                    // of 512 2332 against 1542, 37 seeded channels 640 against 117,
+                    // 4096 9251 against 6050.  Segments of at least 24 cells: an
+                    // item of the persistent kernel reads its tables anew.
+                    G.persist_auto = G.members.size() > 1 && G.nnodes <= 1024;
+                    if (G.persist_auto) sx = std::max(24LL, sx);
                     G.persist_per_sm = per;
                     G.persist_grid = nsm * per;
                     if ((s = upload(G.d_pctl, std::vector<int>(4 + 2 * G.members.size(), 0))) != HLB_OK) return s;
@@ -706,7 +728,8 @@ void wait_moments(hlb_handle* h, cudaStream_t s) {
 // Whether group G steps with the persistent kernel: eligible, enabled, not
 // timed per stage, no per-node force field (that adds a pass per stage).
 bool persist_on(const hlb_handle* h, const Group& G) {
-    return G.persist_ok && G.persist_use && G.march_ok && h->persistent && !h->time_kernels && !G.has_field;
+    return G.persist_ok && G.persist_use && G.march_ok && (h->persistent < 0 ? G.persist_auto : h->persistent != 0) &&
+           !h->time_kernels && !G.has_field;
 }
 
 // One RK-3 step of group G by one launch of the persistent kernel (its
@@ -1655,6 +1678,7 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
 // to FP32 rounding either way).
 hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
     G.persist_use = true;
+    G.persist_auto = true;               // by measurement from here on, not by size
     if (!persist_on(h, G)) return tune_group_stages(h, G, ev, chosen);
     G.persist_use = false;
     hlb_status s = tune_group_stages(h, G, ev, chosen);
@@ -1676,10 +1700,11 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
 }
 
 hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
-    // candidates around the heuristic's segment length, multiples of 6 cells
+    // candidates around the heuristic's segment length, multiples of 6 cells from
+    // 12 on (the heuristic alone goes below, for groups of less than a wave)
     const int base = G.SX;
     std::vector<int> cand;
-    for (int f : {-2, -1, 0, 1, 2}) {
+    for (int f : {-1, 0, 1, 2}) {
         int sx = f < 0 ? base >> (-f) : base << f;
         sx = std::max(12, std::min(1020, (sx + 5) / 6 * 6));
         if (std::find(cand.begin(), cand.end(), sx) == cand.end()) cand.push_back(sx);
@@ -1758,12 +1783,12 @@ hlb_status hlb_df_special_check(const double* z_dev, int n, double* erf_dev, dou
 
 hlb_status hlb_set_persistent(hlb_handle* h, int on) {
     if (!h) return fail(HLB_EINVAL, "handle is NULL");
-    if (h->persistent != (on != 0) && h->graph) {     // the captured steps change: re-capture
+    if (h->persistent != (on != 0 ? 1 : 0) && h->graph) {     // the captured steps change: re-capture
         HLB_CUDA(cudaStreamSynchronize(h->stream));
         cudaGraphExecDestroy(h->graph);
         h->graph = nullptr;
     }
-    h->persistent = on != 0;
+    h->persistent = on != 0 ? 1 : 0;
     return HLB_OK;
 }
 

@@ -528,6 +528,14 @@ __device__ __forceinline__ float2 upwind2_face2(float2 b, float2 c) {
     return __ffma2_rn(f2(1.5f), c, __fmul2_rn(f2(-0.5f), b));
 }
 
+// Quadratic extrapolation of an incident population into the first and second
+// ghost cells beyond the right wall from the wall cell f0 and the next two
+// inward (Sec. IV.C.3), rounded the same way wherever a segment starts.
+__device__ __forceinline__ float wall_ghost1(float f0, float f1, float f2) { return fmaf(3.0f, __fsub_rn(f0, f1), f2); }
+__device__ __forceinline__ float wall_ghost2(float f0, float f1, float f2) {
+    return fmaf(6.0f, f0, fmaf(-8.0f, f1, __fmul_rn(3.0f, f2)));
+}
+
 // Fluxes per unit velocity at NF consecutive faces, two independent rows at
 // once: face f lies between c[f + 2] and c[f + 3] of c[0 .. NF + 4] (cells in
 // ascending order), upwind for a positive (pos) or negative velocity.

@@ -167,6 +167,13 @@ bool node_fused_available(int precision, const GroupDev& g);
 cudaError_t prepare_node_fused(int adv, const GroupDev& g);
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 cudaError_t prepare_node();
+// CTAs per SM that the marching kernels are compiled for (their launch
+// bounds), by slab size S = 2Qx VY and strip height TY.
+inline int march_ctas_per_sm(int precision, int S, int TY) {
+    if (precision == HLB_FP64_) return S <= 32 ? 16 : (S <= 128 ? 4 : 1);
+    if (TY == 2) return S <= 32 ? 16 : (S <= 128 ? 7 : 2);
+    return S <= 32 ? 16 : (S <= 128 ? 8 : (S <= 256 ? 4 : 2));
+}
 // Marching stage kernel for (QX2, VY, TY); returns false if no instantiation exists.
 bool march_available(int precision, int adv, int QX2, int VY, int TY);
 cudaError_t prepare_march(int precision, int adv, int QX2, int VY, int TY, int form);

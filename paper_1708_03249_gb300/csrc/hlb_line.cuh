@@ -127,10 +127,12 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
     const uint32_t row_bytes = S * sizeof(float);
     const int lane = t & 31;
 
+    // test hook: the copies of the second iteration (of the only one) never arrive
+    const int stall = g.inject_stall ? min(1, niter - 1) : -1;
     // warp 0 issues the (at most nine) copies of an iteration, one per lane;
     // thread 0 registers the byte count before any of them
     auto expect = [&](int p) {
-        if (p >= niter || (g.inject_stall && p == 1)) return;   // test hook: iteration 1 never arrives
+        if (p >= niter || p == stall) return;
         const int x0 = xa + 4 * p;
         const int n4 = min(4, xb - x0);
         int nhead = 0;
@@ -141,7 +143,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
         mbar_expect_tx(&bars[p % kLineDepth], bytes);
     };
     auto issue = [&](int p) {
-        if (t >= 32 || p >= niter || (g.inject_stall && p == 1)) return;
+        if (t >= 32 || p >= niter || p == stall) return;
         const int x0 = xa + 4 * p;
         const int n4 = min(4, xb - x0);
         Buf& B = buf[p % kLineDepth];
@@ -190,7 +192,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
             else if (x > nx + 1) val = 0.0f;          // never read by a positive velocity
             else {
                 const float f0 = f[(nx - 1) * V] * sv, f1 = f[(nx - 2) * V] * sv, f2v = f[(nx - 3) * V] * sv;
-                val = x == nx ? 3.0f * f0 - 3.0f * f1 + f2v : 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
+                val = x == nx ? wall_ghost1(f0, f1, f2v) : wall_ghost2(f0, f1, f2v);
             }
             w[j] = val;
         }
@@ -208,8 +210,8 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
     auto enter = [&](int h, const float* hd, float m1, float m2, float m3, float m4) -> float {
         if (h < nx) return hd[vl] * sv;
         if (!xpos) return nwr;                                  // emitted at the right wall
-        if (h == nx) return 3.0f * (m1 - m2) + m3;
-        if (h == nx + 1) return 6.0f * m2 - 8.0f * m3 + 3.0f * m4;
+        if (h == nx) return wall_ghost1(m1, m2, m3);
+        if (h == nx + 1) return wall_ghost2(m2, m3, m4);
         return 0.0f;                                            // never read by v > 0
     };
     float Fm = vx * isv * face1(w);                             // face xa-1/2
@@ -335,7 +337,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
         // a wait ran out at iteration pa: let the copies registered since
         // (less an iteration the test hook withheld) land before the CTA exits
         for (int s2 = pa; s2 < niter && s2 < pa + kLineDepth - 1; ++s2)
-            if (!(g.inject_stall && s2 == 1)) mbar_drain(&bars[s2 % kLineDepth], (s2 / kLineDepth) & 1, g.wait_ns);
+            if (s2 != stall) mbar_drain(&bars[s2 % kLineDepth], (s2 / kLineDepth) & 1, g.wait_ns);
     }
 }
 

@@ -260,7 +260,7 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
                 else if (x > nx + 1) val = 0.0f;          // never read by a positive velocity
                 else {
                     const float f0 = f[(nx - 1) * V] * sv, f1 = f[(nx - 2) * V] * sv, f2v = f[(nx - 3) * V] * sv;
-                    val = x == nx ? 3.0f * f0 - 3.0f * f1 + f2v : 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
+                    val = x == nx ? wall_ghost1(f0, f1, f2v) : wall_ghost2(f0, f1, f2v);
                 }
                 wr[r][j] = val;
             }
@@ -275,8 +275,8 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
                      float2 m4) -> float2 {
         if (h < nx) return __fmul2_rn(make_float2(hd0[vl], hd1[vl]), sv2);
         if (!xpos) return make_float2(nwr_g[0], nwr_g[1]);                     // emitted at the right wall
-        if (h == nx) return __ffma2_rn(f2(3.0f), __fadd2_rn(m1, __fmul2_rn(f2(-1.0f), m2)), m3);
-        if (h == nx + 1) return __ffma2_rn(f2(6.0f), m2, __ffma2_rn(f2(-8.0f), m3, __fmul2_rn(f2(3.0f), m4)));
+        if (h == nx) return make_float2(wall_ghost1(m1.x, m2.x, m3.x), wall_ghost1(m1.y, m2.y, m3.y));
+        if (h == nx + 1) return make_float2(wall_ghost2(m2.x, m3.x, m4.x), wall_ghost2(m2.y, m3.y, m4.y));
         return f2(0.0f);                                                        // never read by v > 0
     };
     float2 Fm;

@@ -324,7 +324,7 @@ __device__ HLB_MARCH_ITEM_ATTR uint32_t march_item(const GroupDev& g, const Pers
             else {
                 const float f0 = __ldcg(f + (nx - 1) * V) * sv, f1 = __ldcg(f + (nx - 2) * V) * sv,
                             f2v = __ldcg(f + (nx - 3) * V) * sv;
-                val = x == nx ? 3.0f * f0 - 3.0f * f1 + f2v : 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
+                val = x == nx ? wall_ghost1(f0, f1, f2v) : wall_ghost2(f0, f1, f2v);
             }
             w[j] = val;
         }
@@ -339,8 +339,8 @@ __device__ HLB_MARCH_ITEM_ATTR uint32_t march_item(const GroupDev& g, const Pers
     auto enter = [&](int h, const float* hd, float m1, float m2, float m3, float m4) -> float {
         if (h < nx) return hd[vl] * sv;
         if (!xpos) return nwr;                                  // emitted at the right wall
-        if (h == nx) return 3.0f * (m1 - m2) + m3;
-        if (h == nx + 1) return 6.0f * m2 - 8.0f * m3 + 3.0f * m4;
+        if (h == nx) return wall_ghost1(m1, m2, m3);
+        if (h == nx + 1) return wall_ghost2(m2, m3, m4);
         return 0.0f;                                            // never read by v > 0
     };
     float Fm = vx * isv * face1(w);
