@@ -675,7 +675,7 @@ hlb_status build_group(hlb_handle* h, Group& G) {
     // separate sums, factor-line and wall kernels and with them their twelve
     // launches per step, which callers can count (hlb_launch_count)
     G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && (G.TY == 1 || G.nnodes >= 1024);
-    if (G.march_ok) HLB_CUDA(G.node_fused ? hlb::prepare_node_fused(G.adv, G.dev) : hlb::prepare_node());
+    if (G.march_ok && G.precision == HLB_FP32) HLB_CUDA(G.node_fused ? hlb::prepare_node_fused(G.adv, G.dev) : hlb::prepare_node());
 
     // launch shape of the stage kernel.  With Kx in global memory each
     // velocity's force term is a 2Qx-term dot product (FP64), so the velocities
@@ -715,6 +715,11 @@ bool group_has_z_force(const hlb_handle* h, const Group& G) {
     for (int i : G.members)
         if (h->cfg[i].az != 0.0) return true;
     return false;
+}
+
+// Whether any instance of the group has a BGK term (Kn finite).
+bool group_relaxes(const Group& G) {
+    return std::any_of(G.inst.begin(), G.inst.end(), [](const hlb::InstDev& I) { return I.inv_Kn != 0.0; });
 }
 
 // Make stream s wait, on the device, for the pending asynchronous moments
@@ -775,11 +780,14 @@ void enqueue_group_step(hlb_handle* h, Group& G, cudaStream_t st_) {
         }
         NvtxRange range(kStageNames[st]);
         const bool march = G.march_ok && !group_has_z_force(h, G);
-        if (G.quad_x) hlb::launch_quad_coef(G.dev, ins[st], st_);
-        if (march && G.node_fused) {
+        const bool relax = group_relaxes(G);
+        if (G.quad_x && relax) hlb::launch_quad_coef(G.dev, ins[st], st_);
+        if (G.precision == HLB_FP64 && (march || relax)) {
+            hlb::launch_node_f64(G.adv, G.dev, ins[st], st_);
+        } else if (march && G.node_fused) {
             hlb::launch_node_fused(G.adv, G.dev, ins[st], st_);
         } else {
-            if (march) hlb::launch_node(G.precision, G.dev, ins[st], st_);
+            if (march) hlb::launch_node(G.dev, ins[st], st_);
             hlb::launch_wall(G.precision, G.adv, G.dev, ins[st], st_);
         }
         if (h->time_kernels) cudaEventRecord(e1, st_);
@@ -821,8 +829,8 @@ long long kernels_per_step(hlb_handle* h) {
     long long n = 0;
     for (auto& G : h->groups)
         n += persist_on(h, *G) ? 1
-                               : 3 * ((G->march_ok && !group_has_z_force(h, *G)) ? (G->node_fused ? 2 : 4) : 2) +
-                                     (G->quad_x ? 3 : 0);
+                               : 3 * ((G->march_ok && !group_has_z_force(h, *G) && G->precision != HLB_FP64 && !G->node_fused) ? 4 : 2) +
+                                     (G->quad_x && group_relaxes(*G) ? 3 : 0);
     return n;
 }
 

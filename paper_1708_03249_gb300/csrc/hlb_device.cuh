@@ -68,6 +68,62 @@ __device__ __forceinline__ R weno5_face(R a, R b, R c, R d, R e) {
     return (w1 * F1 + w2 * F2 + w3 * F3) / (w1 + w2 + w3);
 }
 
+// 1/x for x in [1e-300, 1e300]: the special-function unit's approximation (about
+// 20 bits) refined by one third-order Householder step (r (1 + e + e^2), e = 1 -
+// x r): three FP64 operations, where a division takes about ten and a branch.
+__device__ __forceinline__ double rcp_fp64(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// NF consecutive WENO-5 faces in FP64: face f lies between u[f + 2] and u[f + 3]
+// of the upwind-ordered values; the weights of weno5_face in the form of
+// weno5_scaled (below), with the same scaling of the stencil by the power of
+// two that brings its largest magnitude into [1/2, 1) (here the largest of the
+// NF + 4 values).  The FP64 pipe runs at 1/64 of FP32 and bounds the kernels that
+// call this: about 45 FP64 operations per face, fewer with NF > 1, where the
+// three candidates, the indicators and four divisions took about 95.  The floor
+// of 1e-300 under the indicators is below what their squares resolve (a zero
+// indicator takes the limit of Tab. "weno"), and 2^-200 B_2 keeps the squared
+// ratios in range.
+template <int NF>
+__device__ __forceinline__ void weno5_faces64(const double (&u)[NF + 4], double (&F)[NF]) {
+    int m = 0;
+#pragma unroll
+    for (int j = 0; j < NF + 4; ++j) m = max(m, __double2hiint(u[j]) & 0x7fffffff);
+    const int ex = min(max(m >> 20, 1), 2044);                          // biased exponent of the largest
+    const double sc = __hiloint2double((2045 - ex) << 20, 0), inv = __hiloint2double((ex + 1) << 20, 0);
+    constexpr double k = 39.0 / 64.0, fl = 1e-300, eps = 6.223015277861142e-61;       // 2^-200
+    double d2 = (u[2] - u[1]) * sc, d3 = (u[3] - u[2]) * sc;
+    double s1 = d2 - (u[1] - u[0]) * sc, m2 = fma(k * d2, d2, fl);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const double d4 = (u[f + 4] - u[f + 3]) * sc;
+        const double s2 = d3 - d2, s3 = d4 - d3, m3 = fma(k * d3, d3, fl);
+        const double u1 = fma(0.375, d2, s1), u2 = fma(0.375, d2, s2), u3 = fma(-0.375, d3, s3);
+        const double B1 = fma(u1, u1, m2), B2 = fma(u2, u2, m2), B3 = fma(u3, u3, m3);
+        const double r1 = (0.40824829046386301637 * B2) * rcp_fp64(fma(eps, B2, B1));
+        const double r3 = (0.5 * B2) * rcp_fp64(fma(eps, B2, B3));
+        const double w1 = r1 * r1, v3 = r3 * r3;                         // v3 = w_3 / 2
+        const double den = fma(3.0, w1, fma(6.0, v3, 3.0));
+        const double num = fma(v3, fma(3.0, d3, -s3), fma(w1, fma(1.5, d2, s1), fma(1.5, d2, s2)));
+        F[f] = fma(num * inv, rcp_fp64(den), u[f + 2]);
+        s1 = s2;
+        d2 = d3;
+        d3 = d4;
+        m2 = m3;
+    }
+}
+template <>
+__device__ __forceinline__ double weno5_face<double>(double a, double b, double c, double d, double e) {
+    const double u[5] = {a, b, c, d, e};
+    double F[1];
+    weno5_faces64<1>(u, F);
+    return F[0];
+}
+
 // Same weights as weno5_face, for the marching kernel: the smoothness
 // indicators are formed from the stencil values times a fixed per-velocity
 // scale ``sv`` (the inverse quadrature weight of the population, so that the

@@ -161,16 +161,17 @@ void launch_wall(int precision, int adv, const GroupDev& g, const void* fs, cuda
 // quadrature of the projection integrals (hlb_kernels.cu)
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st);
 void gauss_legendre_rule(int n, std::vector<double>& x, std::vector<double>& w);
-void launch_node(int precision, const GroupDev& g, const void* fs, cudaStream_t st);
+void launch_node(const GroupDev& g, const void* fs, cudaStream_t st);
 // The node pass and the walls in one launch, for the FP32 groups it takes.
 bool node_fused_available(int precision, const GroupDev& g);
 cudaError_t prepare_node_fused(int adv, const GroupDev& g);
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
+void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 cudaError_t prepare_node();
 // CTAs per SM that the marching kernels are compiled for (their launch
 // bounds), by slab size S = 2Qx VY and strip height TY.
 inline int march_ctas_per_sm(int precision, int S, int TY) {
-    if (precision == HLB_FP64_) return S <= 32 ? 16 : (S <= 128 ? 4 : 1);
+    if (precision == HLB_FP64_) return S <= 32 ? 16 : (S <= 128 ? (TY == 2 ? 3 : 4) : 1);
     if (TY == 2) return S <= 32 ? 16 : (S <= 128 ? 7 : 2);
     return S <= 32 ? 16 : (S <= 128 ? 8 : (S <= 256 ? 4 : 2));
 }

@@ -91,7 +91,14 @@ __device__ __forceinline__ R x_value(const R* __restrict__ frow, int pos, int nx
 // window; w[] holds cells x-3..x+2 for v > 0 and x-2..x+3 for v < 0.
 template <typename R, int ADV>
 __device__ __forceinline__ void face_pair(const R* w, bool pos, R& Fp, R& Fm) {
-    if (ADV == HLB_WENO5_) {
+    if constexpr (ADV == HLB_WENO5_ && sizeof(R) == 8) {
+        double u[6], F[2];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) u[j] = pos ? w[j] : w[5 - j];
+        weno5_faces64<2>(u, F);
+        Fp = pos ? F[1] : F[0];
+        Fm = pos ? F[0] : F[1];
+    } else if (ADV == HLB_WENO5_) {
         if (pos) {
             Fp = weno5_face(w[1], w[2], w[3], w[4], w[5]);
             Fm = weno5_face(w[0], w[1], w[2], w[3], w[4]);
@@ -182,6 +189,12 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
         // Collisionless instances (Kn = +inf) have no BGK term at all: no
         // moments and no equilibrium are formed for them.
         const bool collide = I.inv_Kn != 0.0;
+        // FP64 groups: the node pass has formed the factors and 1/tau
+        // (node_f64_kernel); FP32 groups form them here, per node
+        const R* line = static_cast<const R*>(g.coef) + (size_t)node * g.ncp;
+        const bool form = collide && sizeof(R) == 4;
+        if (collide && sizeof(R) == 8)
+            for (int t = tid; t < QX2 + VY + VZ; t += bs) sG[t] = line[t];
         // 1. node values and moment partial sums, accumulated in FP64 for
         // either state precision (T = (E - n|u|^2)/(D n) cancels digits, and
         // the FP32 state's sums are not compensated here)
@@ -189,7 +202,7 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
         for (int v = tid; v < V; v += bs) {
             const R val_r = frow[(size_t)x * V + v];
             sF[v] = val_r;
-            if (!collide) continue;
+            if (!form) continue;
             const int ix = v % QX2, jy = (v / QX2) % VY, kz = v / (QX2 * VY);
             const double px = sPx[ix], py = sPy[jy], pz = sPz[kz], val = val_r;
             a0 += val;
@@ -198,7 +211,7 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
             a3 += pz * val;
             a4 += (px * px + py * py + pz * pz) * val;
         }
-        if (collide) {
+        if (form) {
         a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3); a4 = warp_sum(a4);
         if (lane == 0) {
             sRed[warp * 5 + 0] = a0; sRed[warp * 5 + 1] = a1; sRed[warp * 5 + 2] = a2;
@@ -216,12 +229,7 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
                 sScal[0] = n;
                 sScal[1] = n * I.inv_Kn;     // 1/tau
             }
-            if (g.quad_x && tid < 2) {          // G^{+-} by quadrature (quad_coef_kernel)
-                const double* q = g.gquad + ((size_t)node * 2 + tid) * (g.Nx + 1);
-                for (int l = 0; l <= g.Nx; ++l) sCoef[tid * (g.Nx + 1) + l] = q[l];
-            } else {
-                node_coefficients(g, tid, ux, uy, uz, T, sRec, sCoef);
-            }
+            node_coefficients(g, tid, ux, uy, uz, T, sRec, sCoef);
         }
         __syncthreads();
         // 2. equilibrium factors g_x (times n), g_y, g_z
@@ -257,7 +265,7 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
                 sG[t] = (R)acc;
             }
         }
-        }  // collide
+        }  // form
         __syncthreads();
         if (g.kx_global) {
             // K^h = blockdiag(same-half blocks) + the rank-one jump term
@@ -276,7 +284,7 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
             __syncthreads();
         }
 
-        const R inv_tau = collide ? (R)sScal[1] : R(0);
+        const R inv_tau = !collide ? R(0) : (sizeof(R) == 8 ? line[QX2 + VY + VZ] : (R)sScal[1]);
         const R dt = (R)I.dt;
         const R inv_dx = (R)(1.0 / g.dx[I.dx_off + x]);
         const R inv_dy = (R)I.inv_dy;
@@ -409,29 +417,36 @@ wall_kernel(const GroupDev g, const R* __restrict__ fs) {
 // recurrence's stable order: G^{+-}_l = int_0^inf g(+-p) h_l(p) dp (l <= Nx),
 // g the Gaussian of the node's u_x and T (Sec. IV.B, the projection of Eq.
 // "eq:hh_gk"), by composite Gauss-Legendre quadrature over [0, |u_x| +
-// 15 sqrt(T)] in panels of width sqrt(T) (kQuadNodes points each; 300-440
-// points; 1e-14 of max |G| against a 30-point rule on panels of 0.02
+// 13 sqrt(T)] in panels of width sqrt(T) (kQuadNodes points each; 280-320
+// points; beyond, g h_l is below 1e-17 of its maximum for l <= 31; 1e-14 of max |G| against a 30-point rule on panels of 0.02
 // sqrt(T)), h_l(p) by the three-term recurrence of the orthonormal basis
 // (forward evaluation at a point is stable).  The integration-by-parts
 // recurrence of node_coefficients carries its rounding (and that of its erf
 // and exp start) along a solution that grows about threefold per order:
-// 5e-7 of max g at N = 20.  One CTA per node, both signs from the same h_l(p);
-// moments in FP64 as the stage kernel forms them.
+// 5e-7 of max g at N = 20.  One CTA per node and sign (72 nodes fill 144 of 152
+// SMs; both signs in one CTA save the second evaluation of h_l(p), 2 of 5
+// operations per point and order, but leave half the SMs idle), 128 threads of
+// three points each, their sums over the CTA through shared memory (the FP64
+// adds of a full-warp butterfly for every order cost as much as the points).
+// 72 nodes at order 20: 28 us per stage, 44 with one CTA of 256 threads per node
+// and butterflies (GB300).
 // ---------------------------------------------------------------------------
+constexpr int kQuadThreads = 128;
 template <int NMAX>
-__global__ void __launch_bounds__(256) quad_coef_kernel(const GroupDev g, const double* __restrict__ fs) {
-    __shared__ double red[8][2 * NMAX];
-    __shared__ double sMom[8];
-    const int node = blockIdx.x;
+__global__ void __launch_bounds__(kQuadThreads) quad_coef_kernel(const GroupDev g, const double* __restrict__ fs) {
+    __shared__ double part[NMAX][kQuadThreads + 1];
+    __shared__ double red[kQuadThreads / 32][5];
+    __shared__ double sMom[2];
+    const int node = blockIdx.x >> 1, sg = blockIdx.x & 1;
     const int ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0;
     const InstDev& I = g.inst[ii];
     if (I.inv_Kn == 0.0) return;                // collisionless: no equilibrium is formed
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = kQuadThreads / 32;
     const int V = g.V, QX2 = g.QX2, VY = g.VY, Nx = g.Nx;
     const double* f = fs + I.f_off + (size_t)(node - I.node_off) * V;
     // moments of the node
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
-    for (int v = tid; v < V; v += blockDim.x) {
+    for (int v = tid; v < V; v += kQuadThreads) {
         const double val = f[v];
         const double px = g.pd[v % QX2], py = g.pd[QX2 + (v / QX2) % VY], pz = g.pd[QX2 + VY + v / (QX2 * VY)];
         a0 += val;
@@ -454,51 +469,41 @@ __global__ void __launch_bounds__(256) quad_coef_kernel(const GroupDev g, const 
     __syncthreads();
     const double ux = sMom[0], T = sMom[1];
     const double sT = sqrt(T), width = sT;
-    const int panels = (int)ceil((fabs(ux) + 15.0 * sT) / width);
+    const int panels = (int)ceil((fabs(ux) + 13.0 * sT) / width);
     const int npts = panels * kQuadNodes;
-    const double norm = 1.0 / (kSqrt2Pi * sT), i2T = 0.5 / T;
+    const double norm = 1.0 / (kSqrt2Pi * sT), i2T = 0.5 / T, u = sg ? -ux : ux;
     const double* ra = g.rec;
     const double* rb = g.rec + Nx;
     const double* rc = g.rec + 2 * Nx;
     const double h00 = g.rec[3 * Nx];
-    double Gp[NMAX], Gm[NMAX];
+    double G[NMAX];
 #pragma unroll
-    for (int l = 0; l < NMAX; ++l) Gp[l] = Gm[l] = 0.0;
-    for (int k = tid; k < npts; k += blockDim.x) {
+    for (int l = 0; l < NMAX; ++l) G[l] = 0.0;
+    for (int k = tid; k < npts; k += kQuadThreads) {
         const int pnl = k / kQuadNodes, i = k - pnl * kQuadNodes;
         const double p = (pnl + 0.5 * (1.0 + g.glrule[i])) * width;
-        const double w0 = 0.5 * width * g.glrule[kQuadNodes + i] * norm;
-        const double dp = p - ux, dm = p + ux;
-        const double wp = w0 * exp(-dp * dp * i2T), wm = w0 * exp(-dm * dm * i2T);
-        double hm = 0.0, h = h00;
-        Gp[0] += wp * h;
-        Gm[0] += wm * h;
+        const double d = p - u;
+        const double w = 0.5 * width * g.glrule[kQuadNodes + i] * norm * exp(-d * d * i2T);
+        double hm = 0.0, h = w * h00;            // the weight times h_l(p): the recurrence is linear
+        G[0] += h;
 #pragma unroll
         for (int l = 0; l < NMAX - 1; ++l) {
             if (l < Nx) {
-                const double hn = (ra[l] * p + rb[l]) * h + rc[l] * hm;
+                const double hn = fma(fma(ra[l], p, rb[l]), h, rc[l] * hm);
                 hm = h;
                 h = hn;
-                Gp[l + 1] += wp * h;
-                Gm[l + 1] += wm * h;
+                G[l + 1] += h;
             }
         }
     }
-    __syncthreads();                            // red[] is reused below
 #pragma unroll
-    for (int l = 0; l < NMAX; ++l) {
-        if (l <= Nx) {
-            const double sp = warp_sum(Gp[l]), sm = warp_sum(Gm[l]);
-            if (lane == 0) { red[warp][l] = sp; red[warp][NMAX + l] = sm; }
-        }
-    }
+    for (int l = 0; l < NMAX; ++l)
+        if (l <= Nx) part[l][tid] = G[l];
     __syncthreads();
-    double* out = g.gquad + (size_t)node * 2 * (Nx + 1);
-    for (int t = tid; t < 2 * (Nx + 1); t += blockDim.x) {
-        const int sg = t / (Nx + 1), l = t - sg * (Nx + 1);
-        double acc = 0.0;
-        for (int w = 0; w < nw; ++w) acc += red[w][sg * NMAX + l];
-        out[t] = acc;
+    double* out = g.gquad + ((size_t)node * 2 + sg) * (Nx + 1);
+    for (int l = warp; l <= Nx; l += nw) {
+        const double acc = warp_sum((part[l][lane] + part[l][lane + 32]) + (part[l][lane + 64] + part[l][lane + 96]));
+        if (lane == 0) out[l] = acc;
     }
 }
 
@@ -790,8 +795,8 @@ void launch_stage(int precision, int adv, const GroupDev& g, const void* fs, con
 }
 
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st) {
-    if (g.Nx < 24) quad_coef_kernel<24><<<g.nnodes, 256, 0, st>>>(g, (const double*)fs);
-    else quad_coef_kernel<32><<<g.nnodes, 256, 0, st>>>(g, (const double*)fs);
+    if (g.Nx < 24) quad_coef_kernel<24><<<2 * g.nnodes, kQuadThreads, 0, st>>>(g, (const double*)fs);
+    else quad_coef_kernel<32><<<2 * g.nnodes, kQuadThreads, 0, st>>>(g, (const double*)fs);
 }
 
 void launch_wall(int precision, int adv, const GroupDev& g, const void* fs, cudaStream_t st) {

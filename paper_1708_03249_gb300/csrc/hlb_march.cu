@@ -69,7 +69,7 @@ constexpr size_t march_smem_bytes() {
 // The marching kernel.  Offsets inside an instance are 32-bit (the host
 // only takes this path when an instance holds fewer than 2^31 values).
 template <typename R, int ADV, int QX2, int VY, int TY>
-__global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? 4 : 1)))
+__global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? (TY > 1 ? 3 : 4) : 1)))
 march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restrict__ fs,
              const R* __restrict__ fn, R* __restrict__ fo, int stage) {
     constexpr int S = QX2 * VY;
@@ -237,10 +237,19 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restri
 #pragma unroll
             for (int k = 0; k < 3; ++k) col[TY + 3 + k] = B.halo[3 + k][t];
             R Gf[TY + 1];
+            if constexpr (ADV == HLB_WENO5_ && sizeof(R) == 8) {
+                double u[TY + 5], F[TY + 1];
 #pragma unroll
-            for (int i = 0; i <= TY; ++i)      // face between col[i+2] and col[i+3]
-                Gf[i] = vy * face_value<R, ADV>(ypos, sv, col[i], col[i + 1], col[i + 2], col[i + 3],
-                                                col[i + 4], col[i + 5]);
+                for (int i = 0; i < TY + 5; ++i) u[i] = ypos ? col[i] : col[TY + 5 - i];
+                weno5_faces64<TY + 1>(u, F);
+#pragma unroll
+                for (int i = 0; i <= TY; ++i) Gf[i] = vy * (ypos ? F[i] : F[TY - i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i <= TY; ++i)      // face between col[i+2] and col[i+3]
+                    Gf[i] = vy * face_value<R, ADV>(ypos, sv, col[i], col[i + 1], col[i + 2], col[i + 3],
+                                                    col[i + 4], col[i + 5]);
+            }
 #pragma unroll
             for (int r = 0; r < TY; ++r) divy[r] = (Gf[r + 1] - Gf[r]) * inv_dy;
         }
@@ -298,7 +307,8 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restri
 
 #define HLB_MARCH_LIST(X)                                                              \
     X(float, 8, 1, 1) X(float, 16, 1, 1) X(double, 8, 4, 1) X(double, 8, 1, 1)             \
-    X(double, 16, 8, 1) X(double, 32, 16, 1) X(double, 16, 1, 1)
+    X(double, 16, 8, 1) X(double, 32, 16, 1) X(double, 16, 1, 1) X(double, 8, 4, 2)             \
+    X(double, 16, 8, 2)
 
 namespace {
 template <typename R, int ADV, int QX2, int VY, int TY>

@@ -189,12 +189,7 @@ __global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __r
                         node_coefficients_df(g, role, sIn[lane], sRecF, sGF + lane * ncoef);
                 } else {
                     for (int role = 0; role < 4; ++role) {
-                        if (g.quad_x && role < 2) {      // G^{+-} by quadrature (quad_coef_kernel)
-                            const double* q = g.gquad + ((size_t)node * 2 + role) * (Nx + 1);
-                            for (int l = 0; l <= Nx; ++l) sG[lane * ncoef + role * (Nx + 1) + l] = q[l];
-                        } else {
-                            node_coefficients(g, role, ux, uy, uz, T, sRec, sG + lane * ncoef);
-                        }
+                        node_coefficients(g, role, ux, uy, uz, T, sRec, sG + lane * ncoef);
                     }
                 }
             }
@@ -520,12 +515,227 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
     }
 }
 
+// ---------------------------------------------------------------------------
+// The node pass of FP64 groups in one launch: the first g.nrows g.wchunks CTAs
+// form the walls' emitted densities, every other CTA the moments and factor
+// lines of NB nodes.  FP64 instructions run at 1/64 of FP32, per warp whatever its
+// mask, and in long dependent chains (erf, exp, divisions, recurrences), so a
+// small group waits on one thread's chain and a large one on the pipe: the
+// roles of the recurrences run in different threads (p_x in warp 0, p_y and
+// p_z in warp 1), the dot products over the whole CTA; one node per CTA where
+// that leaves at most two CTAs per SM, eight otherwise.  Per
+// stage (GB300): 5795 nodes of 128 velocities 30 us; 72 nodes of 400 velocities,
+// order 20, 14.7 us with one node per CTA, 47 with eight; the 64 nodes of the
+// FP64 channel (moments, lines and walls in three kernels before) take 9 of the
+// 17 us that a stage is now.
+// ---------------------------------------------------------------------------
+constexpr int kNode64T = 128;
+
+__host__ __device__ inline size_t node64_smem(const GroupDev& g, int NB) {
+    const int ncoef = 2 * (g.Nx + 1) + (g.Ny + 1) + (g.Nz + 1);
+    return sizeof(double) * ((size_t)NB * (6 + ncoef) + 5 * g.Nx + 1 + 3 * g.VY * g.VZ + 20);
+}
+
+// The half-range coefficients of node_coefficients (role r = 0, 1) with exp and
+// erf by their Taylor polynomials where the flow is slow enough.
+__device__ __forceinline__ void half_range_coefficients(const GroupDev& g, int r, double ux, double T, const double* rec,
+                                                        double* G) {
+    const int Nx = g.Nx;
+    double irt;
+    if (T > 1e-30 && T < 1e30) {
+        irt = (double)rsqrtf((float)T);                          // one third-order Householder step
+        const double e = fma(-T * irt, irt, 1.0);
+        irt = fma(irt * e, fma(0.375, e, 0.5), irt);
+    } else {
+        irt = 1.0 / sqrt(T);
+    }
+    const double z = ux * irt * 0.70710678118654752440;
+    double E, F;
+    if (fabs(z) <= 0.7) {
+        exp_erf_small(-z * z, E, F);
+        F *= z * 1.1283791670955125739;                          // 2 / sqrt(pi)
+    } else {
+        E = exp(-z * z);
+        F = erf(z);
+    }
+    const double us = r ? -ux : ux, g0 = E * (irt * (1.0 / kSqrt2Pi));
+    const double* rb = rec + Nx;
+    const double* rc = rec + 2 * Nx;
+    const double* h0 = rec + 3 * Nx;
+    const double* d = rec + 4 * Nx + 1;
+    G[0] = h0[0] * (0.5 + (r ? -0.5 : 0.5) * F);
+    double S = 0.0, gm1 = 0.0;
+    for (int l = 0; l < Nx; ++l) {
+        const double ig = (l ? gm1 * d[l - 1] : 0.0) - g.om0 * h0[l] * S;
+        const double pg = us * G[l] + T * (g0 * h0[l] + ig);
+        G[l + 1] = rec[l] * pg + rb[l] * G[l] + rc[l] * gm1;
+        S += h0[l] * G[l];
+        gm1 = G[l];
+    }
+}
+
+template <int ADV, int NB>
+__global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, const double* __restrict__ fs) {
+    extern __shared__ __align__(16) double dsm[];
+    constexpr int LPN = kNode64T / NB;                        // lanes per node
+    const int nwall = g.nrows * g.wchunks;
+    if ((int)blockIdx.x < nwall) {
+        wall_block<double, ADV>(g, fs, blockIdx.x, dsm);
+        return;
+    }
+    const int Nx = g.Nx, Ny = g.Ny, Nz = g.Nz, Qx = g.Qx, QX2 = g.QX2, VY = g.VY, VZ = g.VZ, rows = VY * VZ;
+    const int ncoef = 2 * (Nx + 1) + (Ny + 1) + (Nz + 1), nf = QX2 + VY + VZ;
+    double* sM = dsm;                        // [NB][6]: n, u_x, u_y, u_z, T, 1/tau
+    double* sG = sM + 6 * NB;                // [NB][ncoef]
+    double* sRec = sG + NB * ncoef;
+    double* sRow = sRec + 5 * Nx + 1;        // [rows][3]: p_y, p_z, p_y^2 + p_z^2
+    double* sPart = sRow + 3 * rows;         // [4][5]: partial moments of the warps (NB = 1)
+    const int tid = threadIdx.x;
+    const int base = ((int)blockIdx.x - nwall) * NB;
+    const int nb = min(NB, g.nnodes - base);
+    const double* P = g.pd;
+    for (int i = tid; i < 5 * Nx + 1; i += kNode64T) sRec[i] = g.rec[i];
+    for (int r = tid; r < rows; r += kNode64T) {
+        const double py = P[QX2 + r % VY], pz = P[QX2 + VY + r / VY];
+        sRow[3 * r] = py;
+        sRow[3 * r + 1] = pz;
+        sRow[3 * r + 2] = py * py + pz * pz;
+    }
+    __syncthreads();
+    // 1. moments: each lane its own p_x, weighted once per column
+    {
+        const int k = tid / LPN, sl = tid % LPN;
+        const int node = base + min(k, nb - 1);
+        const InstDev& I = g.inst[g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0];
+        const double* f = fs + I.f_off + (size_t)(node - I.node_off) * g.V;
+        double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};             // n, j_x, j_y, j_z, E
+        if (I.inv_Kn != 0.0) {
+            for (int ix = sl; ix < QX2; ix += LPN) {
+                double s0 = 0.0, sy = 0.0, sz = 0.0, s2 = 0.0;
+                if (VZ == 1) {
+#pragma unroll 8
+                    for (int r = 0; r < rows; ++r) {
+                        const double val = f[r * QX2 + ix];
+                        s0 += val;
+                        sy = fma(sRow[3 * r], val, sy);
+                        s2 = fma(sRow[3 * r + 2], val, s2);
+                    }
+                } else {
+#pragma unroll 8
+                    for (int r = 0; r < rows; ++r) {
+                        const double val = f[r * QX2 + ix];
+                        s0 += val;
+                        sy = fma(sRow[3 * r], val, sy);
+                        sz = fma(sRow[3 * r + 1], val, sz);
+                        s2 = fma(sRow[3 * r + 2], val, s2);
+                    }
+                }
+                const double p = P[ix], ps = p * s0;
+                m[0] += s0;
+                m[1] += ps;
+                m[2] += sy;
+                m[3] += sz;
+                m[4] += fma(p, ps, s2);
+            }
+            constexpr int W = LPN < 32 ? LPN : 32;
+            const unsigned mask = W == 32 ? 0xffffffffu : ((1u << (W & 31)) - 1u) << (tid & 31 & ~(W - 1));   // a node's lanes
+#pragma unroll
+            for (int o = W / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < 5; ++c) m[c] += __shfl_xor_sync(mask, m[c], o);
+        }
+        if (LPN > 32) {
+            if ((tid & 31) == 0)
+                for (int c = 0; c < 5; ++c) sPart[5 * (tid >> 5) + c] = m[c];
+            __syncthreads();
+            if (tid == 0)
+                for (int w = 1; w < kNode64T / 32; ++w)
+                    for (int c = 0; c < 5; ++c) m[c] += sPart[5 * w + c];
+        }
+        if (sl == 0) {
+            const double in = 1.0 / m[0], ux = m[1] * in, uy = m[2] * in, uz = m[3] * in;
+            double* o = sM + 6 * k;
+            o[0] = m[0]; o[1] = ux; o[2] = uy; o[3] = uz;
+            o[4] = (m[4] - m[0] * (ux * ux + uy * uy + uz * uz)) * in * (g.D == 3 ? 1.0 / 3.0 : (g.D == 2 ? 0.5 : 1.0));
+            o[5] = m[0] * I.inv_Kn;
+        }
+    }
+    __syncthreads();
+    // 2. coefficients: p_x roles in warp 0, p_y and p_z roles in warp 1
+    if (tid < 64 && (tid & 31) < 2 * NB) {
+        const int k = (tid & 31) % NB, r = 2 * (tid >> 5) + ((tid & 31) / NB);
+        const double* m = sM + 6 * k;
+        double* G = sG + k * ncoef;
+        if (k < nb && m[5] != 0.0) {
+            if (r < 2 && g.quad_x) {         // G^{+-} by quadrature (quad_coef_kernel)
+                const double* q = g.gquad + ((size_t)(base + k) * 2 + r) * (Nx + 1);
+                for (int l = 0; l <= Nx; ++l) G[r * (Nx + 1) + l] = q[l];
+            } else if (r < 2 && !g.x_full) {
+                half_range_coefficients(g, r, m[1], m[4], sRec, G + r * (Nx + 1));
+            } else {
+                node_coefficients(g, r, m[1], m[2], m[3], m[4], sRec, G);
+            }
+        }
+    }
+    __syncthreads();
+    // 3. lines, one output per thread and turn
+    double* coef = static_cast<double*>(g.coef);
+    const double* Tx = g.Td;
+    const double* Ty = Tx + Qx * (Nx + 1);
+    const double* Tz = Ty + VY * (Ny + 1);
+    for (int i = tid; i < nb * g.ncp; i += kNode64T) {
+        const int k = i / g.ncp, o = i - k * g.ncp;
+        const double* m = sM + 6 * k;
+        const double* G = sG + k * ncoef;
+        double v = 0.0;
+        if (o == nf) {
+            v = m[5];
+        } else if (g.has_field && o >= g.field_off && o < g.field_off + 3) {      // a = a_uniform + a_field(node)
+            const InstDev& I = g.inst[g.ninst > 1 ? find_slot(g.node_start, g.ninst, base + k) : 0];
+            const int c = o - g.field_off;
+            v = (c == 0 ? I.ax : (c == 1 ? I.ay : I.az)) + g.afield[3 * (size_t)(base + k) + c];
+        } else if (o < nf && m[5] != 0.0) {
+            const double* T;
+            int N = 0;
+            bool absent = false;
+            if (o < QX2) {
+                const int sg = o >= Qx;
+                T = Tx + (o - sg * Qx) * (Nx + 1);
+                G += sg * (Nx + 1);
+                N = Nx;
+            } else if (o < QX2 + VY) {
+                T = Ty + (o - QX2) * (Ny + 1);
+                G += 2 * (Nx + 1);
+                N = Ny;
+                absent = !g.Qy;
+            } else {
+                T = Tz + (o - QX2 - VY) * (Nz + 1);
+                G += 2 * (Nx + 1) + Ny + 1;
+                N = Nz;
+                absent = !g.Qz;
+            }
+            if (absent) {
+                v = 1.0;
+            } else {
+                double a0 = 0.0, a1 = 0.0;
+                int l = 0;
+                for (; l < N; l += 2) {
+                    a0 = fma(T[l], G[l], a0);
+                    a1 = fma(T[l + 1], G[l + 1], a1);
+                }
+                if (l == N) a0 = fma(T[l], G[l], a0);
+                v = a0 + a1;
+                if (o < QX2) v *= m[0];
+            }
+        }
+        coef[(size_t)base * g.ncp + i] = v;
+    }
+}
+
 }  // namespace
 
 cudaError_t prepare_node() {
     cudaError_t e = cudaFuncSetAttribute(coef_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(coef_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(coef_df_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
@@ -533,20 +743,23 @@ cudaError_t prepare_node() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(coef_df_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(sums_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(sums_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    return cudaFuncSetAttribute(sums_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
 }
 
-// Blocks of `func` resident on the whole GPU at once (one wave), at most
-// `want`: a grid-stride kernel then has no partly filled last wave.
-static int one_wave(const void* func, int block, size_t smem, int want) {
+static int sm_count() {
     static int nsm = 0;
     if (!nsm) {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             nsm = 152;
     }
+    return nsm;
+}
+
+// Blocks of `func` resident on the whole GPU at once (one wave), at most
+// `want`: a grid-stride kernel then has no partly filled last wave.
+static int one_wave(const void* func, int block, size_t smem, int want) {
+    const int nsm = sm_count();
     int per = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, func, block, smem) != cudaSuccess || per < 1) per = 1;
     return want < nsm * per ? (want > 0 ? want : 1) : nsm * per;
@@ -589,6 +802,21 @@ cudaError_t prepare_node_fused(int adv, const GroupDev& g) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+// The FP64 node pass and walls (every FP64 group).
+void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
+    const int NB = g.nnodes <= 2 * sm_count() ? 1 : 8;
+    const int grid = g.nrows * g.wchunks + (g.nnodes + NB - 1) / NB;
+    const size_t smem = node64_smem(g, NB);
+    const double* f = static_cast<const double*>(fs);
+    if (adv == HLB_WENO5_) {
+        if (NB == 1) node_f64_kernel<HLB_WENO5_, 1><<<grid, kNode64T, smem, st>>>(g, f);
+        else node_f64_kernel<HLB_WENO5_, 8><<<grid, kNode64T, smem, st>>>(g, f);
+    } else {
+        if (NB == 1) node_f64_kernel<HLB_UPWIND2_, 1><<<grid, kNode64T, smem, st>>>(g, f);
+        else node_f64_kernel<HLB_UPWIND2_, 8><<<grid, kNode64T, smem, st>>>(g, f);
+    }
+}
+
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
     const int grid = g.nrows * g.wchunks + (g.nnodes + kNodeNB - 1) / kNodeNB;
     const size_t smem = node_smem(g).bytes;
@@ -603,40 +831,27 @@ void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t 
     }
 }
 
-// Node pass of a stage: the quadrature sums of every node, then the factor
-// lines.  The sums live in the first 8 R of each node's factor line slot of
-// an auxiliary buffer (g.sums).
-void launch_node(int precision, const GroupDev& g, const void* fs, cudaStream_t st) {
-    const size_t es = precision == HLB_FP64_ ? 8 : 4;
-    const size_t smem_a = 4 * (g.V + g.VY * g.VZ) * es;
-    const int want_a = (g.nnodes + 7) / 8;
-    const int blocks_a = precision == HLB_FP64_
-                             ? one_wave(reinterpret_cast<const void*>(&sums_kernel<double>), 256, smem_a, want_a)
-                             : one_wave(reinterpret_cast<const void*>(&sums_kernel<float>), 256, smem_a, want_a);
+// Node pass of a stage of the FP32 groups that the one-launch pass does not
+// take: the quadrature sums of every node (in the first 8 values of each
+// node's slot of g.sums), then the factor lines.
+void launch_node(const GroupDev& g, const void* fs, cudaStream_t st) {
+    const size_t smem_a = 4 * (g.V + g.VY * g.VZ) * sizeof(float);
+    const int blocks_a = one_wave(reinterpret_cast<const void*>(&sums_kernel<float>), 256, smem_a, (g.nnodes + 7) / 8);
     const int nrec = 5 * g.Nx + 1;
-    const int nT = g.Qx * (g.Nx + 1) + g.VY * (g.Ny + 1) + g.VZ * (g.Nz + 1);
-    const int ncoef = 2 * (g.Nx + 1) + (g.Ny + 1) + (g.Nz + 1);
-    const int block_b = 32;
-    const size_t per_warp = 8 * (32 * ncoef + 64) + 32 * sizeof(NodeDF);
-    const size_t smem_b = 8 * (nrec + nT) + (block_b / 32) * per_warp;
-    const int batches = (g.nnodes + 31) / 32;
-    const int blocks_b = batches;
-    if (precision == HLB_FP64_) {
-        sums_kernel<double><<<blocks_a, 256, smem_a, st>>>(g, (const double*)fs, (double*)g.sums);
-        coef_kernel<double><<<blocks_b, block_b, smem_b, st>>>(g, (const double*)g.sums);
+    sums_kernel<float><<<blocks_a, 256, smem_a, st>>>(g, (const float*)fs, (float*)g.sums);
+    const int nmax = max(g.Nx, max(g.Ny, g.Nz));
+    if (g.use_df && nmax < 16) {
+        const int nP = (g.Qx + 1) / 2 * (g.Nx + 1) + (g.VY + 1) / 2 * (g.Ny + 1) + (g.VZ + 1) / 2 * (g.Nz + 1);
+        const size_t smem_c = 16 * ((size_t)nP + (nrec + 1) / 2) + 4 * 32 * (size_t)g.ncp * 4;
+        const int blocks_c = (g.nnodes + 127) / 128;
+        if (nmax < 8) coef_df_kernel<8><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
+        else if (nmax < 12) coef_df_kernel<12><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
+        else coef_df_kernel<16><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
     } else {
-        sums_kernel<float><<<blocks_a, 256, smem_a, st>>>(g, (const float*)fs, (float*)g.sums);
-        const int nmax = max(g.Nx, max(g.Ny, g.Nz));
-        if (g.use_df && nmax < 16) {
-            const int nP = (g.Qx + 1) / 2 * (g.Nx + 1) + (g.VY + 1) / 2 * (g.Ny + 1) + (g.VZ + 1) / 2 * (g.Nz + 1);
-            const size_t smem_c = 16 * ((size_t)nP + (nrec + 1) / 2) + 4 * 32 * (size_t)g.ncp * 4;
-            const int blocks_c = (g.nnodes + 127) / 128;
-            if (nmax < 8) coef_df_kernel<8><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
-            else if (nmax < 12) coef_df_kernel<12><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
-            else coef_df_kernel<16><<<blocks_c, 128, smem_c, st>>>(g, (const float*)g.sums);
-        } else {
-            coef_kernel<float><<<blocks_b, block_b, smem_b, st>>>(g, (const float*)g.sums);
-        }
+        const int nT = g.Qx * (g.Nx + 1) + g.VY * (g.Ny + 1) + g.VZ * (g.Nz + 1);
+        const int ncoef = 2 * (g.Nx + 1) + (g.Ny + 1) + (g.Nz + 1);
+        const size_t smem_b = 8 * (nrec + nT) + 8 * (32 * ncoef + 64) + 32 * sizeof(NodeDF);
+        coef_kernel<float><<<(g.nnodes + 31) / 32, 32, smem_b, st>>>(g, (const float*)g.sums);
     }
 }
 
