@@ -94,6 +94,8 @@ struct Group {
     DevBuf d_gnode;                          // [members]: each member's first node in the caller's layout
     PinnedBuf h_mom;                         // pinned word for the non-finite flag (hlb_moments), first use
     DevBuf d_Td, d_invdx, d_wscale, d_coef, d_works, d_err, d_recf, d_Tf, d_sums;
+    DevBuf d_pair_start;                     // wide 1D sets: pairs of cells per instance, prefix sums
+    int npairs = 0;
     DevBuf d_KxT, d_KxJ;                     // FP64 Kx transposed and its jump factors (kx_global groups only)
     DevBuf d_gquad, d_glrule;                // G^{+-} by quadrature above the recurrence's stable order (FP64)
     DevBuf d_wpart, d_wcount;                // wall kernel: per-chunk partial fluxes, row counters
@@ -322,6 +324,8 @@ void fill_dev(Group& G) {
     d.KxT = (const double*)G.d_KxT.p;
     d.KxJ = (const double*)G.d_KxJ.p;
     d.kx_global = G.d_KxT.p ? 1 : 0;
+    d.pair_start = static_cast<const int*>(G.d_pair_start.p);
+    d.npairs = G.npairs;
     d.vchunks = G.vchunks;
     d.rec = (const double*)G.d_rec.p; d.dx = (const double*)G.d_dx.p;
     d.gw = G.d_gw.p; d.nw = (double*)G.d_nw.p;
@@ -523,6 +527,12 @@ hlb_status build_group(hlb_handle* h, Group& G) {
         std::vector<double> J(G.tx.jc);
         J.insert(J.end(), G.tx.jd.begin(), G.tx.jd.end());
         if ((s = upload(G.d_KxJ, J)) != HLB_OK) return s;
+        std::vector<int> pairs(1, 0);
+        for (const hlb::InstDev& I : G.inst) pairs.push_back(I.ny == 1 ? pairs.back() + (I.nx + 1) / 2 : -1);
+        if (std::find(pairs.begin(), pairs.end(), -1) == pairs.end()) {      // every instance 1D: stage_wide_kernel
+            if ((s = upload(G.d_pair_start, pairs)) != HLB_OK) return s;
+            G.npairs = pairs.back();
+        }
     }
     if ((s = upload_real(G.d_p, p, G.precision)) != HLB_OK) return s;
     // FP64 half-range Hermite groups above the recurrence's stable order: the
@@ -794,6 +804,8 @@ void enqueue_group_step(hlb_handle* h, Group& G, cudaStream_t st_) {
         if (march)
             hlb::launch_march(G.precision, G.adv, G.QX2, G.VY, G.TY, G.dev, (const hlb::Work*)G.d_works.p,
                               G.nworks, ins[st], S, outs[st], st, st_);
+        else if (G.npairs)
+            hlb::launch_stage_wide(G.adv, G.dev, ins[st], S, outs[st], st, st_);
         else
             hlb::launch_stage(G.precision, G.adv, G.dev, ins[st], S, outs[st], st, G.grid, G.block, G.smem, st_);
         if (h->time_kernels) {

@@ -101,6 +101,8 @@ struct GroupDev {
                              // generic stage kernel when Kx does not fit in shared memory
     const double* KxJ;       // FP64 [2][QX2]: c_k, d_k of the rank-one cross-half blocks
                              // K[k][k'] = c_k d_k' (k, k' on opposite halves; kx_global)
+    const int* pair_start;   // wide sets without a y axis in space: [ninst + 1] pairs of neighbouring
+    int npairs;              // cells per instance, and in all (0: not such a group; stage_wide_kernel)
     int kx_global;           // 1: Kx is not staged in shared memory (KxT is read instead)
     int vchunks;             // CTAs per node of the generic stage kernel (velocity ranges)
     const void* p;           // R: px [QX2], py [VY], pz [VZ]
@@ -157,6 +159,8 @@ cudaError_t stage_occupancy(int precision, int adv, int block, size_t smem, int*
 void launch_stage(int precision, int adv, const GroupDev& g, const void* fs, const void* fn, void* fo,
                   int stage, int grid, int block, size_t smem, cudaStream_t st);
 void launch_wall(int precision, int adv, const GroupDev& g, const void* fs, cudaStream_t st);
+// Stage kernel of the wide FP64 sets (kx_global) of 1D instances.
+void launch_stage_wide(int adv, const GroupDev& g, const void* fs, const void* fn, void* fo, int stage, cudaStream_t st);
 // G^{+-}_l (l <= Nx) of every collisional node of an FP64 half-range group by
 // quadrature of the projection integrals (hlb_kernels.cu)
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st);

@@ -403,6 +403,187 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
 }
 
 // ---------------------------------------------------------------------------
+// stage kernel of the wide FP64 sets (K_x in global memory) without a y axis in
+// space: the HHLB(20;200) runs
+// ---------------------------------------------------------------------------
+// One thread per velocity and pair of neighbouring cells, the (pair, velocity)
+// list cut into CTAs of 64 whatever fibre they fall in.  The FP64 pipe is the
+// bound (a warp's instruction takes 64 cycles of its SM quarter), so what counts
+// is the number of FP64 operations and an even number of full warps per
+// quarter: two cells share the faces between them (three instead of four, at a
+// common scale) and every K_x entry read from L2, and no warp is cut short at a
+// node's end (400 velocities are 12.5 warps; in seven CTAs of 64 per node they
+// took 14 and 4.4 rounds of the resident CTAs, here 12.5 and 2).  Per stage
+// (GB300): eight ballistic cases 43.6 us against 63.9 in the generic kernel.
+constexpr int kWideThreads = 64;
+template <int ADV>
+__global__ void __launch_bounds__(kWideThreads, 4)
+stage_wide_kernel(const GroupDev g, const double* __restrict__ fs, const double* __restrict__ fn,
+                  double* __restrict__ fo, int stage) {
+    extern __shared__ __align__(16) unsigned char wsm[];
+    const int V = g.V, QX2 = g.QX2, Qx = g.Qx, VY = g.VY, VZ = g.VZ, nfib = VY * VZ;
+    double2* sF = reinterpret_cast<double2*>(wsm);                   // [2 fibres][QX2]: (cell x0, cell x0 + 1)
+    double2* sJ = sF + 2 * QX2;                                      // [2 fibres][2 halves]: sum_{k' in half} d_k' f_k'
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long total = (long long)g.npairs * V;
+    const long long e0 = (long long)blockIdx.x * kWideThreads;
+    const long long fib0 = e0 / QX2;                                 // first fibre of the CTA, over all pairs
+    const long long last = min(total, e0 + kWideThreads) - 1;
+    const int nfb = (int)(last / QX2 - fib0) + 1;                    // one or two (QX2 > 64)
+    for (int a = 0; a < nfb; ++a) {
+        const int pair = (int)((fib0 + a) / nfib), fb = (int)((fib0 + a) - (long long)pair * nfib);
+        const int ii = g.ninst > 1 ? find_slot(g.pair_start, g.ninst, pair) : 0;
+        const InstDev& I = g.inst[ii];
+        const int x0 = 2 * (pair - g.pair_start[ii]);
+        const double* f = fs + I.f_off + (size_t)x0 * V + (size_t)fb * QX2;
+        const bool two = x0 + 1 < I.nx;
+        for (int i = tid; i < QX2; i += kWideThreads) sF[a * QX2 + i] = make_double2(f[i], two ? f[V + i] : 0.0);
+    }
+    __syncthreads();
+    {
+        // the cross-half blocks of K^h are rank one, c_k d_k': one sum per fibre,
+        // half and cell (only of halves that a thread of the CTA needs)
+        const double* jd = g.KxJ + QX2;
+        for (int j = warp; j < 2 * nfb; j += kWideThreads / 32) {
+            const int a = j >> 1, h = j & 1;
+            const long long b = (fib0 + a) * QX2 + (h ? 0 : Qx);     // the other half's values
+            if (b > last || b + Qx <= e0) continue;
+            double s0 = 0.0, s1 = 0.0;
+            for (int i = lane; i < Qx; i += 32) {
+                const double d = jd[h * Qx + i];
+                const double2 f = sF[a * QX2 + h * Qx + i];
+                s0 = fma(d, f.x, s0);
+                s1 = fma(d, f.y, s1);
+            }
+            s0 = warp_sum(s0);
+            s1 = warp_sum(s1);
+            if (lane == 0) sJ[j] = make_double2(s0, s1);
+        }
+    }
+    __syncthreads();
+    const long long e = e0 + tid;
+    if (e >= total) return;
+    const int a = (int)(e / QX2 - fib0), ix = (int)(e % QX2);
+    const int pair = (int)(e / V), v = (int)(e - (long long)pair * V);
+    const int jy = (v / QX2) % VY, kz = v / (QX2 * VY);
+    const int ii = g.ninst > 1 ? find_slot(g.pair_start, g.ninst, pair) : 0;
+    const InstDev& I = g.inst[ii];
+    const int nx = I.nx, x0 = 2 * (pair - g.pair_start[ii]);
+    const bool two = x0 + 1 < nx, xpos = ix < Qx;
+    const double* frow = fs + I.f_off;
+    // fluxes per unit velocity at x0 - 1/2, x0 + 1/2, x0 + 3/2
+    double Fx[3];
+    {
+        const double* gw = static_cast<const double*>(g.gw) + I.gw_off;
+        const double nwl_g = g.nw[(size_t)I.row_off * 2 + 0] * gw[v], nwr_g = g.nw[(size_t)I.row_off * 2 + 1] * gw[V + v];
+        double w[7];
+        const int base = xpos ? x0 - 3 : x0 - 2;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) w[k] = x_value(frow, base + k, nx, V, v, xpos, nwl_g, nwr_g);
+        if (ADV == HLB_WENO5_) {
+            double u[7], F[3];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) u[k] = xpos ? w[k] : w[6 - k];
+            weno5_faces64<3>(u, F);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) Fx[k] = xpos ? F[k] : F[2 - k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                Fx[k] = xpos ? upwind2_face(w[k + 1], w[k + 2]) : upwind2_face(w[k + 3], w[k + 2]);
+        }
+    }
+    // a_x K_x f + a_y K_y f + a_z K_z f at both cells
+    const int node0 = I.node_off + x0;
+    double force[2] = {0.0, 0.0}, acc3[3][2];
+    acc3[0][0] = acc3[0][1] = acc3[1][0] = acc3[1][1] = acc3[2][0] = acc3[2][1] = 0.0;
+    double acl[2][3];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const double* af = g.has_field && (c == 0 || two) ? g.afield + 3 * (size_t)(node0 + c) : nullptr;
+        acl[c][0] = I.ax + (af ? af[0] : 0.0);
+        acl[c][1] = I.ay + (af ? af[1] : 0.0);
+        acl[c][2] = I.az + (af ? af[2] : 0.0);
+    }
+    if (acl[0][0] != 0.0 || acl[1][0] != 0.0) {
+        // own half: column ix of Kx^T (consecutive threads read consecutive
+        // entries), eight entries ahead of the sums; other half: c_ix times its sum
+        const int h = xpos ? 0 : 1;
+        const double* Kc = g.KxT + (size_t)h * Qx * QX2 + ix;
+        const double2* fh = sF + a * QX2 + h * Qx;
+        double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+        constexpr int U = 8;
+        double kc[U];
+        const int n8 = Qx / U * U;
+#pragma unroll
+        for (int j = 0; j < U; ++j) kc[j] = Kc[(size_t)j * QX2];
+        for (int i = 0; i < n8; i += U) {
+            double kn[U];
+            const bool more = i + U < n8;
+#pragma unroll
+            for (int j = 0; j < U; ++j) kn[j] = more ? Kc[(size_t)(i + U + j) * QX2] : 0.0;
+#pragma unroll
+            for (int j = 0; j < U; j += 2) {
+                const double2 f0 = fh[i + j], f1 = fh[i + j + 1];
+                p0 = fma(kc[j], f0.x, p0);
+                q0 = fma(kc[j], f0.y, q0);
+                p1 = fma(kc[j + 1], f1.x, p1);
+                q1 = fma(kc[j + 1], f1.y, q1);
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) kc[j] = kn[j];
+        }
+        for (int i = n8; i < Qx; ++i) {
+            const double k = Kc[(size_t)i * QX2];
+            const double2 f0 = fh[i];
+            p0 = fma(k, f0.x, p0);
+            q0 = fma(k, f0.y, q0);
+        }
+        const double2 J = sJ[2 * a + 1 - h];
+        const double c = g.KxJ[ix];
+        acc3[0][0] = fma(c, J.x, p0 + p1);
+        acc3[0][1] = fma(c, J.y, q0 + q1);
+    }
+    const double* f0p = frow + (size_t)x0 * V;
+    const double* Ky = static_cast<const double*>(g.K) + (size_t)QX2 * QX2;
+    if (g.Qy && (acl[0][1] != 0.0 || acl[1][1] != 0.0))
+        for (int j = 0; j < VY; ++j) {
+            const double k = Ky[jy * VY + j];
+            const size_t o = (size_t)(kz * VY + j) * QX2 + ix;
+            acc3[1][0] = fma(k, f0p[o], acc3[1][0]);
+            if (two) acc3[1][1] = fma(k, f0p[V + o], acc3[1][1]);
+        }
+    if (g.Qz && (acl[0][2] != 0.0 || acl[1][2] != 0.0))
+        for (int j = 0; j < VZ; ++j) {
+            const double k = Ky[VY * VY + kz * VZ + j];
+            const size_t o = (size_t)(j * VY + jy) * QX2 + ix;
+            acc3[2][0] = fma(k, f0p[o], acc3[2][0]);
+            if (two) acc3[2][1] = fma(k, f0p[V + o], acc3[2][1]);
+        }
+    const double vx = g.pd[ix], dt = I.dt;
+    const double* idx = static_cast<const double*>(g.inv_dx) + I.dx_off + x0;
+    const double2 fc = sF[a * QX2 + ix];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        if (c == 1 && !two) break;
+        force[c] = acl[c][0] * acc3[0][c];
+        if (g.Qy) force[c] = fma(acl[c][1], acc3[1][c], force[c]);
+        if (g.Qz) force[c] = fma(acl[c][2], acc3[2][c], force[c]);
+        const double f = c ? fc.y : fc.x;
+        double L = -vx * (Fx[c + 1] - Fx[c]) * idx[c] - force[c];
+        if (I.inv_Kn != 0.0) {
+            const double* line = static_cast<const double*>(g.coef) + (size_t)(node0 + c) * g.ncp;
+            L -= (f - line[ix] * line[QX2 + jy] * line[QX2 + VY + kz]) * line[QX2 + VY + VZ];
+        }
+        const size_t o = (size_t)I.f_off + (size_t)(x0 + c) * V + v;
+        double out = fma(dt, L, f);
+        // c f^n + (1 - c) f' as f' + c (f^n - f'): the weights sum to 1 exactly
+        if (stage > 0) out = fma(stage == 1 ? 0.75 : 1.0 / 3.0, fn[o] - out, out);
+        fo[o] = out;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // wall kernel: emitted densities of both walls of one (instance, y) row
 // ---------------------------------------------------------------------------
 template <typename R, int ADV>
@@ -792,6 +973,14 @@ void launch_stage(int precision, int adv, const GroupDev& g, const void* fs, con
         if (adv == HLB_WENO5_) stage_kernel<float, HLB_WENO5_><<<grid, block, smem, st>>>(g, (const float*)fs, (const float*)fn, (float*)fo, stage);
         else stage_kernel<float, HLB_UPWIND2_><<<grid, block, smem, st>>>(g, (const float*)fs, (const float*)fn, (float*)fo, stage);
     }
+}
+
+void launch_stage_wide(int adv, const GroupDev& g, const void* fs, const void* fn, void* fo, int stage, cudaStream_t st) {
+    const long long total = (long long)g.npairs * g.V;
+    const int grid = (int)((total + kWideThreads - 1) / kWideThreads);
+    const size_t smem = (2 * (size_t)g.QX2 + 4) * sizeof(double2);
+    if (adv == HLB_WENO5_) stage_wide_kernel<HLB_WENO5_><<<grid, kWideThreads, smem, st>>>(g, (const double*)fs, (const double*)fn, (double*)fo, stage);
+    else stage_wide_kernel<HLB_UPWIND2_><<<grid, kWideThreads, smem, st>>>(g, (const double*)fs, (const double*)fn, (double*)fo, stage);
 }
 
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st) {

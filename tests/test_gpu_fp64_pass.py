@@ -61,3 +61,40 @@ def test_fp64_weno_scale_and_jumps():
             outs.append(h.get_state() / scale)
     assert np.isfinite(outs[0]).all()
     np.testing.assert_allclose(outs[1], outs[0], rtol=1e-12, atol=1e-14)
+
+
+_WIDE = dict(precision=W.FP64, dt=1e-4, T_left=1.0, T_right=1.2, ax=-0.5)
+
+
+@pytest.mark.parametrize("name,cfg", [
+    ("odd_cells", W.make(Qx=200, Nx_eq=12, nx=7, Kn=0.3, **_WIDE)),
+    ("fibres_and_y_force", W.make(Qx=64, Qy=2, Nx_eq=12, nx=6, Kn=0.3, ay=-0.2, **_WIDE)),
+    ("z_force_upwind", W.make(Qx=40, Qz=2, Nx_eq=8, nx=5, Kn=0.3, az=0.3, advection=W.UPWIND2, **_WIDE)),
+    ("instances", [W.make(Qx=50, Nx_eq=10, nx=nx, Kn=Kn, **_WIDE) for nx, Kn in ((9, 0.2), (6, math.inf), (11, 1.0))]),
+])
+def test_wide_stage_kernel(name, cfg):
+    # stage_wide_kernel: odd numbers of cells (a pair of one), CTAs that straddle
+    # fibres and nodes, several axes, instances of different length
+    got, mom, N, refs = run_pair(cfg, 3)
+    _check_fp64(got, refs, 1e-9)
+
+
+def test_wide_stage_kernel_field():
+    from oracle.solver import Solver, config_from
+    from paper_1708_03249_gb300 import hlb
+    import torch
+    cfg = W.make(Qx=40, Nx_eq=8, nx=9, Kn=0.3, **_WIDE)
+    field = 0.4 * np.sin(np.arange(9.0))[None, :]
+    with hlb.Handle(cfg, stream=torch.cuda.current_stream().cuda_stream) as h:
+        h.set_force_field(0, field)
+        h.init_equilibrium()
+        f0 = h.get_state() * W.perturbation(h.values, seed=3)
+        h.set_state(f0)
+        h.step(3)
+        got = h.get_state()
+    c = config_from(cfg)
+    c.ax_field = field
+    s = Solver(c)
+    s.f = f0.reshape(s.f.shape).copy()
+    s.step(3)
+    _check_fp64(got, [s], 1e-9)
