@@ -907,6 +907,112 @@ moments_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, double
     }
 }
 
+// The moments of FP32 groups with 2Q_x a power of two up to 32: 32 nodes per CTA
+// of 128 threads, the nine sums of a node by eight lanes as in moments_kernel's
+// 4-vector path (the same loop, lane by lane: how the compiler joins its packed
+// products and sums shows in the last digits of u and q), then one thread per
+// node in FP64.  HBM-bound work: what counts is enough loads in flight, so the
+// sums of finished nodes wait in shared memory and the kernel stays at 80
+// registers, 24 warps per SM (moments_kernel keeps them in registers: 104, 16
+// warps of 256-thread CTAs, 30 % of the DRAM rate).  1024 x 512 nodes of 1024
+// velocities (GB300): 0.459 ms against 0.771; reading the state alone takes 0.317.
+constexpr int kMomNodes = 32, kMomThreads = 128;
+template <typename R>
+__global__ void __launch_bounds__(kMomThreads, 6)
+moments_rows_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, double* u_out, double* T_out,
+                    double* q_out, int node_base, const long long* __restrict__ gnode) {
+    extern __shared__ __align__(16) unsigned char mom_smem[];
+    __shared__ long long sOff[kMomNodes];
+    __shared__ float sSum[kMomNodes][21];                // nine sums, nine error terms (padded)
+    float4* sYZ = reinterpret_cast<float4*>(mom_smem);   // [VY VZ]: p_y, p_z, p_y^2 + p_z^2
+    const int V = g.V, QX2 = g.QX2, VY = g.VY, rows = g.VY * g.VZ;
+    const R* P = static_cast<const R*>(g.p);
+    const int tid = threadIdx.x, base = blockIdx.x * kMomNodes, nb = min(kMomNodes, g.nnodes - base);
+    int ii = 0;
+    if (tid < nb) {
+        ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, base + tid) : 0;
+        sOff[tid] = g.inst[ii].f_off + (long long)(base + tid - g.inst[ii].node_off) * V;
+    }
+    for (int k = tid; k < rows; k += kMomThreads) {
+        float4 y;
+        y.x = P[QX2 + k % VY]; y.y = P[QX2 + VY + k / VY]; y.z = y.x * y.x + y.y * y.y; y.w = R(0);
+        sYZ[k] = y;
+    }
+    __syncthreads();
+    const int lane = tid & 31, sl = lane & 7, lg = __ffs(QX2) - 1;
+    const int x0 = (4 * sl) & (QX2 - 1);
+    R px[4], px2[4], px3[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        px[e] = P[x0 + e]; px2[e] = px[e] * px[e]; px3[e] = px2[e] * px[e];
+    }
+    for (int kn = tid >> 3; (kn & ~3) < nb; kn += kMomThreads / 8) {
+        float2 s2[5], c2[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) s2[q] = c2[q] = make_float2(0.0f, 0.0f);
+        if (kn < nb) {
+            const float4* f4 = reinterpret_cast<const float4*>(fs + sOff[kn]);
+            float2 pjx[4], p13[4];                   // (p_x, p_x^2), (1, p_x^3) per element
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                pjx[e] = make_float2((float)px[e], (float)px2[e]);
+                p13[e] = make_float2(1.0f, (float)px3[e]);
+            }
+#pragma unroll 4
+            for (int k = sl; k < (V >> 2); k += 8) {
+                const float4 x = __ldcs(f4 + k);
+                const float4 yz = sYZ[k >> (lg - 2)];
+                const float xe[4] = {x.x, x.y, x.z, x.w};
+                float2 jp = make_float2(0.0f, 0.0f), sq = make_float2(0.0f, 0.0f);   // (j_x, P_xx), (n, Q_x)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    jp = __ffma2_rn(pjx[e], f2(xe[e]), jp);
+                    sq = __ffma2_rn(p13[e], f2(xe[e]), sq);
+                }
+                const float2 yzv = make_float2(yz.x, yz.y);
+                csum_add2(s2[0], c2[0], make_float2(sq.x, jp.x));
+                csum_add2(s2[1], c2[1], __fmul2_rn(yzv, f2(sq.x)));
+                csum_add2(s2[2], c2[2], make_float2(jp.y, yz.z * sq.x));
+                csum_add2(s2[3], c2[3], __fmul2_rn(yzv, f2(jp.x)));
+                csum_add2(s2[4], c2[4], make_float2(fmaf(yz.z, jp.x, sq.y), 0.0f));
+            }
+        }
+        R a[9], c[9];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            a[2 * q] = s2[q].x; c[2 * q] = c2[q].x;
+            if (q < 4) { a[2 * q + 1] = s2[q].y; c[2 * q + 1] = c2[q].y; }
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            csum_warp<R, 4>(a[k], c[k]);
+            if (sl == 0 && kn < nb) {
+                sSum[kn][k] = a[k];
+                sSum[kn][10 + k] = c[k];
+            }
+        }
+    }
+    __syncthreads();
+    if (tid < nb) {
+        const int node = base + tid;
+        double d[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) d[k] = (double)sSum[tid][k] + (double)sSum[tid][10 + k];
+        const double n = d[0];
+        const double ux = d[1] / n, uy = d[2] / n, uz = d[3] / n;
+        const double u2 = ux * ux + uy * uy + uz * uz;
+        const double E = d[4] + d[5];
+        const double Tn = (E - n * u2) / (g.D * n);
+        const double qx = 0.5 * (d[8] - 2.0 * (ux * d[4] + uy * d[6] + uz * d[7]) - ux * E + 2.0 * n * ux * u2);
+        const long long o = gnode ? gnode[ii] + (node - g.node_start[ii]) : (long long)node_base + node;
+        if (n_out) n_out[o] = n;
+        if (u_out) { u_out[3 * o] = ux; u_out[3 * o + 1] = uy; u_out[3 * o + 2] = uz; }
+        if (T_out) T_out[o] = Tn;
+        if (q_out) q_out[o] = qx;
+        if (!(isfinite(n) && isfinite(Tn))) *g.nonfinite = 1;
+    }
+}
+
 __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
     atomicMax(reinterpret_cast<unsigned long long*>(addr), (unsigned long long)__double_as_longlong(v));
 }
@@ -1012,6 +1118,11 @@ void launch_moments(int precision, const GroupDev& g, const void* fs, double* n,
     const int block = 256;                               // 8 warps, 32 nodes per warp and batch
     const int grid = (g.nnodes + 255) / 256 < 152 * 8 ? (g.nnodes + 255) / 256 : 152 * 8;
     const bool table = g.V + g.VY * g.VZ <= kMomentTableMax;
+    if (precision != HLB_FP64_ && table && (g.QX2 & 3) == 0 && (g.QX2 & (g.QX2 - 1)) == 0 && g.QX2 <= 32) {
+        moments_rows_kernel<float><<<(g.nnodes + kMomNodes - 1) / kMomNodes, kMomThreads, g.VY * g.VZ * sizeof(float4), st>>>(
+            g, (const float*)fs, n, u, T, q, node_base, gnode);
+        return;
+    }
     if (precision == HLB_FP64_) {
         if (table) moments_kernel<double, true><<<grid, block, (g.V + g.VY * g.VZ) * sizeof(double4), st>>>(g, (const double*)fs, n, u, T, q, node_base, gnode);
         else moments_kernel<double, false><<<grid, block, 0, st>>>(g, (const double*)fs, n, u, T, q, node_base, gnode);
