@@ -156,18 +156,22 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
     // Copy `lane` of pair p (22 lanes: 12 halo rows, 4 head rows, 4 f^n rows,
     // 2 factor-line runs): source, bytes and destination in B; false if the
     // lane has none for this pair.
-    // The copies are spread over the warps so that no warp carries them all:
-    // with four or more warps, warps 0 and 1 take the halo rows of cells x0
-    // and x0+1, warp 2 the head rows and factor lines, warp 3 the f^n rows; a
-    // single warp takes all 22.  Thread 0 registers each pair's byte count
+    // Slabs of up to four warps take turns: pair p's copies are issued by warp p %
+    // (S / 32), so that each warp runs the issue code once in that many pairs
+    // (large channel, 16 x 8 slabs: 2.90 against 2.92 ms per stage with the
+    // copies spread over the warps).  With 16 warps the spread is the better one
+    // (32 x 16 slabs of the 256^2 box: 296 against 298 us): warps 0 and 1 take the
+    // halo rows of cells x0 and x0+1, warp 2 the head rows and factor lines, warp
+    // 3 the f^n rows.  Thread 0 registers each pair's byte count
     // (arrive.expect_tx) before any warp can issue that pair's copies.
+    constexpr bool kTurns = S / 32 <= 4;
     int my_copy = -1;
-    if (S / 32 >= 4) {
+    if (kTurns) {
+        my_copy = lane < 22 ? lane : -1;
+    } else {
         if (warp < 2 && lane < 6) my_copy = 6 * warp + lane;
         else if (warp == 2 && lane < 6) my_copy = lane < 4 ? 12 + lane : 16 + lane;    // 12..15, 20..21
         else if (warp == 3 && lane < 4) my_copy = 16 + lane;
-    } else if (warp == 0 && lane < 22) {
-        my_copy = lane;
     }
     auto expect = [&](int p) {                     // thread 0 only
         if (p >= npairs || (g.inject_stall && p == 1)) return;   // test hook: pair 1 never arrives
@@ -211,7 +215,7 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         cp_kind = 3;
     }
     auto issue = [&](int p) {
-        if (my_copy < 0 || p >= npairs || (g.inject_stall && p == 1)) return;
+        if ((kTurns && p % (S / 32) != warp) || my_copy < 0 || p >= npairs || (g.inject_stall && p == 1)) return;
         const int x0 = xa + 2 * p;
         const int n2 = min(2, xb - x0);
         bool go = cp_i < n2;
