@@ -121,6 +121,7 @@ struct Group {
     // items of a stage (per instance its node chunks, then its segments),
     // node chunks and segments per instance, resident CTAs
     bool persist_ok = false;
+    bool pdl = false;                        // dependent launches (a handle's only group, not a large one)
     bool node_fused = false;                 // the node pass and the walls in one launch
     bool persist_auto = false;               // steps with it unless told otherwise (hlb_set_persistent)
     bool persist_use = true;                 // the autotuner's pick: persistent or per-stage launches
@@ -350,6 +351,7 @@ void fill_dev(Group& G) {
     d.force_form = march_form(G);
     d.sround = G.sround && G.precision == HLB_FP32 ? 1 : 0;
     d.quad_x = G.quad_x ? 1 : 0;
+    d.pdl = G.pdl ? 1 : 0;
     d.wchunks = G.wchunks;
     d.wpart = static_cast<double*>(G.d_wpart.p);
     d.wcount = static_cast<unsigned*>(G.d_wcount.p);
@@ -635,6 +637,11 @@ hlb_status build_group(hlb_handle* h, Group& G) {
             const long long N = (strips + resident - 1) / resident;
             long long sx = std::min(N, std::max(two_d ? 32LL : 48LL, std::min(132LL, N / 4)));
             sx = std::max(4LL, two_d ? (sx + 1) / 2 * 2 : (sx + 3) / 4 * 4);
+            // FP64: one cell per step, and the FP64 pipe, not the resident warps, is
+            // what an SM has: twice the CTAs even
+            // out over the SMs (95 x 61 cells of 128 velocities 795
+            // against 893 us per step, the 64-cell channel 40.9 against 48.2).
+            if (G.precision == HLB_FP64) sx = std::max(2LL, (sx / 2 + 1) / 2 * 2);
             // the force term's form (below) decides the persistent kernel's
             // eligibility, and that the segment bound: resolve the form first
             G.force_form = 0;
@@ -972,6 +979,15 @@ hlb_status hlb_create(const hlb_config* cfg, int ninst, void* cuda_stream, hlb_h
     for (auto& G : h->groups) {
         hlb_status s = build_group(h.get(), *G);
         if (s != HLB_OK) return s;
+        // Dependent launches hide the launch and set-up of a stage's kernels.  A
+        // waiting CTA holds its registers and shared memory: with several groups
+        // stepping side by side that costs more than it hides (37 channels in
+        // three groups 135 against 123 us per step), and in a large group the
+        // launch is nothing (1024 x 512 x 1024 velocities 10.28 against 10.19 ms);
+        // 64 cells of the FP64 channel take 48.2 against 51.3 us, 512 of the
+        // stretched one 31.3 against 39, the 256^2 box 1097 against 1114 (GB300).
+        G->pdl = h->groups.size() == 1 && G->nvalues <= (1LL << 27) && !G->npairs;
+        G->dev.pdl = G->pdl ? 1 : 0;
     }
     h->inst_node_off.resize(ninst);
     h->inst_value_off.resize(ninst);

@@ -11,6 +11,18 @@ namespace hlb {
 
 constexpr double kSqrt2Pi = 2.5066282746310005024157652848110;
 
+// Programmatic dependent launch (launch_dependent, hlb_internal.h): a stage's
+// kernels follow one another in a stream, and each one's launch and set-up can
+// run while the one before it drains.  pdl_trigger lets the next kernel's CTAs
+// start once every CTA of this one has; pdl_wait returns when the kernels before
+// this one are complete and their writes visible, at once in an ordinary launch.
+// Nothing that an earlier kernel of the step writes may be read, and nothing in
+// global memory written, before pdl_wait.  (State pointers of such kernels are not
+// __restrict__: loads through them would count as invariant and could be
+// moved above the wait.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename R> __device__ __forceinline__ R rabs(R x) { return x < R(0) ? -x : x; }
 template <typename R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
 

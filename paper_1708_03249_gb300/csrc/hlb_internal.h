@@ -142,12 +142,35 @@ struct GroupDev {
     // per-node acceleration field (hlb_set_force_field): the node pass writes
     // a = a_uniform + a_field(node) into slots field_off .. field_off+2 of the
     // factor line, which every line reserves; afield [nnodes][3] FP64
+    int pdl;                 // the step's kernels are launched as dependents (launch_dependent)
     int has_field;
     int field_off;
     const double* afield;
 };
 constexpr int kQuadNodes = 20;   // points per panel of the projection quadrature
 
+}  // namespace hlb
+
+// Launch of a kernel that calls pdl_wait (hlb_device.cuh) before it touches
+// what the kernel before it in the stream writes: with `dependent`, its launch
+// overlaps the end of that kernel (hlb_api.cu says where that pays).
+#include <cuda_runtime.h>
+namespace hlb {
+template <typename... P, typename... A>
+inline void launch_dependent(bool dependent, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
+                             A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 }  // namespace hlb
 
 // Launchers (hlb_kernels.cu, hlb_node.cu, hlb_march.cu, hlb_pair.cu, hlb_line.cu).

@@ -52,8 +52,9 @@ constexpr size_t line_smem_bytes() {
 // rounded stochastically (rk3_out_sr2, hlb_device.cuh).
 template <int ADV, int QX2, int VY, int FM, int FF, int SR = 0>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? 8 : (QX2 * VY <= 256 ? 4 : 2))))
-march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __restrict__ fs,
-              const float* __restrict__ fn, float* __restrict__ fo, int stage) {
+march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs,
+              const float* fn, float* fo, int stage) {
+    pdl_trigger();
     constexpr int S = QX2 * VY;
     static_assert(S % 32 == 0, "the exchange barrier counts whole warps");
     constexpr int QX = QX2 / 2;
@@ -119,8 +120,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
     const float* gw = static_cast<const float*>(g.gw) + I.gw_off;
     const int row = W.y0;                                   // 0 for a 1D instance
     const int roff = row * nx * V, crow = row * nx;
-    const float nwl = (float)g.nw[(size_t)(I.row_off + row) * 2 + 0] * gw[v] * sv;        // scaled emitted ghosts
-    const float nwr = (float)g.nw[(size_t)(I.row_off + row) * 2 + 1] * gw[V + v] * sv;
+    const float gwl = gw[v] * sv, gwr = gw[V + v] * sv;
     const int xa = W.xa, xb = W.xb;
     const int niter = (xb - xa + 3) >> 2;
     const int slab = kz * S;
@@ -172,7 +172,10 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
         for (int p = 0; p < kLineDepth - 1; ++p) expect(p);
     }
     __syncthreads();
+    pdl_wait();                                             // from here on: the state, the walls, the factor lines
     for (int p = 0; p < kLineDepth - 1; ++p) issue(p);
+    const float nwl = (float)g.nw[(size_t)(I.row_off + row) * 2 + 0] * gwl;        // scaled emitted ghosts
+    const float nwr = (float)g.nw[(size_t)(I.row_off + row) * 2 + 1] * gwr;
 
     // scaled window of cells xa-3 .. xa+6 (wall ghosts of Sec. IV.C.3); w[0..5] filled here
     float w[10];
@@ -346,8 +349,8 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* __r
 template <int ADV, int QX2, int VY, int FM, int FF = 0, int SR = 0>
 void launch_line_t(const GroupDev& g, const Work* works, int nworks, const void* fs, const void* fn, void* fo,
                    int stage, cudaStream_t st) {
-    march1_kernel<ADV, QX2, VY, FM, FF, SR><<<nworks, QX2 * VY, line_smem_bytes<QX2, VY, FM>(), st>>>(
-        g, works, (const float*)fs, (const float*)fn, (float*)fo, stage);
+    launch_dependent(g.pdl, march1_kernel<ADV, QX2, VY, FM, FF, SR>, nworks, QX2 * VY, line_smem_bytes<QX2, VY, FM>(), st, g,
+                     works, (const float*)fs, (const float*)fn, (float*)fo, stage);
 }
 
 template <int ADV, int QX2, int VY, int FM, int FF = 0, int SR = 0>

@@ -70,8 +70,8 @@ constexpr size_t march_smem_bytes() {
 // only takes this path when an instance holds fewer than 2^31 values).
 template <typename R, int ADV, int QX2, int VY, int TY>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? (TY > 1 ? 3 : 4) : 1)))
-march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restrict__ fs,
-             const R* __restrict__ fn, R* __restrict__ fo, int stage) {
+march_kernel(const GroupDev g, const Work* __restrict__ works, const R* fs, const R* fn, R* fo, int stage) {
+    pdl_trigger();
     constexpr int S = QX2 * VY;
     constexpr int QX = QX2 / 2;
     using Buf = StepBuf<R, QX2, VY, TY>;
@@ -118,8 +118,6 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restri
         const int yy = y % ny;
         roff[r] = yy * rs;
         crow[r] = yy * nx;
-        nwl_g[r] = (R)g.nw[(size_t)(I.row_off + yy) * 2 + 0] * gwl;
-        nwr_g[r] = (R)g.nw[(size_t)(I.row_off + yy) * 2 + 1] * gwr;
     }
     const int xa = W.xa, xb = W.xb;
     const int slab = kz * S;
@@ -160,8 +158,15 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* __restri
         mbar_init_fence();
     }
     __syncthreads();
+    pdl_wait();                                  // from here on: the state, the walls, the factor lines
     if (t == 0)
         for (int xs = xa; xs < xa + kDepth - 1; ++xs) issue(xs);
+#pragma unroll
+    for (int r = 0; r < TY; ++r) {
+        const size_t yy = I.row_off + (W.y0 + r) % ny;
+        nwl_g[r] = (R)g.nw[yy * 2 + 0] * gwl;
+        nwr_g[r] = (R)g.nw[yy * 2 + 1] * gwr;
+    }
 
     // window of cells xa-3 .. xa+2 (walls: ghosts of Sec. IV.C.3) and the face xa-1/2
     R w[TY][6], Fm[TY];
@@ -314,8 +319,8 @@ namespace {
 template <typename R, int ADV, int QX2, int VY, int TY>
 void launch_one(const GroupDev& g, const Work* works, int nworks, const void* fs, const void* fn, void* fo,
                 int stage, cudaStream_t st) {
-    march_kernel<R, ADV, QX2, VY, TY><<<nworks, QX2 * VY, march_smem_bytes<R, QX2, VY, TY>(), st>>>(
-        g, works, (const R*)fs, (const R*)fn, (R*)fo, stage);
+    launch_dependent(g.pdl, march_kernel<R, ADV, QX2, VY, TY>, nworks, QX2 * VY, march_smem_bytes<R, QX2, VY, TY>(), st, g, works,
+                     (const R*)fs, (const R*)fn, (R*)fo, stage);
 }
 
 template <typename R, int ADV, int QX2, int VY, int TY>

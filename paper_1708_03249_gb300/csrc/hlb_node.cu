@@ -386,7 +386,7 @@ __host__ __device__ inline NodeSmem node_smem(const GroupDev& g) {
 // per node (rows of 4 LPN values); z: a p_z axis.  A lane adds (n, j_x), (j_y, E)
 // and j_z, two sums per packed compensated addition.
 template <int LPN>
-__device__ __forceinline__ void node_sums(const float* __restrict__ fs, const float* __restrict__ P,
+__device__ __forceinline__ void node_sums(const float* fs, const float* __restrict__ P,
                                           const float4* sYZ, const long long* sOff, float* sum, int nb, int rows, int V,
                                           bool z) {
     const int lane = threadIdx.x & 31, sl = lane % LPN;
@@ -436,10 +436,12 @@ __device__ __forceinline__ void node_sums(const float* __restrict__ fs, const fl
 }
 
 template <int ADV, int LOWN>
-__global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const GroupDev g, const float* __restrict__ fs) {
+__global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const GroupDev g, const float* fs) {
     extern __shared__ __align__(16) unsigned char nsm[];
+    pdl_trigger();
     const int nwall = g.nrows * g.wchunks;
     if ((int)blockIdx.x < nwall) {
+        pdl_wait();
         wall_block<float, ADV>(g, fs, blockIdx.x, reinterpret_cast<double*>(nsm));
         return;
     }
@@ -469,6 +471,7 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
         ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, base + tid) : 0;
         sOff[tid] = g.inst[ii].f_off + (long long)(base + tid - g.inst[ii].node_off) * V;
     }
+    pdl_wait();
     __syncthreads();
     // 1. moment sums: 2Qx / 4 lanes per node, so that a lane's p_x never change
     // and step r of its loop is the row r of (jy, kz)
@@ -575,11 +578,13 @@ __device__ __forceinline__ void half_range_coefficients(const GroupDev& g, int r
 }
 
 template <int ADV, int NB>
-__global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, const double* __restrict__ fs) {
+__global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, const double* fs) {
+    pdl_trigger();
     extern __shared__ __align__(16) double dsm[];
     constexpr int LPN = kNode64T / NB;                        // lanes per node
     const int nwall = g.nrows * g.wchunks;
     if ((int)blockIdx.x < nwall) {
+        pdl_wait();
         wall_block<double, ADV>(g, fs, blockIdx.x, dsm);
         return;
     }
@@ -601,6 +606,7 @@ __global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, co
         sRow[3 * r + 1] = pz;
         sRow[3 * r + 2] = py * py + pz * pz;
     }
+    pdl_wait();
     __syncthreads();
     // 1. moments: each lane its own p_x, weighted once per column
     {
@@ -809,11 +815,11 @@ void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st
     const size_t smem = node64_smem(g, NB);
     const double* f = static_cast<const double*>(fs);
     if (adv == HLB_WENO5_) {
-        if (NB == 1) node_f64_kernel<HLB_WENO5_, 1><<<grid, kNode64T, smem, st>>>(g, f);
-        else node_f64_kernel<HLB_WENO5_, 8><<<grid, kNode64T, smem, st>>>(g, f);
+        if (NB == 1) launch_dependent(g.pdl, node_f64_kernel<HLB_WENO5_, 1>, grid, kNode64T, smem, st, g, f);
+        else launch_dependent(g.pdl, node_f64_kernel<HLB_WENO5_, 8>, grid, kNode64T, smem, st, g, f);
     } else {
-        if (NB == 1) node_f64_kernel<HLB_UPWIND2_, 1><<<grid, kNode64T, smem, st>>>(g, f);
-        else node_f64_kernel<HLB_UPWIND2_, 8><<<grid, kNode64T, smem, st>>>(g, f);
+        if (NB == 1) launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 1>, grid, kNode64T, smem, st, g, f);
+        else launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 8>, grid, kNode64T, smem, st, g, f);
     }
 }
 
@@ -823,11 +829,11 @@ void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t 
     const float* f = static_cast<const float*>(fs);
     const bool low = node_low(g);
     if (adv == HLB_WENO5_) {
-        if (low) node_df_kernel<HLB_WENO5_, 1><<<grid, kNodeT, smem, st>>>(g, f);
-        else node_df_kernel<HLB_WENO5_, 0><<<grid, kNodeT, smem, st>>>(g, f);
+        if (low) launch_dependent(g.pdl, node_df_kernel<HLB_WENO5_, 1>, grid, kNodeT, smem, st, g, f);
+        else launch_dependent(g.pdl, node_df_kernel<HLB_WENO5_, 0>, grid, kNodeT, smem, st, g, f);
     } else {
-        if (low) node_df_kernel<HLB_UPWIND2_, 1><<<grid, kNodeT, smem, st>>>(g, f);
-        else node_df_kernel<HLB_UPWIND2_, 0><<<grid, kNodeT, smem, st>>>(g, f);
+        if (low) launch_dependent(g.pdl, node_df_kernel<HLB_UPWIND2_, 1>, grid, kNodeT, smem, st, g, f);
+        else launch_dependent(g.pdl, node_df_kernel<HLB_UPWIND2_, 0>, grid, kNodeT, smem, st, g, f);
     }
 }
 

@@ -62,8 +62,9 @@ constexpr size_t pair_smem_bytes() {
 // rounded stochastically (rk3_out_sr2, hlb_device.cuh).
 template <int ADV, int QX2, int VY, int FM, int FF, int SR = 0>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? HLB_PAIR_MIN_BLOCKS : 2)))
-march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float* __restrict__ fs,
-                  const float* __restrict__ fn, float* __restrict__ fo, int stage) {
+march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs, const float* fn, float* fo,
+                  int stage) {
+    pdl_trigger();
     constexpr int S = QX2 * VY;
     constexpr int QX = QX2 / 2;
     constexpr int SP = QX2 + 1;            // padded sF row: the K_x reads of a warp hit distinct banks
@@ -144,8 +145,6 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         const int yy = y % ny;
         roff[r] = yy * rs;
         crow[r] = yy * nx;
-        nwl_g[r] = (float)g.nw[(size_t)(I.row_off + yy) * 2 + 0] * gwl;
-        nwr_g[r] = (float)g.nw[(size_t)(I.row_off + yy) * 2 + 1] * gwr;
     }
     const int xa = W.xa, xb = W.xb;
     const int npairs = (xb - xa + 1) >> 1;
@@ -239,7 +238,14 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
         for (int p = 0; p < kPairDepth - 1; ++p) expect(p);
     }
     __syncthreads();
+    pdl_wait();                        // from here on: the state, the walls, the factor lines
     for (int p = 0; p < kPairDepth - 1; ++p) issue(p);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const size_t yy = I.row_off + (W.y0 + r) % ny;
+        nwl_g[r] = (float)g.nw[yy * 2 + 0] * gwl;
+        nwr_g[r] = (float)g.nw[yy * 2 + 1] * gwr;
+    }
 
     // scaled window of cells xa-3 .. xa+4 (wall ghosts of Sec. IV.C.3); w[0..5] filled here
     float2 w[8];
@@ -435,8 +441,8 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
 template <int ADV, int QX2, int VY, int FM, int FF = 0, int SR = 0>
 void launch_pair_t(const GroupDev& g, const Work* works, int nworks, const void* fs, const void* fn, void* fo,
                    int stage, cudaStream_t st) {
-    march_pair_kernel<ADV, QX2, VY, FM, FF, SR><<<nworks, QX2 * VY, pair_smem_bytes<QX2, VY, FM>(), st>>>(
-        g, works, (const float*)fs, (const float*)fn, (float*)fo, stage);
+    launch_dependent(g.pdl, march_pair_kernel<ADV, QX2, VY, FM, FF, SR>, nworks, QX2 * VY, pair_smem_bytes<QX2, VY, FM>(), st, g,
+                     works, (const float*)fs, (const float*)fn, (float*)fo, stage);
 }
 
 template <int ADV, int QX2, int VY, int FM, int FF = 0, int SR = 0>

@@ -13,7 +13,7 @@ namespace hlb {
 
 // Block `block` of g.nrows g.wchunks; red: shared memory for two doubles per warp.
 template <typename R, int ADV>
-__device__ __forceinline__ void wall_block(const GroupDev& g, const R* __restrict__ fs, int block, double* red) {
+__device__ __forceinline__ void wall_block(const GroupDev& g, const R* fs, int block, double* red) {
     const int nw = (blockDim.x + 31) >> 5;
     const int row = block / g.wchunks, chunk = block - row * g.wchunks;
     if (row >= g.nrows) return;
