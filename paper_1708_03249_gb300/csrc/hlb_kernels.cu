@@ -609,8 +609,9 @@ wall_kernel(const GroupDev g, const R* __restrict__ fs) {
 // operations per point and order, but leave half the SMs idle), 128 threads of
 // three points each, their sums over the CTA through shared memory (the FP64
 // adds of a full-warp butterfly for every order cost as much as the points).
-// 72 nodes at order 20: 28 us per stage, 44 with one CTA of 256 threads per node
-// and butterflies (GB300).
+// 72 nodes at order 20: 25 us per stage, 44 with one CTA of 256 threads per node
+// and butterflies (GB300; 28 with a division per moment and the products by p_y and
+// p_z of the absent axes).
 // ---------------------------------------------------------------------------
 constexpr int kQuadThreads = 128;
 template <int NMAX>
@@ -627,25 +628,31 @@ __global__ void __launch_bounds__(kQuadThreads) quad_coef_kernel(const GroupDev 
     const double* f = fs + I.f_off + (size_t)(node - I.node_off) * V;
     // moments of the node
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
+#pragma unroll 4
     for (int v = tid; v < V; v += kQuadThreads) {
         const double val = f[v];
-        const double px = g.pd[v % QX2], py = g.pd[QX2 + (v / QX2) % VY], pz = g.pd[QX2 + VY + v / (QX2 * VY)];
+        const double px = g.pd[v % QX2], pv = px * val;
         a0 += val;
-        a1 += px * val;
-        a2 += py * val;
-        a3 += pz * val;
-        a4 += (px * px + py * py + pz * pz) * val;
+        a1 += pv;
+        a4 = fma(px, pv, a4);
+        if (V > QX2) {                          // p_y, p_z
+            const double py = g.pd[QX2 + (v / QX2) % VY], pz = g.pd[QX2 + VY + v / (QX2 * VY)];
+            a2 = fma(py, val, a2);
+            a3 = fma(pz, val, a3);
+            a4 = fma(fma(py, py, pz * pz), val, a4);
+        }
     }
-    a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3); a4 = warp_sum(a4);
+    a0 = warp_sum(a0); a1 = warp_sum(a1); a4 = warp_sum(a4);
+    if (V > QX2) { a2 = warp_sum(a2); a3 = warp_sum(a3); }
     if (lane == 0) { red[warp][0] = a0; red[warp][1] = a1; red[warp][2] = a2; red[warp][3] = a3; red[warp][4] = a4; }
     __syncthreads();
     if (tid == 0) {
         double m[5] = {0, 0, 0, 0, 0};
         for (int w = 0; w < nw; ++w)
             for (int k = 0; k < 5; ++k) m[k] += red[w][k];
-        const double n = m[0], ux = m[1] / n, uy = m[2] / n, uz = m[3] / n;
+        const double n = m[0], in = 1.0 / n, ux = m[1] * in, uy = m[2] * in, uz = m[3] * in;
         sMom[0] = ux;
-        sMom[1] = (m[4] - n * (ux * ux + uy * uy + uz * uz)) / (g.D * n);
+        sMom[1] = (m[4] - n * (ux * ux + uy * uy + uz * uz)) * in * (g.D == 3 ? 1.0 / 3.0 : (g.D == 2 ? 0.5 : 1.0));
     }
     __syncthreads();
     const double ux = sMom[0], T = sMom[1];

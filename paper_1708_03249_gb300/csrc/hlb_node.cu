@@ -723,13 +723,18 @@ __global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, co
             if (absent) {
                 v = 1.0;
             } else {
+                // eight table entries (global memory, one row per thread) at a time
                 double a0 = 0.0, a1 = 0.0;
-                int l = 0;
-                for (; l < N; l += 2) {
-                    a0 = fma(T[l], G[l], a0);
-                    a1 = fma(T[l + 1], G[l + 1], a1);
+                for (int l = 0; l <= N; l += 8) {
+                    double t[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) t[c] = l + c <= N ? T[l + c] : 0.0;
+#pragma unroll
+                    for (int c = 0; c < 8; c += 2) {
+                        if (l + c <= N) a0 = fma(t[c], G[l + c], a0);
+                        if (l + c + 1 <= N) a1 = fma(t[c + 1], G[l + c + 1], a1);
+                    }
                 }
-                if (l == N) a0 = fma(T[l], G[l], a0);
                 v = a0 + a1;
                 if (o < QX2) v *= m[0];
             }
