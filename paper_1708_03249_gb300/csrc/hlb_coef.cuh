@@ -302,8 +302,8 @@ __device__ inline double node_inputs_from_sums_df(const float* sm, int D, NodeDF
 // 15 of the 256^2 box, where the instructions alone take about 20).  Here thread
 // t works on node t % NB, and every double-float operation on two values in
 // the lanes of f32x2 registers:
-//  - recurrences: G^+ with G^- (slot 0), G_y with G_z (slot 1), a thread per
-//    node and pair; the coefficients go to shared memory;
+//  - recurrences: G^+ with G^- (slot 0), G_y with G_z (a slot of the next warp), a
+//    thread per node and pair; the coefficients go to shared memory;
 //  - dot products (Dot2 of Ogita, Rump and Oishi, as in dot2_pair), items of two
 //    rows over all threads of the node: n g_x of +z_k with that of -z_k (one
 //    table entry for both lanes); along p_y and p_z the even orders in one lane
@@ -461,7 +461,7 @@ __device__ __forceinline__ void node_lines(const GroupDev& g, const NodeTables& 
                 put(l + 1, cur);
             }
         }
-    } else if (active && slot == 1 % SLOTS) {
+    } else if (active && slot == (NB < 32 ? 32 / NB : 1)) {     // in another warp than slot 0
         // G_l(u_y) with G_l(u_z); an order past an axis's last is a zero
         const float2 ua = in(1), ub = in(2);
         float* fy = reinterpret_cast<float*>(Gy);

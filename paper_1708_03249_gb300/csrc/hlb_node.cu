@@ -363,11 +363,12 @@ __global__ void __launch_bounds__(128) coef_df_kernel(const GroupDev g, const fl
 // box), and a resident grid that loops over the batches runs its CTAs in step,
 // all streaming or all computing (0.93 ms for the large channel).
 // ---------------------------------------------------------------------------
-constexpr int kNodeNB = 32, kNodeT = 128;
+constexpr int kNodeT = 128;
 
 struct NodeSmem {                        // byte offsets
     size_t tab, yz, rec, in, G, line, bytes;
 };
+template <int NB>
 __host__ __device__ inline NodeSmem node_smem(const GroupDev& g) {
     const NodeTables nt(g);
     NodeSmem L;
@@ -375,9 +376,9 @@ __host__ __device__ inline NodeSmem node_smem(const GroupDev& g) {
     L.yz = L.tab + nt.table_bytes();
     L.rec = L.yz + (size_t)g.VY * g.VZ * 16;
     L.in = L.rec + node_rec_bytes(g.Nx);
-    L.G = L.in + (size_t)kNodeNB * kNodeFields * 8;
-    L.line = L.G + nt.coef_bytes<kNodeNB>(g);            // the moment sums, then the lines
-    const size_t lines = (size_t)kNodeNB * node_line_stride(g.ncp) * 4, sums = (size_t)kNodeNB * kSumStride * 4;
+    L.G = L.in + (size_t)NB * kNodeFields * 8;
+    L.line = L.G + nt.coef_bytes<NB>(g);            // the moment sums, then the lines
+    const size_t lines = (size_t)NB * node_line_stride(g.ncp) * 4, sums = (size_t)NB * kSumStride * 4;
     L.bytes = L.line + (lines > sums ? lines : sums);
     return L;
 }
@@ -435,7 +436,7 @@ __device__ __forceinline__ void node_sums(const float* fs, const float* __restri
     }
 }
 
-template <int ADV, int LOWN>
+template <int ADV, int LOWN, int NB>
 __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const GroupDev g, const float* fs) {
     extern __shared__ __align__(16) unsigned char nsm[];
     pdl_trigger();
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
         wall_block<float, ADV>(g, fs, blockIdx.x, reinterpret_cast<double*>(nsm));
         return;
     }
-    const NodeSmem L = node_smem(g);
+    const NodeSmem L = node_smem<NB>(g);
     float4* tab = reinterpret_cast<float4*>(nsm + L.tab);
     float4* sYZ = reinterpret_cast<float4*>(nsm + L.yz);
     float4* rec = reinterpret_cast<float4*>(nsm + L.rec);
@@ -463,9 +464,9 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
     }
     node_load_rec(g, rec, tid, kNodeT);
     node_load_tables(g, nt, tab, tid, kNodeT);
-    const int base = ((int)blockIdx.x - nwall) * kNodeNB;
-    const int nb = min(kNodeNB, g.nnodes - base);
-    __shared__ long long sOff[kNodeNB];      // each node's values in the state
+    const int base = ((int)blockIdx.x - nwall) * NB;
+    const int nb = min(NB, g.nnodes - base);
+    __shared__ long long sOff[NB];      // each node's values in the state
     int ii = 0;
     if (tid < nb) {
         ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, base + tid) : 0;
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
     else node_sums<2>(fs, P, sYZ, sOff, sSum, nb, VY * VZ, V, VZ > 1);
     __syncthreads();
     // 2. n, u, T, 1/tau and what starts the recurrences, one thread per node
-    if (tid < kNodeNB) {
+    if (tid < NB) {
         NodeDF in;
         double itau = 0.0;
         if (tid < nb) {
@@ -490,14 +491,14 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
         }
         const float2 v[kNodeFields] = {in.ux, in.uy, in.uz, in.T, in.Tm1, in.erf_z, in.g0, in.n, make_float2((float)itau, 0.0f)};
 #pragma unroll
-        for (int f = 0; f < kNodeFields; ++f) sIn[f * kNodeNB + tid] = v[f];
+        for (int f = 0; f < kNodeFields; ++f) sIn[f * NB + tid] = v[f];
     }
     __syncthreads();
-    node_lines<kNodeNB, kNodeT>(g, nt, sIn, sG, sLine, tab, rec);
+    node_lines<NB, kNodeT>(g, nt, sIn, sG, sLine, tab, rec);
     if (tid < nb) {                                      // the lines' tails: 1/tau, the field's accelerations
         float* line = sLine + tid * node_line_stride(g.ncp);
         const int t0 = QX2 + VY + VZ;
-        line[t0] = sIn[8 * kNodeNB + tid].x;
+        line[t0] = sIn[8 * NB + tid].x;
         for (int o = t0 + 1; o < g.ncp; ++o) line[o] = 0.0f;
         if (g.has_field) {                           // a = a_uniform + a_field(node)
             const InstDev& I = g.inst[ii];
@@ -758,12 +759,14 @@ cudaError_t prepare_node() {
 }
 
 static int sm_count() {
-    static int nsm = 0;
-    if (!nsm) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            nsm = 152;
-    }
+    static const int nsm = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            n = 152;
+        }
+        return n;
+    }();
     return nsm;
 }
 
@@ -800,17 +803,42 @@ bool node_fused_available(int precision, const GroupDev& g) {
     return precision != HLB_FP64_ && g.use_df && max(g.Nx, max(g.Ny, g.Nz)) < 16 && (g.QX2 == 8 || g.QX2 == 16 || g.QX2 == 32);
 }
 
-static bool node_low(const GroupDev& g) { return g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12; }
+// Nodes per CTA of the one-launch node pass.  With rows of 32 values (the longest
+// recurrences and dot products) a group of up to 64 nodes per SM waits on the
+// chain of one CTA, and at 8 nodes the dot products take one turn of the CTA
+// instead of three; else 32.  us per step of order-16 channels (GB300), 8
+// against 32: 64 nodes 44.5 / 55.9, 1216 nodes 56 / 79, 4864 105 / 107, 9728
+// 171 / 183, 19456 379 / 347; order 8: 1216 nodes 38.5 / 36.8, 4864 46.5 / 45.2.
+static int node_nb(const GroupDev& g) { return g.QX2 == 32 && g.nnodes <= 64 * sm_count() ? 8 : 32; }
 
-// Needed only above the 48 KB that a launch has without asking (setting an
-// attribute loads the kernel, which a handle's creation would wait for).
-cudaError_t prepare_node_fused(int adv, const GroupDev& g) {
-    const size_t smem = node_smem(g).bytes;
-    if (smem <= 48 * 1024) return cudaSuccess;
-    const bool low = node_low(g);
-    const void* f = adv == HLB_WENO5_ ? (low ? (const void*)node_df_kernel<HLB_WENO5_, 1> : (const void*)node_df_kernel<HLB_WENO5_, 0>)
-                                      : (low ? (const void*)node_df_kernel<HLB_UPWIND2_, 1> : (const void*)node_df_kernel<HLB_UPWIND2_, 0>);
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int ADV, int LOWN>
+static cudaError_t node_df_launch(const GroupDev& g, const float* fs, cudaStream_t st, bool prepare) {
+    const int NB = node_nb(g);
+    const size_t smem = NB == 8 ? node_smem<8>(g).bytes : node_smem<32>(g).bytes;
+    if (prepare) {
+        // needed only above the 48 KB that a launch has without asking (setting
+        // an attribute loads the kernel, which a handle's creation would wait for)
+        if (smem <= 48 * 1024) return cudaSuccess;
+        return cudaFuncSetAttribute(NB == 8 ? (const void*)node_df_kernel<ADV, LOWN, 8> : (const void*)node_df_kernel<ADV, LOWN, 32>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
+    const int grid = g.nrows * g.wchunks + (g.nnodes + NB - 1) / NB;
+    if (NB == 8) launch_dependent(g.pdl, node_df_kernel<ADV, LOWN, 8>, grid, kNodeT, smem, st, g, fs);
+    else launch_dependent(g.pdl, node_df_kernel<ADV, LOWN, 32>, grid, kNodeT, smem, st, g, fs);
+    return cudaSuccess;
+}
+
+static cudaError_t node_df_dispatch(int adv, const GroupDev& g, const float* fs, cudaStream_t st, bool prepare) {
+    const bool low = g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12;
+    if (adv == HLB_WENO5_)
+        return low ? node_df_launch<HLB_WENO5_, 1>(g, fs, st, prepare) : node_df_launch<HLB_WENO5_, 0>(g, fs, st, prepare);
+    return low ? node_df_launch<HLB_UPWIND2_, 1>(g, fs, st, prepare) : node_df_launch<HLB_UPWIND2_, 0>(g, fs, st, prepare);
+}
+
+cudaError_t prepare_node_fused(int adv, const GroupDev& g) { return node_df_dispatch(adv, g, nullptr, nullptr, true); }
+
+void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
+    node_df_dispatch(adv, g, static_cast<const float*>(fs), st, false);
 }
 
 // The FP64 node pass and walls (every FP64 group).
@@ -825,20 +853,6 @@ void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st
     } else {
         if (NB == 1) launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 1>, grid, kNode64T, smem, st, g, f);
         else launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 8>, grid, kNode64T, smem, st, g, f);
-    }
-}
-
-void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
-    const int grid = g.nrows * g.wchunks + (g.nnodes + kNodeNB - 1) / kNodeNB;
-    const size_t smem = node_smem(g).bytes;
-    const float* f = static_cast<const float*>(fs);
-    const bool low = node_low(g);
-    if (adv == HLB_WENO5_) {
-        if (low) launch_dependent(g.pdl, node_df_kernel<HLB_WENO5_, 1>, grid, kNodeT, smem, st, g, f);
-        else launch_dependent(g.pdl, node_df_kernel<HLB_WENO5_, 0>, grid, kNodeT, smem, st, g, f);
-    } else {
-        if (low) launch_dependent(g.pdl, node_df_kernel<HLB_UPWIND2_, 1>, grid, kNodeT, smem, st, g, f);
-        else launch_dependent(g.pdl, node_df_kernel<HLB_UPWIND2_, 0>, grid, kNodeT, smem, st, g, f);
     }
 }
 

@@ -1,5 +1,5 @@
 """The one-launch node pass of FP32 groups (moment sums, factor lines and walls)
-against the oracle, at the sizes where its batches of 32 nodes, its rows and
+against the oracle, at the sizes where its batches of 8 or 32 nodes (8 for rows of 32 and at most 9728 nodes), its rows and
 its orders end: ragged and single batches, each row length (2 Qx = 8, 16, 32),
 absent axes, a collisionless instance among others, and flows fast enough to
 leave the polynomial range of exp and erf (|u_x| / sqrt(2T) > 0.7).  The
@@ -23,6 +23,8 @@ CASES = {
     "1d_full_range": (W.make(Qx=16, Qy=8, nx=40, x_basis=W.X_FULL, ay=-0.2, **_PHYS), 3),
     "2d_q4_1025_nodes": (W.make(Qx=4, Qy=4, nx=41, ny=25, Ly=0.6, ay=-0.2, advection=W.UPWIND2, **_PHYS), 2),
     "2d_q4_z": (W.make(Qx=4, Qy=4, Qz=4, nx=40, ny=27, Ly=0.6, ay=-0.2, **_PHYS), 1),
+    "2d_q4_5041_nodes": (W.make(Qx=4, Qy=4, nx=71, ny=71, Ly=0.6, ay=-0.2, **_PHYS), 1),
+    "1d_q16_9789_nodes": ([W.make(Qx=16, Qy=4, nx=nx, **_PHYS) for nx in (4903, 7, 4879)], 1),
     "mixed_with_collisionless": ([W.make(Qx=4, Qy=4, nx=nx, precision=W.FP32, Kn=Kn, T_right=1.3, ax=-0.2)
                                   for nx, Kn in ((19, 0.1), (45, math.inf), (7, 1.0))], 4),
 }
