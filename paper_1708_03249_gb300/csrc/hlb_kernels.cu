@@ -415,29 +415,42 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
 // node's end (400 velocities are 12.5 warps; in seven CTAs of 64 per node they
 // took 14 and 4.4 rounds of the resident CTAs, here 12.5 and 2).  Per stage
 // (GB300): eight ballistic cases 43.6 us against 63.9 in the generic kernel.
+//   A group of few cells leaves SM quarters idle that way (one transition-regime
+// run of 72 cells: 450 warps for 608 quarters), and is spread at one cell per
+// thread (NC = 1).
 constexpr int kWideThreads = 64;
-template <int ADV>
+template <int NC>
+struct alignas(8 * NC) CellVals {            // one population's values at a thread's cells
+    double c[NC];
+};
+template <int ADV, int NC>
 __global__ void __launch_bounds__(kWideThreads, 4)
 stage_wide_kernel(const GroupDev g, const double* __restrict__ fs, const double* __restrict__ fn,
                   double* __restrict__ fo, int stage) {
     extern __shared__ __align__(16) unsigned char wsm[];
     const int V = g.V, QX2 = g.QX2, Qx = g.Qx, VY = g.VY, VZ = g.VZ, nfib = VY * VZ;
-    double2* sF = reinterpret_cast<double2*>(wsm);                   // [2 fibres][QX2]: (cell x0, cell x0 + 1)
-    double2* sJ = sF + 2 * QX2;                                      // [2 fibres][2 halves]: sum_{k' in half} d_k' f_k'
+    CellVals<NC>* sF = reinterpret_cast<CellVals<NC>*>(wsm);         // [2 fibres][QX2]
+    CellVals<NC>* sJ = sF + 2 * QX2;                                      // [2 fibres][2 halves]: sum_{k' in half} d_k' f_k'
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long total = (long long)g.npairs * V;
+    const int* start = NC == 2 ? g.pair_start : g.node_start;        // cell pairs or cells before each instance
+    const long long total = (long long)(NC == 2 ? g.npairs : g.nnodes) * V;
     const long long e0 = (long long)blockIdx.x * kWideThreads;
     const long long fib0 = e0 / QX2;                                 // first fibre of the CTA, over all pairs
     const long long last = min(total, e0 + kWideThreads) - 1;
     const int nfb = (int)(last / QX2 - fib0) + 1;                    // one or two (QX2 > 64)
     for (int a = 0; a < nfb; ++a) {
         const int pair = (int)((fib0 + a) / nfib), fb = (int)((fib0 + a) - (long long)pair * nfib);
-        const int ii = g.ninst > 1 ? find_slot(g.pair_start, g.ninst, pair) : 0;
+        const int ii = g.ninst > 1 ? find_slot(start, g.ninst, pair) : 0;
         const InstDev& I = g.inst[ii];
-        const int x0 = 2 * (pair - g.pair_start[ii]);
+        const int x0 = NC * (pair - start[ii]);
         const double* f = fs + I.f_off + (size_t)x0 * V + (size_t)fb * QX2;
-        const bool two = x0 + 1 < I.nx;
-        for (int i = tid; i < QX2; i += kWideThreads) sF[a * QX2 + i] = make_double2(f[i], two ? f[V + i] : 0.0);
+        const bool two = NC == 2 && x0 + 1 < I.nx;
+        for (int i = tid; i < QX2; i += kWideThreads) {
+            CellVals<NC> val;
+            val.c[0] = f[i];
+            if (NC == 2) val.c[NC - 1] = two ? f[V + i] : 0.0;
+            sF[a * QX2 + i] = val;
+        }
     }
     __syncthreads();
     {
@@ -448,16 +461,16 @@ stage_wide_kernel(const GroupDev g, const double* __restrict__ fs, const double*
             const int a = j >> 1, h = j & 1;
             const long long b = (fib0 + a) * QX2 + (h ? 0 : Qx);     // the other half's values
             if (b > last || b + Qx <= e0) continue;
-            double s0 = 0.0, s1 = 0.0;
+            CellVals<NC> s = {};
             for (int i = lane; i < Qx; i += 32) {
                 const double d = jd[h * Qx + i];
-                const double2 f = sF[a * QX2 + h * Qx + i];
-                s0 = fma(d, f.x, s0);
-                s1 = fma(d, f.y, s1);
+                const CellVals<NC> f = sF[a * QX2 + h * Qx + i];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) s.c[c] = fma(d, f.c[c], s.c[c]);
             }
-            s0 = warp_sum(s0);
-            s1 = warp_sum(s1);
-            if (lane == 0) sJ[j] = make_double2(s0, s1);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s.c[c] = warp_sum(s.c[c]);
+            if (lane == 0) sJ[j] = s;
         }
     }
     __syncthreads();
@@ -466,52 +479,53 @@ stage_wide_kernel(const GroupDev g, const double* __restrict__ fs, const double*
     const int a = (int)(e / QX2 - fib0), ix = (int)(e % QX2);
     const int pair = (int)(e / V), v = (int)(e - (long long)pair * V);
     const int jy = (v / QX2) % VY, kz = v / (QX2 * VY);
-    const int ii = g.ninst > 1 ? find_slot(g.pair_start, g.ninst, pair) : 0;
+    const int ii = g.ninst > 1 ? find_slot(start, g.ninst, pair) : 0;
     const InstDev& I = g.inst[ii];
-    const int nx = I.nx, x0 = 2 * (pair - g.pair_start[ii]);
-    const bool two = x0 + 1 < nx, xpos = ix < Qx;
+    const int nx = I.nx, x0 = NC * (pair - start[ii]);
+    const bool two = NC == 2 && x0 + 1 < nx, xpos = ix < Qx;
     const double* frow = fs + I.f_off;
-    // fluxes per unit velocity at x0 - 1/2, x0 + 1/2, x0 + 3/2
-    double Fx[3];
+    // fluxes per unit velocity at x0 - 1/2, x0 + 1/2 (and x0 + 3/2)
+    constexpr int NF = NC + 1;
+    double Fx[NF];
     {
         const double* gw = static_cast<const double*>(g.gw) + I.gw_off;
         const double nwl_g = g.nw[(size_t)I.row_off * 2 + 0] * gw[v], nwr_g = g.nw[(size_t)I.row_off * 2 + 1] * gw[V + v];
-        double w[7];
+        double w[NF + 4];
         const int base = xpos ? x0 - 3 : x0 - 2;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) w[k] = x_value(frow, base + k, nx, V, v, xpos, nwl_g, nwr_g);
+        for (int k = 0; k < NF + 4; ++k) w[k] = x_value(frow, base + k, nx, V, v, xpos, nwl_g, nwr_g);
         if (ADV == HLB_WENO5_) {
-            double u[7], F[3];
+            double u[NF + 4], F[NF];
 #pragma unroll
-            for (int k = 0; k < 7; ++k) u[k] = xpos ? w[k] : w[6 - k];
-            weno5_faces64<3>(u, F);
+            for (int k = 0; k < NF + 4; ++k) u[k] = xpos ? w[k] : w[NF + 3 - k];
+            weno5_faces64<NF>(u, F);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) Fx[k] = xpos ? F[k] : F[2 - k];
+            for (int k = 0; k < NF; ++k) Fx[k] = xpos ? F[k] : F[NF - 1 - k];
         } else {
 #pragma unroll
-            for (int k = 0; k < 3; ++k)
+            for (int k = 0; k < NF; ++k)
                 Fx[k] = xpos ? upwind2_face(w[k + 1], w[k + 2]) : upwind2_face(w[k + 3], w[k + 2]);
         }
     }
-    // a_x K_x f + a_y K_y f + a_z K_z f at both cells
+    // a_x K_x f + a_y K_y f + a_z K_z f at the cells (accelerations; at the last cell c1 too)
     const int node0 = I.node_off + x0;
-    double force[2] = {0.0, 0.0}, acc3[3][2];
-    acc3[0][0] = acc3[0][1] = acc3[1][0] = acc3[1][1] = acc3[2][0] = acc3[2][1] = 0.0;
-    double acl[2][3];
+    constexpr int c1 = NC - 1;
+    double acc3[3][NC] = {};
+    double acl[NC][3];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < NC; ++c) {
         const double* af = g.has_field && (c == 0 || two) ? g.afield + 3 * (size_t)(node0 + c) : nullptr;
         acl[c][0] = I.ax + (af ? af[0] : 0.0);
         acl[c][1] = I.ay + (af ? af[1] : 0.0);
         acl[c][2] = I.az + (af ? af[2] : 0.0);
     }
-    if (acl[0][0] != 0.0 || acl[1][0] != 0.0) {
+    if (acl[0][0] != 0.0 || acl[c1][0] != 0.0) {
         // own half: column ix of Kx^T (consecutive threads read consecutive
         // entries), eight entries ahead of the sums; other half: c_ix times its sum
         const int h = xpos ? 0 : 1;
         const double* Kc = g.KxT + (size_t)h * Qx * QX2 + ix;
-        const double2* fh = sF + a * QX2 + h * Qx;
-        double p0 = 0.0, p1 = 0.0, q0 = 0.0, q1 = 0.0;
+        const CellVals<NC>* fh = sF + a * QX2 + h * Qx;
+        double p[NC][2] = {};
         constexpr int U = 8;
         double kc[U];
         const int n8 = Qx / U * U;
@@ -523,54 +537,52 @@ stage_wide_kernel(const GroupDev g, const double* __restrict__ fs, const double*
 #pragma unroll
             for (int j = 0; j < U; ++j) kn[j] = more ? Kc[(size_t)(i + U + j) * QX2] : 0.0;
 #pragma unroll
-            for (int j = 0; j < U; j += 2) {
-                const double2 f0 = fh[i + j], f1 = fh[i + j + 1];
-                p0 = fma(kc[j], f0.x, p0);
-                q0 = fma(kc[j], f0.y, q0);
-                p1 = fma(kc[j + 1], f1.x, p1);
-                q1 = fma(kc[j + 1], f1.y, q1);
+            for (int j = 0; j < U; ++j) {
+                const CellVals<NC> f0 = fh[i + j];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) p[c][j & 1] = fma(kc[j], f0.c[c], p[c][j & 1]);
             }
 #pragma unroll
             for (int j = 0; j < U; ++j) kc[j] = kn[j];
         }
         for (int i = n8; i < Qx; ++i) {
             const double k = Kc[(size_t)i * QX2];
-            const double2 f0 = fh[i];
-            p0 = fma(k, f0.x, p0);
-            q0 = fma(k, f0.y, q0);
+            const CellVals<NC> f0 = fh[i];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) p[c][0] = fma(k, f0.c[c], p[c][0]);
         }
-        const double2 J = sJ[2 * a + 1 - h];
-        const double c = g.KxJ[ix];
-        acc3[0][0] = fma(c, J.x, p0 + p1);
-        acc3[0][1] = fma(c, J.y, q0 + q1);
+        const CellVals<NC> J = sJ[2 * a + 1 - h];
+        const double cj = g.KxJ[ix];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc3[0][c] = fma(cj, J.c[c], p[c][0] + p[c][1]);
     }
     const double* f0p = frow + (size_t)x0 * V;
     const double* Ky = static_cast<const double*>(g.K) + (size_t)QX2 * QX2;
-    if (g.Qy && (acl[0][1] != 0.0 || acl[1][1] != 0.0))
+    if (g.Qy && (acl[0][1] != 0.0 || acl[c1][1] != 0.0))
         for (int j = 0; j < VY; ++j) {
             const double k = Ky[jy * VY + j];
             const size_t o = (size_t)(kz * VY + j) * QX2 + ix;
             acc3[1][0] = fma(k, f0p[o], acc3[1][0]);
-            if (two) acc3[1][1] = fma(k, f0p[V + o], acc3[1][1]);
+            if (two) acc3[1][c1] = fma(k, f0p[V + o], acc3[1][c1]);
         }
-    if (g.Qz && (acl[0][2] != 0.0 || acl[1][2] != 0.0))
+    if (g.Qz && (acl[0][2] != 0.0 || acl[c1][2] != 0.0))
         for (int j = 0; j < VZ; ++j) {
             const double k = Ky[VY * VY + kz * VZ + j];
             const size_t o = (size_t)(j * VY + jy) * QX2 + ix;
             acc3[2][0] = fma(k, f0p[o], acc3[2][0]);
-            if (two) acc3[2][1] = fma(k, f0p[V + o], acc3[2][1]);
+            if (two) acc3[2][c1] = fma(k, f0p[V + o], acc3[2][c1]);
         }
     const double vx = g.pd[ix], dt = I.dt;
     const double* idx = static_cast<const double*>(g.inv_dx) + I.dx_off + x0;
-    const double2 fc = sF[a * QX2 + ix];
+    const CellVals<NC> fc = sF[a * QX2 + ix];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; c < NC; ++c) {
         if (c == 1 && !two) break;
-        force[c] = acl[c][0] * acc3[0][c];
-        if (g.Qy) force[c] = fma(acl[c][1], acc3[1][c], force[c]);
-        if (g.Qz) force[c] = fma(acl[c][2], acc3[2][c], force[c]);
-        const double f = c ? fc.y : fc.x;
-        double L = -vx * (Fx[c + 1] - Fx[c]) * idx[c] - force[c];
+        double force = acl[c][0] * acc3[0][c];
+        if (g.Qy) force = fma(acl[c][1], acc3[1][c], force);
+        if (g.Qz) force = fma(acl[c][2], acc3[2][c], force);
+        const double f = fc.c[c];
+        double L = -vx * (Fx[c + 1] - Fx[c]) * idx[c] - force;
         if (I.inv_Kn != 0.0) {
             const double* line = static_cast<const double*>(g.coef) + (size_t)(node0 + c) * g.ncp;
             L -= (f - line[ix] * line[QX2 + jy] * line[QX2 + VY + kz]) * line[QX2 + VY + VZ];
@@ -1088,12 +1100,24 @@ void launch_stage(int precision, int adv, const GroupDev& g, const void* fs, con
     }
 }
 
+template <int ADV>
+static void stage_wide_launch(const GroupDev& g, const double* fs, const double* fn, double* fo, int stage, cudaStream_t st) {
+    const long long pairs = (long long)g.npairs * g.V, cells = (long long)g.nnodes * g.V;
+    // Two cells per thread once their CTAs give every SM two (each quarter a
+    // warp); below, one.  us per step, one cell against two (GB300): 72 cells of 400
+    // velocities 209 / 228, 144 279 / 275, 288 479 / 437, 576 930 / 898.
+    if (pairs <= 2LL * sm_count() * kWideThreads) {
+        const int grid = (int)((cells + kWideThreads - 1) / kWideThreads);
+        stage_wide_kernel<ADV, 1><<<grid, kWideThreads, (2 * (size_t)g.QX2 + 4) * sizeof(CellVals<1>), st>>>(g, fs, fn, fo, stage);
+    } else {
+        const int grid = (int)((pairs + kWideThreads - 1) / kWideThreads);
+        stage_wide_kernel<ADV, 2><<<grid, kWideThreads, (2 * (size_t)g.QX2 + 4) * sizeof(CellVals<2>), st>>>(g, fs, fn, fo, stage);
+    }
+}
+
 void launch_stage_wide(int adv, const GroupDev& g, const void* fs, const void* fn, void* fo, int stage, cudaStream_t st) {
-    const long long total = (long long)g.npairs * g.V;
-    const int grid = (int)((total + kWideThreads - 1) / kWideThreads);
-    const size_t smem = (2 * (size_t)g.QX2 + 4) * sizeof(double2);
-    if (adv == HLB_WENO5_) stage_wide_kernel<HLB_WENO5_><<<grid, kWideThreads, smem, st>>>(g, (const double*)fs, (const double*)fn, (double*)fo, stage);
-    else stage_wide_kernel<HLB_UPWIND2_><<<grid, kWideThreads, smem, st>>>(g, (const double*)fs, (const double*)fn, (double*)fo, stage);
+    if (adv == HLB_WENO5_) stage_wide_launch<HLB_WENO5_>(g, (const double*)fs, (const double*)fn, (double*)fo, stage, st);
+    else stage_wide_launch<HLB_UPWIND2_>(g, (const double*)fs, (const double*)fn, (double*)fo, stage, st);
 }
 
 void launch_quad_coef(const GroupDev& g, const void* fs, cudaStream_t st) {

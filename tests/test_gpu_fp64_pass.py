@@ -79,6 +79,13 @@ def test_wide_stage_kernel(name, cfg):
     _check_fp64(got, refs, 1e-9)
 
 
+def test_wide_stage_kernel_two_cells_per_thread():
+    # more than 19456 (pair, velocity) items: odd cells, a CTA that straddles instances
+    cfg = [W.make(Qx=200, Nx_eq=12, nx=nx, Kn=Kn, **_WIDE) for nx, Kn in ((49, 0.3), (51, math.inf))]
+    got, mom, N, refs = run_pair(cfg, 2)
+    _check_fp64(got, refs, 1e-9)
+
+
 def test_wide_stage_kernel_field():
     from oracle.solver import Solver, config_from
     from paper_1708_03249_gb300 import hlb
