@@ -335,7 +335,7 @@ hlb_status hlb_equilibrium_x(int Qx, int Nx_eq, double u, double T, double* g);
  * walls they hold), then its x-segments (the marching update), and each item
  * waits on per-instance counters for what it reads (bounded: a wait that
  * runs out records HLB_ETIMEOUT and ends the launch).  Off, or with per-launch timing, or for a group with
- * a force field, those groups launch the node pass, the wall kernel and the
+ * a force field, those groups launch the node pass (with the walls) and the
  * stage kernel per stage.  The results agree to FP32 rounding (the moment
  * sums are formed in another order).  Drops a captured graph (synchronises).
  * No counterpart in the paper.  Errors: HLB_EINVAL. */

@@ -17,7 +17,9 @@ namespace hlb {
 namespace {
 
 // ---------------------------------------------------------------------------
-// node kernel
+// node kernels of the FP32 groups that node_df_kernel does not take (orders
+// above 15, rows that are not 8, 16 or 32 values, 2D groups of fewer than 1024
+// nodes)
 // ---------------------------------------------------------------------------
 // Per-node equilibrium factors, in two passes with no block-wide barrier:
 //   sums_kernel   streams the stage input once (one warp per node) and writes
@@ -352,7 +354,7 @@ __global__ void __launch_bounds__(128) coef_df_kernel(const GroupDev g, const fl
 // ---------------------------------------------------------------------------
 // The node pass of FP32 groups in one launch: the first g.nrows g.wchunks CTAs
 // form the walls' emitted densities, every other CTA the moment sums and the
-// factor lines of kNodeNB nodes.  The sums stream the state (HBM-bound), the
+// factor lines of NB nodes (32, or 8 in small groups; node_nb).  The sums stream the state (HBM-bound), the
 // lines are double-float arithmetic (issue- and latency-bound) and the walls a
 // few CTAs: in one launch they share the SMs instead of running in a row, and a
 // line's work is spread over the CTA (node_lines).  Per stage, against the three
