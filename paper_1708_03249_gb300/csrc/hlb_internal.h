@@ -147,7 +147,8 @@ struct GroupDev {
     int field_off;
     const double* afield;
 };
-constexpr int kQuadNodes = 20;   // points per panel of the projection quadrature
+constexpr int kQuadNodes = 24;   // points per panel of the projection quadrature, and
+constexpr double kQuadWidth = 1.5;   // the panels' width in units of sqrt(T)
 
 }  // namespace hlb
 

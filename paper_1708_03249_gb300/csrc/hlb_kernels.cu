@@ -612,8 +612,10 @@ wall_kernel(const GroupDev g, const R* __restrict__ fs) {
 // recurrence's stable order: G^{+-}_l = int_0^inf g(+-p) h_l(p) dp (l <= Nx),
 // g the Gaussian of the node's u_x and T (Sec. IV.B, the projection of Eq.
 // "eq:hh_gk"), by composite Gauss-Legendre quadrature over [0, |u_x| +
-// 13 sqrt(T)] in panels of width sqrt(T) (kQuadNodes points each; 280-320
-// points; beyond, g h_l is below 1e-17 of its maximum for l <= 31; 1e-14 of max |G| against a 30-point rule on panels of 0.02
+// 13 sqrt(T)] in panels of 1.5 sqrt(T) (kQuadNodes = 24 points each: 216 to 240
+// points while |u_x| <= 2 sqrt(T); beyond the end g h_l is below 1e-17 of its
+// maximum for l <= 31; 3.7e-15 of max |G| at order 20 against a 30-point rule on
+// panels of 0.1 sqrt(T) in extended precision, 3.8e-15 with 20 points on panels of
 // sqrt(T)), h_l(p) by the three-term recurrence of the orthonormal basis
 // (forward evaluation at a point is stable).  The integration-by-parts
 // recurrence of node_coefficients carries its rounding (and that of its erf
@@ -621,11 +623,12 @@ wall_kernel(const GroupDev g, const R* __restrict__ fs) {
 // 5e-7 of max g at N = 20.  One CTA per node and sign (72 nodes fill 144 of 152
 // SMs; both signs in one CTA save the second evaluation of h_l(p), 2 of 5
 // operations per point and order, but leave half the SMs idle), 128 threads of
-// three points each, their sums over the CTA through shared memory (the FP64
-// adds of a full-warp butterfly for every order cost as much as the points).
-// 72 nodes at order 20: 25 us per stage, 44 with one CTA of 256 threads per node
-// and butterflies (GB300; 28 with a division per moment and the products by p_y and
-// p_z of the absent axes).
+// two points each (one warp per SM quarter: the FP64 pipe is the bound, and 260 to
+// 300 points would take every quarter a third round), their sums over the CTA
+// through shared memory (the FP64 adds of a full-warp butterfly for every order
+// cost as much as the points).  72 nodes at order 20: 18.7 us per stage, 25 with
+// three rounds and two more divisions, 44 with one CTA of 256 threads per node and
+// butterflies (GB300).
 // ---------------------------------------------------------------------------
 constexpr int kQuadThreads = 128;
 template <int NMAX>
@@ -670,10 +673,10 @@ __global__ void __launch_bounds__(kQuadThreads) quad_coef_kernel(const GroupDev 
     }
     __syncthreads();
     const double ux = sMom[0], T = sMom[1];
-    const double sT = sqrt(T), width = sT;
-    const int panels = (int)ceil((fabs(ux) + 13.0 * sT) / width);
+    const double sT = sqrt(T), isT = 1.0 / sT, width = kQuadWidth * sT;
+    const int panels = (int)ceil(fma(fabs(ux), isT, 13.0) * (1.0 / kQuadWidth));
     const int npts = panels * kQuadNodes;
-    const double norm = 1.0 / (kSqrt2Pi * sT), i2T = 0.5 / T, u = sg ? -ux : ux;
+    const double norm = isT * (1.0 / kSqrt2Pi), i2T = 0.5 * isT * isT, u = sg ? -ux : ux;
     const double* ra = g.rec;
     const double* rb = g.rec + Nx;
     const double* rc = g.rec + 2 * Nx;
@@ -703,9 +706,22 @@ __global__ void __launch_bounds__(kQuadThreads) quad_coef_kernel(const GroupDev 
         if (l <= Nx) part[l][tid] = G[l];
     __syncthreads();
     double* out = g.gquad + ((size_t)node * 2 + sg) * (Nx + 1);
-    for (int l = warp; l <= Nx; l += nw) {
-        const double acc = warp_sum((part[l][lane] + part[l][lane + 32]) + (part[l][lane + 64] + part[l][lane + 96]));
-        if (lane == 0) out[l] = acc;
+    // four threads per order, 32 partial sums each
+    static_assert(4 * NMAX <= kQuadThreads, "four threads per order");
+    if (tid < 4 * NMAX) {                        // whole warps: NMAX is a multiple of 8
+        const int l = min(tid >> 2, Nx), q = tid & 3;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll 4
+        for (int i = q; i < kQuadThreads; i += 16) {
+            s0 += part[l][i];
+            s1 += part[l][i + 4];
+            s2 += part[l][i + 8];
+            s3 += part[l][i + 12];
+        }
+        double acc = (s0 + s1) + (s2 + s3);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (q == 0 && (tid >> 2) <= Nx) out[l] = acc;
     }
 }
 
