@@ -497,9 +497,11 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                 wscale[(k * G.VY + j) * G.QX2 + i] =
                     std::exp2(std::round(std::log2(1.0 / (G.tx.w[i] * G.ty.w[j] * G.tz.w[k]))));
     if (G.precision == HLB_FP32)
-        for (double ws : wscale)
+        for (double& ws : wscale) {
             if (!(ws < 1e36))
                 return fail(HLB_EUNSUPPORTED, "velocity set with weights below 1e-36: the FP32 state cannot hold it");
+            ws *= hlb::kWenoScale;
+        }
     hlb_status s;
     {
         auto split = [](const std::vector<double>& v) {

@@ -407,8 +407,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// WENO-5 face values from stencils already divided by the population's weight
-// (values O(1) wherever the population matters), without epsilon (Sec.
+// WENO-5 face values from stencils already divided by 2^10 times the
+// population's weight (kWenoScale: values of about 1e-3 wherever the population
+// matters, and B_k in range for jumps up to 1.8e22 w), without epsilon (Sec.
 // IV.C.2), face between c and d of the upwind-ordered stencil a..e, in terms
 // of the first differences d1 = b - a .. d4 = e - d and the second differences
 // s1 = d2 - d1, s2 = d3 - d2, s3 = d4 - d3:
@@ -422,8 +423,13 @@ __device__ __forceinline__ float rcp_approx(float x) {
 //   Tab. "weno");
 // - the nonlinear weights relative to the second one's, r_k = B_2 / B_k.
 //   B_2 <= C (B_1 + B_3) (a, b, c and c, d, e both smooth leave b, c, d
-//   smooth), so at most one of r_1, r_3 is large; 2^-60 B_2 added to B_1 and
-//   B_3 keeps its square in range and changes no weight that FP32 resolves;
+//   smooth), so at most one of r_1, r_3 is large; eps B_2 added to B_1 and B_3,
+//   eps = 2^-43, bounds it.  The numerator below, at most r_3^2 |R_3| plus half
+//   as much, is then below 0.4 eps^(-3/2) sqrt(B_2) (largest where B_3 = eps B_2
+//   / 3), finite wherever B_2 is: 2^-60 let r_3^2 R_3 overflow where a stencil
+//   jumps by more than 5e11, as f / w does at the fast velocities of the order-16
+//   sets beside a hot wall (8e15 at T_w = 3).  What eps adds to a weight is
+//   below 2^-86 of the jump (B_3 -> 0) or 2^-64 of R_3;
 // - face = c + (w_1 R_1 + R_2 + w_3 R_3) / (6 (w_1 + 1 + w_3)), w_1 = r_1^2 / 6
 //   and w_3 = r_3^2 / 2 the linear weights' ratios folded into r.
 // What the form saves is issue slots, which bound the marching kernels: two
@@ -435,7 +441,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // The scalar form performs the same roundings in the same order (explicit _rn
 // operations, no contraction), so a face gives the same bits in either form:
 // the wall kernel's incident flux is the stage kernels'.
-constexpr float kWenoK = 39.0f / 64.0f, kWenoFloor = 8.125e-31f, kWenoEps = 8.673617379884035e-19f,   // 2^-60
+constexpr float kWenoK = 39.0f / 64.0f, kWenoFloor = 7.7486038e-37f, kWenoEps = 1.1368684e-13f,       // 2^-43
                 kWenoR1 = 0.408248290463863f;                                                         // 1 / sqrt(6)
 __device__ __forceinline__ float weno5_scaled(float a, float b, float c, float d, float e) {
     const float d1 = __fsub_rn(b, a), d2 = __fsub_rn(c, b), d3 = __fsub_rn(d, c), d4 = __fsub_rn(e, d);

@@ -90,8 +90,8 @@ struct GroupDev {
     void* sums;              // R: [node][16] = n, j_x, j_y, j_z, E of the stage input at [0..4],
                              //    their compensation terms at [8..12]
     const void* inv_dx;      // R: 1/dx, concatenated per instance (same offsets as dx)
-    const void* wscale;      // R: [V] the power of two nearest 1/(w_x w_y w_z) per velocity (WENO
-                             //    smoothness scale; exact to apply and to undo)
+    const void* wscale;      // R: [V] the power of two nearest 1/(w_x w_y w_z) per velocity, FP32 sets times
+                             //    kWenoScale (WENO smoothness scale; exact to apply and to undo)
     int ninst, nnodes, nrows;
     const InstDev* inst;
     const int* node_start;   // [ninst + 1]
@@ -147,6 +147,10 @@ struct GroupDev {
     int field_off;
     const double* afield;
 };
+// The FP32 WENO faces' stencils in units of 2^10 w: the smoothness indicators'
+// floor then lies just above the FP32 underflow and their range above it is the
+// widest there is.
+constexpr double kWenoScale = 1.0 / 1024.0;
 constexpr int kQuadNodes = 24;   // points per panel of the projection quadrature, and
 constexpr double kQuadWidth = 1.5;   // the panels' width in units of sqrt(T)
 

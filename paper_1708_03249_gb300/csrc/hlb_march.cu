@@ -90,7 +90,7 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* fs, cons
     const R* P = static_cast<const R*>(g.p);
     const R vx = P[ix], vy = P[QX2 + jy];
     const bool xpos = ix < QX, ypos = vy > R(0);
-    const R sv = static_cast<const R*>(g.wscale)[v];
+    const R sv = static_cast<const R*>(g.wscale)[v] * R(1.0 / kWenoScale);      // the FP32 faces here want f / w itself
     const R* K = static_cast<const R*>(g.K);
     R kx[QX2], ky[VY];
 #pragma unroll
