@@ -401,7 +401,8 @@ def run_gpu(args):
     force_form = h.force_form(0)
     V = values // nodes
     h.init_equilibrium(1.0, 0.0, 0.0, 1.0)
-    segments = h.autotune()              # marching-kernel segment length, timed per group (untimed here)
+    h.autotune()                         # marching-kernel segment length, timed per group (untimed here)
+    segments = [h.step_form(0)["segment_cells"]]
 
     def barrier():
         if dist is not None:
@@ -762,7 +763,8 @@ def run_other(args):
     stream = torch.cuda.Stream()
     with hlb.Handle(cfgs, stream=stream.cuda_stream) as h:
         h.init_equilibrium()
-        segments = h.autotune()
+        h.autotune()
+        segments = sorted({h.step_form(i)["segment_cells"] for i in range(len(h.cfgs))})
         force_form = h.force_form(0)
         h.set_options(use_graphs=True, time_kernels=False)
         h.step(max(args.warmup, 30))

@@ -259,17 +259,20 @@ hlb_status hlb_get_state_dev(hlb_handle* h, void* f_dev, size_t bytes);
 hlb_status hlb_set_state_dev(hlb_handle* h, const void* f_dev, size_t bytes);
 
 /* Autotuner of the marching kernels' launch shape: for every velocity-set
- * group that runs them, times the three stage launches of one step for x-
- * segment lengths from half to four times the built-in heuristic's (CUDA
- * events on the handle's stream, one untimed round, three timed) and keeps the
- * fastest; for groups on the persistent kernel, whole persistent steps for
+ * group that runs them, times the three stage launches of one step for the
+ * built-in x-segment length and for half, one, two and four times the present
+ * one, rounded up to multiples of 6 cells from 12 on (CUDA events on the
+ * handle's stream, one untimed round, three timed) and keeps the fastest; for groups on the persistent kernel, whole persistent steps for
  * segment lengths (cells per work item) of 24 to 264 cells times one or half
  * the resident CTAs per SM.  The state is only read (the launches write the two scratch
  * buffers), so the call may come at any time between steps; it synchronises
  * the handle's streams and drops the captured graph.  The results do not
  * depend on the segment length (every cell's update is computed the same way),
  * only the time does.  segments_out (may be NULL): one entry per group in
- * creation order, the chosen length in cells (0: the group does not march).
+ * creation order, the fastest of the multiples of 6 in cells (the items' length
+ * for a group left on the persistent kernel; 0: the group does not march).  The
+ * group steps with it unless the built-in length was faster still:
+ * hlb_step_form tells the length in use.
  * No counterpart in the paper.  Errors: HLB_ECUDA, HLB_ETIMEOUT. */
 hlb_status hlb_autotune(hlb_handle* h, int* segments_out);
 

@@ -107,6 +107,7 @@ struct Group {
     size_t smem = 0;
     // marching stage kernel (node + march) or the generic per-node kernel
     int TY = 1, SX = 0, nworks = 0;
+    int SX_builtin = 0;                      // the heuristic's segment length, one of the autotuner's candidates
     bool march_ok = false;
     // per-node acceleration field (hlb_set_force_field): [nnodes][3] doubles,
     // allocated on first use; one flag per member instance
@@ -676,6 +677,7 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                     cudaGetLastError();
                 }
             }
+            G.SX_builtin = (int)sx;
             if ((s = set_segments(h, G, (int)sx)) != HLB_OK) return s;
             // the force term's form (set above): on the tensor cores where the
             // caller asked for it and the slab tiles into 16 x 8 x 8 blocks;
@@ -1721,7 +1723,7 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
     G.persist_use = false;
     hlb_status s = tune_group_stages(h, G, ev, chosen);
     if (s != HLB_OK) { G.persist_use = true; return s; }
-    const int sx_stages = G.SX;
+    const int sx_stages = G.SX, chosen_stages = *chosen;
     float ms_stages = 0.0f, ms_persist = 0.0f;
     if ((s = time_per_stage_step(h, G, ev, &ms_stages)) != HLB_OK) { G.persist_use = true; return s; }
     G.persist_use = true;
@@ -1732,20 +1734,25 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
         G.persist_use = false;
         s = set_segments(h, G, sx_stages);
         if (s != HLB_OK) G.march_ok = false;
-        *chosen = G.march_ok ? G.SX : 0;
+        *chosen = G.march_ok ? chosen_stages : 0;
     }
     return s;
 }
 
 hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
-    // candidates around the heuristic's segment length, multiples of 6 cells from
-    // 12 on (the heuristic alone goes below, for groups of less than a wave)
+    // The built-in length, which is the shortest for groups of less than a wave,
+    // and half, one, two and four times the present one as multiples of 6 cells
+    // from 12 on.  Stage kernels only, so that the node pass does not hide the
+    // difference.  us per step, tuned among the multiples of 6 alone against the
+    // built-in length (GB300): 95 x 61 cells of 128 FP64 velocities 1252 (12
+    // cells) against 795 (4), 60 x 40 of 128 FP32 72.6 against 53.3, 512 cells of
+    // 128 39.2 against 31.4.
     const int base = G.SX;
-    std::vector<int> cand;
+    std::vector<int> cand = {G.SX_builtin};
     for (int f : {-1, 0, 1, 2}) {
         int sx = f < 0 ? base >> (-f) : base << f;
         sx = std::max(12, std::min(1020, (sx + 5) / 6 * 6));
-        if (std::find(cand.begin(), cand.end(), sx) == cand.end()) cand.push_back(sx);
+        if (std::find(cand.begin() + 1, cand.end(), sx) == cand.end()) cand.push_back(sx);
     }
     // each candidate: one untimed and three timed rounds of the three stage
     // launches; inputs are the state buffer (read only) and the two scratch
@@ -1755,10 +1762,11 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
     void* Y = G.buf[(G.cur + 2) % 3].p;
     const void* ins[3] = {S, X, Y};
     void* outs[3] = {X, Y, X};
-    int best = base;
-    float best_ms = 0.0f;
+    int best = base, best_timed = 0;         // of all, and of the multiples of 6
+    float best_ms = -1.0f, best_timed_ms = -1.0f;
     hlb_status s = HLB_OK;
-    for (int sx : cand) {
+    for (size_t c = 0; c < cand.size(); ++c) {
+        const int sx = cand[c];
         if ((s = set_segments(h, G, sx)) != HLB_OK) break;
         for (int round = 0; round < 4; ++round) {
             if (round == 1) cudaEventRecord(ev.e0, h->stream);
@@ -1771,12 +1779,13 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
         cudaError_t e = cudaEventSynchronize(ev.e1);
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev.e0, ev.e1);
         if (e != cudaSuccess) { s = fail(HLB_ECUDA, std::string("autotune timing: ") + cudaGetErrorString(e)); break; }
-        if (sx == cand.front() || ms < best_ms) { best_ms = ms; best = sx; }
+        if (best_ms < 0.0f || ms < best_ms) { best_ms = ms; best = sx; }
+        if (c > 0 && (best_timed_ms < 0.0f || ms < best_timed_ms)) { best_timed_ms = ms; best_timed = sx; }
     }
-    // the chosen length (the heuristic's after an error), or no marching at all
+    // the chosen length (the one before after an error), or no marching at all
     const hlb_status s2 = set_segments(h, G, s == HLB_OK ? best : base);
     if (s2 != HLB_OK) G.march_ok = false;
-    *chosen = G.march_ok ? G.SX : 0;
+    *chosen = !G.march_ok ? 0 : (best_timed ? best_timed : G.SX);
     return s != HLB_OK ? s : s2;
 }
 }  // namespace

@@ -266,7 +266,8 @@ class Handle:
         _check(lib().hlb_moments_wait(self._h))
 
     def autotune(self):
-        """hlb_autotune: time segment lengths per velocity-set group, keep the fastest; returns them."""
+        """hlb_autotune: time segment lengths per velocity-set group and keep the fastest; returns per group the
+        fastest multiple of 6 cells (step_form tells the length in use, which may be the built-in one)."""
         out = (C.c_int * len(self.cfgs))(*([-1] * len(self.cfgs)))     # groups <= instances
         _check(lib().hlb_autotune(self._h, out))
         return [v for v in out if v >= 0]

