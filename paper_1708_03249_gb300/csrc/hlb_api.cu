@@ -1712,26 +1712,30 @@ hlb_status time_per_stage_step(hlb_handle* h, Group& G, EventPair& ev, float* st
 
 hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen);
 
-// A group the persistent kernel can step: the per-stage launches with their
-// best segment length against the persistent kernel with its best segment
-// length and grid, whole steps timed; the faster is kept (the results agree
-// to FP32 rounding either way).
+// A group the persistent kernel can step as the handle stands (switched on, no
+// per-launch timing, no field): the per-stage launches with their best segment
+// length against the persistent kernel with its best segment length and grid,
+// whole steps timed; the faster is kept from here on, whatever the group's
+// size (the results agree to FP32 rounding either way).  Else, and after an
+// error, the group's form stays what it was: a form that was not timed is not
+// switched on.
 hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
-    G.persist_use = true;
-    G.persist_auto = true;               // by measurement from here on, not by size
-    if (!persist_on(h, G)) return tune_group_stages(h, G, ev, chosen);
-    G.persist_use = false;
+    const bool use = G.persist_use, by_default = G.persist_auto;
+    G.persist_use = G.persist_auto = true;
+    const bool both = persist_on(h, G);
+    G.persist_use = use;
+    G.persist_auto = by_default;
     hlb_status s = tune_group_stages(h, G, ev, chosen);
-    if (s != HLB_OK) { G.persist_use = true; return s; }
+    if (s != HLB_OK || !both) return s;
     const int sx_stages = G.SX, chosen_stages = *chosen;
     float ms_stages = 0.0f, ms_persist = 0.0f;
-    if ((s = time_per_stage_step(h, G, ev, &ms_stages)) != HLB_OK) { G.persist_use = true; return s; }
-    G.persist_use = true;
+    if ((s = time_per_stage_step(h, G, ev, &ms_stages)) != HLB_OK) return s;
     if ((s = tune_persist(h, G, ev, chosen, &ms_persist)) != HLB_OK) return s;
     G.tuned_ms_stages = ms_stages;
     G.tuned_ms_persist = ms_persist;
-    if (ms_stages < ms_persist) {
-        G.persist_use = false;
+    G.persist_auto = true;
+    G.persist_use = ms_persist <= ms_stages;
+    if (!G.persist_use) {
         s = set_segments(h, G, sx_stages);
         if (s != HLB_OK) G.march_ok = false;
         *chosen = G.march_ok ? chosen_stages : 0;

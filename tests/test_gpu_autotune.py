@@ -1,7 +1,7 @@
 """hlb_autotune on groups whose built-in segments are shorter than a multiple of 6
 from 12 cells on: it times the built-in length too and keeps it where it is
-the fastest (by 1.2 to 1.6 times on these handles), and the step after it
-gives the same bits."""
+the fastest (by 1.2 to 1.6 times on these handles), and the steps after it
+give the same bits.  A form that it could not time is not switched on."""
 import numpy as np
 import pytest
 
@@ -40,3 +40,25 @@ def test_autotune_keeps_the_short_built_in_segments(name):
             h.step(3)
             outs.append(h.get_state())
     np.testing.assert_array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("what", ["per_launch_timing", "force_field"])
+def test_autotune_switches_no_untimed_form_on(what):
+    # with per-launch timing or a force field on, hlb_autotune can time the
+    # per-stage launches alone: once that is off again the group steps as before
+    from paper_1708_03249_gb300 import hlb
+    cfg = W.make(Qx=8, Qy=8, nx=300, Kn=0.1, precision=W.FP32, ax=-0.2)
+    with hlb.Handle(cfg, stream=_stream()) as h:
+        assert not h.step_form(0)["persistent"]
+        h.init_equilibrium()
+        if what == "force_field":
+            h.set_force_field(0, ax=np.full(300, 0.1))
+        else:
+            h.set_options(use_graphs=True, time_kernels=True)
+        h.autotune()
+        if what == "force_field":
+            h.set_force_field(0)
+        else:
+            h.set_options(use_graphs=True, time_kernels=False)
+        form = h.step_form(0)
+        assert not form["persistent"] and form["tuned_ms"] == (0.0, 0.0)
