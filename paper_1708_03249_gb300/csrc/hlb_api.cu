@@ -128,7 +128,8 @@ struct Group {
     bool persist_use = true;                 // the autotuner's pick: persistent or per-stage launches
     float tuned_ms_persist = 0.0f, tuned_ms_stages = 0.0f;   // its best step times (0: not timed)
     int persist_per_sm = 0, persist_grid = 0, persist_nitems = 0;
-    DevBuf d_pctl, d_nseg, d_nchunk, d_pitems;
+    int PSX = 0;                             // cells per segment item (SX is the per-stage launches')
+    DevBuf d_pctl, d_pworks, d_nseg, d_nchunk, d_pitems;
 };
 
 // Host-side NVTX range (the library's calls and the RK-3 stages they enqueue,
@@ -360,29 +361,39 @@ void fill_dev(Group& G) {
     d.glrule = static_cast<const double*>(G.d_glrule.p);
 }
 
-// The marching kernel's work list: one CTA per (p_z slab, instance, strip of
-// TY rows, x-segment of SX cells).
-hlb_status set_segments(hlb_handle* h, Group& G, int SX) {
-    G.SX = SX;
+// A marching work list: one item per (p_z slab, instance, strip of TY rows,
+// x-segment of SX cells).
+std::vector<hlb::Work> segment_list(const hlb_handle* h, const Group& G, int SX) {
     std::vector<hlb::Work> works;
     for (int kz = 0; kz < G.VZ; ++kz)
         for (size_t m = 0; m < G.members.size(); ++m) {
             const hlb_config& c = h->cfg[G.members[m]];
-            for (int xa = 0; xa < c.nx; xa += G.SX)
+            for (int xa = 0; xa < c.nx; xa += SX)
                 for (int y0 = 0; y0 < c.ny; y0 += G.TY) {
                     hlb::Work w{};
-                    w.inst = (int)m; w.y0 = y0; w.xa = xa; w.xb = std::min(c.nx, xa + G.SX); w.kz = kz;
+                    w.inst = (int)m; w.y0 = y0; w.xa = xa; w.xb = std::min(c.nx, xa + SX); w.kz = kz;
                     works.push_back(w);
                 }
         }
+    return works;
+}
+
+// The per-stage marching launch's work list (one CTA per item).
+hlb_status set_segments(hlb_handle* h, Group& G, int SX) {
+    G.SX = SX;
+    const std::vector<hlb::Work> works = segment_list(h, G, SX);
     G.nworks = (int)works.size();
-    hlb_status st = upload(G.d_works, works);
-    if (st != HLB_OK || !G.persist_ok) return st;
-    // the persistent kernel's items of one stage: the node chunks (one cell
-    // per thread) of every instance, then the segments of every instance (in
-    // the work list's order: instance, then x).  A segment then rarely finds
-    // its instance's node chunks unfinished (they were taken long before),
-    // and a node chunk of the next stage its instance's segments.
+    return upload(G.d_works, works);
+}
+
+// The persistent kernel's items of one stage: the node chunks (one cell per
+// thread) of every instance, then the segments of every instance (in the work
+// list's order: instance, then x).  A segment then rarely finds its instance's
+// node chunks unfinished (they were taken long before), and a node chunk of
+// the next stage its instance's segments.
+hlb_status set_persist_items(hlb_handle* h, Group& G, int PSX) {
+    G.PSX = PSX;
+    const std::vector<hlb::Work> works = segment_list(h, G, PSX);
     const int chunk = std::min(G.V, hlb::kPersistNodeChunk);
     std::vector<int> nseg(G.members.size(), 0), nchunk(G.members.size(), 0);
     std::vector<hlb::PersistItem> items;
@@ -398,6 +409,8 @@ hlb_status set_segments(hlb_handle* h, Group& G, int SX) {
         ++nseg[works[j].inst];
     }
     G.persist_nitems = (int)items.size();
+    hlb_status st;
+    if ((st = upload(G.d_pworks, works)) != HLB_OK) return st;
     if ((st = upload(G.d_pitems, items)) != HLB_OK) return st;
     if ((st = upload(G.d_nchunk, nchunk)) != HLB_OK) return st;
     return upload(G.d_nseg, nseg);
@@ -666,13 +679,21 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                     // launches.  us per step, persistent against per-stage
                     // (GB300): 512 cells of 128 velocities 170 against 39, 131072
                     // of 512 2332 against 1542, 37 seeded channels 640 against 117,
-                    // 4096 9251 against 6050.  Segments of at least 24 cells: an
-                    // item of the persistent kernel reads its tables anew.
+                    // 4096 9251 against 6050.
                     G.persist_auto = G.members.size() > 1 && G.nnodes <= 1024;
-                    if (G.persist_auto) sx = std::max(24LL, sx);
+                    // Its segment items, which read their tables anew, have a
+                    // length of their own: in small groups one wave of the
+                    // shortest that fill it, up to 24 cells; in large ones the
+                    // cells over eight CTAs per SM, up to 512.  us per step (GB300):
+                    // 100000 cells of 128 velocities 567 with 84 cells against 610
+                    // with the per-stage launches' 48, two channels of 64 cells 107
+                    // with 4 against 133 with 24.
+                    const long long wave = (xwork + (long long)nsm * per - 1) / ((long long)nsm * per);
+                    const long long psx = std::max(std::min(24LL, wave), std::min(512LL, xwork / (8LL * nsm)));
                     G.persist_per_sm = per;
                     G.persist_grid = nsm * per;
                     if ((s = upload(G.d_pctl, std::vector<int>(4 + 2 * G.members.size(), 0))) != HLB_OK) return s;
+                    if ((s = set_persist_items(h, G, (int)std::max(4LL, (psx + 3) / 4 * 4))) != HLB_OK) return s;
                 } else {
                     cudaGetLastError();
                 }
@@ -776,7 +797,7 @@ void enqueue_persist_step(Group& G, cudaStream_t st) {
     a.nchunk = static_cast<const int*>(G.d_nchunk.p);
     a.nseg = static_cast<const int*>(G.d_nseg.p);
     cudaMemsetAsync(ctl, 0, (4 + 2 * ninst) * sizeof(int), st);
-    hlb::launch_persist(G.adv, G.QX2, G.VY, G.force_form, G.dev, (const hlb::Work*)G.d_works.p, a,
+    hlb::launch_persist(G.adv, G.QX2, G.VY, G.force_form, G.dev, (const hlb::Work*)G.d_pworks.p, a,
                         std::min(G.persist_grid, 3 * G.persist_nitems), st);
 }
 
@@ -1655,14 +1676,14 @@ hlb_status tune_persist(hlb_handle* h, Group& G, EventPair& ev, int* chosen, flo
     int dev = 0, nsm = 1;
     HLB_CUDA(cudaGetDevice(&dev));
     HLB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int base_sx = G.SX, base_grid = G.persist_grid;
+    const int base_sx = G.PSX, base_grid = G.persist_grid;
     std::vector<int> per_sm = {G.persist_per_sm};
     if (G.persist_per_sm >= 2) per_sm.push_back(G.persist_per_sm / 2);
     int best_sx = base_sx, best_grid = base_grid;
     float best_ms = -1.0f;
     hlb_status s = HLB_OK;
-    for (int sx : {24, 36, 48, 72, 96, 132, 192, 264}) {
-        if ((s = set_segments(h, G, sx)) != HLB_OK) break;
+    for (int sx : {base_sx, 24, 36, 48, 72, 96, 132, 192, 264}) {
+        if ((s = set_persist_items(h, G, sx)) != HLB_OK) break;
         for (int per : per_sm) {
             G.persist_grid = nsm * per;
             for (int round = 0; round < 4; ++round) {
@@ -1679,9 +1700,9 @@ hlb_status tune_persist(hlb_handle* h, Group& G, EventPair& ev, int* chosen, flo
         if (s != HLB_OK) break;
     }
     G.persist_grid = s == HLB_OK ? best_grid : base_grid;
-    const hlb_status s2 = set_segments(h, G, s == HLB_OK ? best_sx : base_sx);
-    if (s2 != HLB_OK) G.march_ok = false;
-    *chosen = G.march_ok ? G.SX : 0;
+    const hlb_status s2 = set_persist_items(h, G, s == HLB_OK ? best_sx : base_sx);
+    if (s2 != HLB_OK) G.persist_ok = false;
+    *chosen = G.PSX;
     *step_ms = best_ms / 3.0f;
     return s != HLB_OK ? s : s2;
 }
@@ -1727,7 +1748,7 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
     G.persist_auto = by_default;
     hlb_status s = tune_group_stages(h, G, ev, chosen);
     if (s != HLB_OK || !both) return s;
-    const int sx_stages = G.SX, chosen_stages = *chosen;
+    const int chosen_stages = *chosen;
     float ms_stages = 0.0f, ms_persist = 0.0f;
     if ((s = time_per_stage_step(h, G, ev, &ms_stages)) != HLB_OK) return s;
     if ((s = tune_persist(h, G, ev, chosen, &ms_persist)) != HLB_OK) return s;
@@ -1735,12 +1756,8 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
     G.tuned_ms_persist = ms_persist;
     G.persist_auto = true;
     G.persist_use = ms_persist <= ms_stages;
-    if (!G.persist_use) {
-        s = set_segments(h, G, sx_stages);
-        if (s != HLB_OK) G.march_ok = false;
-        *chosen = G.march_ok ? chosen_stages : 0;
-    }
-    return s;
+    if (!G.persist_use) *chosen = chosen_stages;
+    return HLB_OK;
 }
 
 hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
@@ -1867,7 +1884,7 @@ hlb_status hlb_step_form(const hlb_handle* h, int inst, int* persistent, int* se
     const Group& G = *h->groups[h->inst_group[inst]];
     const bool p = persist_on(h, G);
     if (persistent) *persistent = p ? 1 : 0;
-    if (segment_cells) *segment_cells = G.march_ok ? G.SX : 0;
+    if (segment_cells) *segment_cells = p ? G.PSX : (G.march_ok ? G.SX : 0);
     if (ctas) *ctas = p ? std::min(G.persist_grid, 3 * G.persist_nitems) : (G.march_ok ? G.nworks : G.grid);
     if (tuned_ms) {
         tuned_ms[0] = G.tuned_ms_persist;

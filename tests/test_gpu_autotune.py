@@ -62,3 +62,45 @@ def test_autotune_switches_no_untimed_form_on(what):
             h.set_options(use_graphs=True, time_kernels=False)
         form = h.step_form(0)
         assert not form["persistent"] and form["tuned_ms"] == (0.0, 0.0)
+
+
+def test_persistent_items_have_their_own_length():
+    # the persistent kernel's segment items do not follow the per-stage
+    # launches' segments: longer in a large group (an item reads its tables
+    # anew), and untouched where the tuner lengthens or shortens the latter
+    from paper_1708_03249_gb300 import hlb
+    with hlb.Handle(W.make(Qx=8, Qy=8, nx=100000, Kn=0.1, precision=W.FP32), stream=_stream()) as h:
+        per_stage = h.step_form(0)["segment_cells"]
+        h.set_persistent(True)
+        items = h.step_form(0)["segment_cells"]
+        assert items > per_stage
+        h.set_persistent(False)
+        h.init_equilibrium()
+        h.autotune()
+        h.set_persistent(True)
+        form = h.step_form(0)
+        assert form["persistent"] and form["segment_cells"] == items
+
+
+@pytest.mark.parametrize("nx", [6, 7, 9, 53])
+def test_persistent_short_items_give_the_same_bits(nx):
+    # items of 4 cells (one iteration each), ragged last ones among them,
+    # against the lengths that the tuner may pick
+    from paper_1708_03249_gb300 import hlb
+    cfgs = [W.make(Qx=8, Qy=8, nx=n, Kn=0.1, precision=W.FP32, T_right=1.3, ax=-0.2) for n in (nx, 150)]
+    outs = []
+    for tune in (False, True):
+        with hlb.Handle(cfgs, stream=_stream()) as h:
+            h.set_persistent(True)
+            h.init_equilibrium(1.0, 0.05, 0.0, 1.1)
+            if tune:
+                h.autotune()
+            else:
+                assert h.step_form(0)["segment_cells"] == 4
+            persistent = h.step_form(0)["persistent"]
+            h.step(5)
+            outs.append(h.get_state())
+    if persistent:
+        np.testing.assert_array_equal(outs[0], outs[1])
+    else:
+        np.testing.assert_allclose(outs[0], outs[1], rtol=0, atol=2e-6 * np.abs(outs[1]).max())
