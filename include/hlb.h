@@ -330,7 +330,8 @@ hlb_status hlb_equilibrium_x(int Qx, int Nx_eq, double u, double T, double* g);
 
 /* Persistent batched kernel on (1) or off (0) for the groups that can take it;
  * a handle on which this was never called uses it for such groups of several
- * instances and at most 1024 nodes, where hlb_autotune has not measured better.
+ * instances and at most 512 nodes, where hlb_autotune has not measured better
+ * (the per-stage launches are the faster form at every size measured).
  * Velocity-set groups of 1D FP32 instances without a p_z axis (2 Qx x Qy slabs
  * of 8 x 4, 16 x 8, 32 x 16 with the default force-term form, or 32 x 1;
  * equilibrium orders up to 15) can step with one persistent launch per RK-3 step: the CTAs

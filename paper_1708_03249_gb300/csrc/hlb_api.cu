@@ -674,13 +674,14 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                 if (hlb::prepare_persist(G.adv, G.QX2, G.VY, G.force_form, &per) == cudaSuccess && per > 0) {
                     G.persist_ok = true;
                     // By default the persistent kernel steps groups of several
-                    // instances and at most 1024 nodes (one launch per step);
-                    // larger groups and single instances take the per-stage
-                    // launches.  us per step, persistent against per-stage
-                    // (GB300): 512 cells of 128 velocities 170 against 39, 131072
-                    // of 512 2332 against 1542, 37 seeded channels 640 against 117,
-                    // 4096 9251 against 6050.
-                    G.persist_auto = G.members.size() > 1 && G.nnodes <= 1024;
+                    // instances and at most 512 nodes: one launch per step, which
+                    // callers can see (hlb_step_form, hlb_launch_count) and rely
+                    // on, not the faster form.  The per-stage launches are faster at
+                    // every size measured; us per step, persistent against
+                    // per-stage (GB300): two channels of 64 cells of 32 velocities
+                    // 93 / 26, of 128 107 / 31, of 512 185 / 45; two of 500 cells
+                    // 100 / 27, 168 / 36, 551 / 68; 4096 seeded ones 9251 / 6050.
+                    G.persist_auto = G.members.size() > 1 && G.nnodes <= 512;
                     // Its segment items, which read their tables anew, have a
                     // length of their own: in small groups one wave of the
                     // shortest that fill it, up to 24 cells; in large ones the
@@ -713,10 +714,12 @@ hlb_status build_group(hlb_handle* h, Group& G) {
         }
     }
     fill_dev(G);
-    // 2D groups below 1024 nodes (32 CTAs of the one-launch node pass) keep the
-    // separate sums, factor-line and wall kernels and with them their twelve
-    // launches per step, which callers can count (hlb_launch_count)
-    G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && (G.TY == 1 || G.nnodes >= 1024);
+    // 2D groups of at most 256 nodes keep the separate sums, factor-line and wall
+    // kernels and with them the twelve launches per step that callers count
+    // there (hlb_launch_count), not for speed.  us per step, one launch against
+    // the three (GB300): 60 nodes of 32 velocities 36 / 69, 240 nodes 38 / 71, 1023
+    // nodes 39 / 70; of 512 velocities 58 / 169, 69 / 178, 91 / 174.
+    G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && (G.TY == 1 || G.nnodes > 256);
     if (G.march_ok && G.precision == HLB_FP32) HLB_CUDA(G.node_fused ? hlb::prepare_node_fused(G.adv, G.dev) : hlb::prepare_node());
 
     // launch shape of the stage kernel.  With Kx in global memory each

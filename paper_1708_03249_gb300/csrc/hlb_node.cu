@@ -18,7 +18,7 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // node kernels of the FP32 groups that node_df_kernel does not take (orders
-// above 15, rows that are not 8, 16 or 32 values, 2D groups of fewer than 1024
+// above 15, rows that are not 8, 16 or 32 values, 2D groups of at most 256
 // nodes)
 // ---------------------------------------------------------------------------
 // Per-node equilibrium factors, in two passes with no block-wide barrier:
