@@ -603,8 +603,10 @@ __device__ __forceinline__ float2 upwind2_face2(float2 b, float2 c) {
 }
 
 // Quadratic extrapolation of an incident population into the first and second
-// ghost cells beyond the right wall from the wall cell f0 and the next two
-// inward (Sec. IV.C.3), rounded the same way wherever a segment starts.
+// ghost cells beyond a wall from the wall cell f0 and the next two inward (Sec.
+// IV.C.3).  Every FP32 kernel that runs on the packed faces forms them with
+// these: the flux that fixes n_w is then the stage kernels' to the last bit,
+// wherever a segment starts, and the two walls are mirror images.
 __device__ __forceinline__ float wall_ghost1(float f0, float f1, float f2) { return fmaf(3.0f, __fsub_rn(f0, f1), f2); }
 __device__ __forceinline__ float wall_ghost2(float f0, float f1, float f2) {
     return fmaf(6.0f, f0, fmaf(-8.0f, f1, __fmul_rn(3.0f, f2)));

@@ -191,7 +191,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs,
                 else if (x < -2) val = 0.0f;          // never read by a negative velocity
                 else {
                     const float f0 = f[0] * sv, f1 = f[V] * sv, f2v = f[2 * V] * sv;
-                    val = x == -1 ? 3.0f * f0 - 3.0f * f1 + f2v : 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
+                    val = x == -1 ? wall_ghost1(f0, f1, f2v) : wall_ghost2(f0, f1, f2v);
                 }
             } else if (!xpos) val = nwr;
             else if (x > nx + 1) val = 0.0f;          // never read by a positive velocity

@@ -169,8 +169,7 @@ __device__ __forceinline__ void node_item(const GroupDev& g, const PersistArgs& 
                         f2v = __ldcg(fin + a0 + 2 * st + t) * sv;
             float face;
             if (ADV == HLB_WENO5_) {
-                const float d = 3.0f * f0 - 3.0f * f1 + f2v, e = 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
-                face = weno5_scaled(f2v, f1, f0, d, e);
+                face = weno5_scaled(f2v, f1, f0, wall_ghost1(f0, f1, f2v), wall_ghost2(f0, f1, f2v));
             } else {
                 face = upwind2_face<float>(f1, f0);
             }
@@ -317,7 +316,7 @@ __device__ HLB_MARCH_ITEM_ATTR uint32_t march_item(const GroupDev& g, const Pers
                 else if (x < -2) val = 0.0f;          // never read by a negative velocity
                 else {
                     const float f0 = __ldcg(f) * sv, f1 = __ldcg(f + V) * sv, f2v = __ldcg(f + 2 * V) * sv;
-                    val = x == -1 ? 3.0f * f0 - 3.0f * f1 + f2v : 6.0f * f0 - 8.0f * f1 + 3.0f * f2v;
+                    val = x == -1 ? wall_ghost1(f0, f1, f2v) : wall_ghost2(f0, f1, f2v);
                 }
             } else if (!xpos) val = nwr;
             else if (x > nx + 1) val = 0.0f;          // never read by a positive velocity

@@ -38,8 +38,7 @@ __device__ __forceinline__ void wall_block(const GroupDev& g, const R* fs, int b
             const float f0 = frow[a + v] * sv, f1 = frow[a + step + v] * sv, f2 = frow[a + 2 * step + v] * sv;
             float face;
             if (ADV == HLB_WENO5_) {
-                const float d = 3.0f * f0 - 3.0f * f1 + f2, e = 6.0f * f0 - 8.0f * f1 + 3.0f * f2;
-                face = weno5_scaled(f2, f1, f0, d, e);
+                face = weno5_scaled(f2, f1, f0, wall_ghost1(f0, f1, f2), wall_ghost2(f0, f1, f2));
             } else {
                 face = upwind2_face<float>(f1, f0);
             }
