@@ -263,9 +263,9 @@ hlb_status hlb_set_state_dev(hlb_handle* h, const void* f_dev, size_t bytes);
  * built-in x-segment length and for half, one, two and four times the present
  * one, rounded up to multiples of 6 cells from 12 on (CUDA events on the
  * handle's stream, one untimed round, three timed) and keeps the fastest; for
- * groups on the persistent kernel, whole persistent steps for the built-in
- * length of its segment items and 24 to 264 cells times one or half the
- * resident CTAs per SM.  The state is only read (the launches write the two scratch
+ * groups on the persistent kernel, whole persistent steps for segment items of
+ * 24 to 264 cells, and of the built-in length where that is shorter, times one
+ * or half the resident CTAs per SM.  The state is only read (the launches write the two scratch
  * buffers), so the call may come at any time between steps; it synchronises
  * the handle's streams and drops the captured graph.  The results do not
  * depend on the segment length (every cell's update is computed the same way),

@@ -1685,7 +1685,9 @@ hlb_status tune_persist(hlb_handle* h, Group& G, EventPair& ev, int* chosen, flo
     int best_sx = base_sx, best_grid = base_grid;
     float best_ms = -1.0f;
     hlb_status s = HLB_OK;
-    for (int sx : {base_sx, 24, 36, 48, 72, 96, 132, 192, 264}) {
+    std::vector<int> cand = {24, 36, 48, 72, 96, 132, 192, 264};
+    if (base_sx < 24) cand.push_back(base_sx);           // the built-in length of small groups
+    for (int sx : cand) {
         if ((s = set_persist_items(h, G, sx)) != HLB_OK) break;
         for (int per : per_sm) {
             G.persist_grid = nsm * per;
@@ -1772,12 +1774,14 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
     // cells) against 795 (4), 60 x 40 of 128 FP32 72.6 against 53.3, 512 cells of
     // 128 39.2 against 31.4.
     const int base = G.SX;
-    std::vector<int> cand = {G.SX_builtin};
+    std::vector<int> cand;
     for (int f : {-1, 0, 1, 2}) {
         int sx = f < 0 ? base >> (-f) : base << f;
         sx = std::max(12, std::min(1020, (sx + 5) / 6 * 6));
-        if (std::find(cand.begin() + 1, cand.end(), sx) == cand.end()) cand.push_back(sx);
+        if (std::find(cand.begin(), cand.end(), sx) == cand.end()) cand.push_back(sx);
     }
+    const size_t multiples = cand.size();
+    if (std::find(cand.begin(), cand.end(), G.SX_builtin) == cand.end()) cand.push_back(G.SX_builtin);
     // each candidate: one untimed and three timed rounds of the three stage
     // launches; inputs are the state buffer (read only) and the two scratch
     // buffers, outputs only the scratch buffers, so the state is kept
@@ -1804,7 +1808,7 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev.e0, ev.e1);
         if (e != cudaSuccess) { s = fail(HLB_ECUDA, std::string("autotune timing: ") + cudaGetErrorString(e)); break; }
         if (best_ms < 0.0f || ms < best_ms) { best_ms = ms; best = sx; }
-        if (c > 0 && (best_timed_ms < 0.0f || ms < best_timed_ms)) { best_timed_ms = ms; best_timed = sx; }
+        if (c < multiples && (best_timed_ms < 0.0f || ms < best_timed_ms)) { best_timed_ms = ms; best_timed = sx; }
     }
     // the chosen length (the one before after an error), or no marching at all
     const hlb_status s2 = set_segments(h, G, s == HLB_OK ? best : base);
