@@ -197,7 +197,6 @@ void launch_node(const GroupDev& g, const void* fs, cudaStream_t st);
 // The node pass and the walls in one launch, for the FP32 groups it takes.
 bool node_fused_available(int precision, const GroupDev& g);
 int sm_count();          // of the current device when first called (152 if it cannot be asked)
-cudaError_t prepare_node_fused(int adv, const GroupDev& g);
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 cudaError_t prepare_node();

@@ -158,8 +158,10 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
     const R* gT = static_cast<const R*>(g.Tt);
     for (int i = tid; i < L.nK; i += bs) sK[i] = gK[i];
     for (int i = tid; i < L.nP; i += bs) sP[i] = gP[i];
-    for (int i = tid; i < L.nT; i += bs) sT[i] = gT[i];
-    for (int i = tid; i < L.nRec; i += bs) sRec[i] = g.rec[i];
+    if (sizeof(R) == 4) {                     // FP64 groups read the node pass's lines instead
+        for (int i = tid; i < L.nT; i += bs) sT[i] = gT[i];
+        for (int i = tid; i < L.nRec; i += bs) sRec[i] = g.rec[i];
+    }
     __syncthreads();
 
     const int V = g.V, QX2 = g.QX2, VY = g.VY, VZ = g.VZ, Qx = g.Qx;
@@ -237,11 +239,8 @@ stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ f
         // 2. equilibrium factors g_x (times n), g_y, g_z
         {
             const int nf = QX2 + VY + VZ;
-            // a velocity range of a 1D set (VY = VZ = 1) needs its own g_x only
-            const bool x_range = nvc > 1 && VY * VZ == 1;
             for (int t = tid; t < nf; t += bs) {
                 double acc = 0.0;
-                if (t < QX2 && x_range && (t < v0 || t >= v1)) continue;
                 if (t < QX2) {
                     const int k = t % Qx, sg = t / Qx;
                     const double* G = sCoef + sg * (g.Nx + 1);
@@ -918,16 +917,15 @@ moments_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, double
 // warps of 256-thread CTAs, 30 % of the DRAM rate).  1024 x 512 nodes of 1024
 // velocities (GB300): 0.459 ms against 0.771; reading the state alone takes 0.317.
 constexpr int kMomNodes = 32, kMomThreads = 128;
-template <typename R>
 __global__ void __launch_bounds__(kMomThreads, 6)
-moments_rows_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, double* u_out, double* T_out,
+moments_rows_kernel(const GroupDev g, const float* __restrict__ fs, double* n_out, double* u_out, double* T_out,
                     double* q_out, int node_base, const long long* __restrict__ gnode) {
     extern __shared__ __align__(16) unsigned char mom_smem[];
     __shared__ long long sOff[kMomNodes];
     __shared__ float sSum[kMomNodes][21];                // nine sums, nine error terms (padded)
     float4* sYZ = reinterpret_cast<float4*>(mom_smem);   // [VY VZ]: p_y, p_z, p_y^2 + p_z^2
     const int V = g.V, QX2 = g.QX2, VY = g.VY, rows = g.VY * g.VZ;
-    const R* P = static_cast<const R*>(g.p);
+    const float* P = static_cast<const float*>(g.p);
     const int tid = threadIdx.x, base = blockIdx.x * kMomNodes, nb = min(kMomNodes, g.nnodes - base);
     int ii = 0;
     if (tid < nb) {
@@ -936,13 +934,13 @@ moments_rows_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, d
     }
     for (int k = tid; k < rows; k += kMomThreads) {
         float4 y;
-        y.x = P[QX2 + k % VY]; y.y = P[QX2 + VY + k / VY]; y.z = y.x * y.x + y.y * y.y; y.w = R(0);
+        y.x = P[QX2 + k % VY]; y.y = P[QX2 + VY + k / VY]; y.z = y.x * y.x + y.y * y.y; y.w = 0.0f;
         sYZ[k] = y;
     }
     __syncthreads();
     const int lane = tid & 31, sl = lane & 7, lg = __ffs(QX2) - 1;
     const int x0 = (4 * sl) & (QX2 - 1);
-    R px[4], px2[4], px3[4];
+    float px[4], px2[4], px3[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         px[e] = P[x0 + e]; px2[e] = px[e] * px[e]; px3[e] = px2[e] * px[e];
@@ -978,7 +976,7 @@ moments_rows_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, d
                 csum_add2(s2[4], c2[4], make_float2(fmaf(yz.z, jp.x, sq.y), 0.0f));
             }
         }
-        R a[9], c[9];
+        float a[9], c[9];
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
             a[2 * q] = s2[q].x; c[2 * q] = c2[q].x;
@@ -986,7 +984,7 @@ moments_rows_kernel(const GroupDev g, const R* __restrict__ fs, double* n_out, d
         }
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            csum_warp<R, 4>(a[k], c[k]);
+            csum_warp<float, 4>(a[k], c[k]);
             if (sl == 0 && kn < nb) {
                 sSum[kn][k] = a[k];
                 sSum[kn][10 + k] = c[k];
@@ -1132,7 +1130,7 @@ void launch_moments(int precision, const GroupDev& g, const void* fs, double* n,
     const int grid = (g.nnodes + 255) / 256 < 152 * 8 ? (g.nnodes + 255) / 256 : 152 * 8;
     const bool table = g.V + g.VY * g.VZ <= kMomentTableMax;
     if (precision != HLB_FP64_ && table && (g.QX2 & 3) == 0 && (g.QX2 & (g.QX2 - 1)) == 0 && g.QX2 <= 32) {
-        moments_rows_kernel<float><<<(g.nnodes + kMomNodes - 1) / kMomNodes, kMomThreads, g.VY * g.VZ * sizeof(float4), st>>>(
+        moments_rows_kernel<<<(g.nnodes + kMomNodes - 1) / kMomNodes, kMomThreads, g.VY * g.VZ * sizeof(float4), st>>>(
             g, (const float*)fs, n, u, T, q, node_base, gnode);
         return;
     }

@@ -6,7 +6,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <type_traits>
 
 #include "hlb_coef.cuh"
 #include "hlb_device.cuh"
@@ -31,29 +30,27 @@ namespace {
 // whatever its mask, so every FP64 instruction runs on full warps; FP32
 // groups with Nx <= 15 run the recurrences and dot products in double-float
 // (FP64 only for erf, exp, sqrt, once per node).
-template <typename R>
-__global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __restrict__ fs, R* __restrict__ sums) {
+__global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const float* __restrict__ fs, float* __restrict__ sums) {
     extern __shared__ __align__(16) double ssm[];
-    using R4 = typename std::conditional<sizeof(R) == 4, float4, double4>::type;
     const int QX2 = g.QX2, VY = g.VY, VZ = g.VZ, V = g.V;
     const int tid = threadIdx.x, bs = blockDim.x;
     const int warp = tid >> 5, lane = tid & 31, nw = bs >> 5;
-    R4* sM = reinterpret_cast<R4*>(ssm);                 // [V]: p_x, p_y, p_z, |p|^2
-    R4* sYZ = sM + V;                                    // [VY * VZ]: p_y, p_z, p_y^2 + p_z^2
-    const R* px = static_cast<const R*>(g.p);
-    const R* py = px + QX2;
-    const R* pz = py + VY;
+    float4* sM = reinterpret_cast<float4*>(ssm);         // [V]: p_x, p_y, p_z, |p|^2
+    float4* sYZ = sM + V;                                // [VY * VZ]: p_y, p_z, p_y^2 + p_z^2
+    const float* px = static_cast<const float*>(g.p);
+    const float* py = px + QX2;
+    const float* pz = py + VY;
     for (int v = tid; v < V; v += bs) {
         const int ix = v % QX2, jy = (v / QX2) % VY, kz = v / (QX2 * VY);
-        const R a = px[ix], b = py[jy], c = pz[kz];
-        R4 m4;
+        const float a = px[ix], b = py[jy], c = pz[kz];
+        float4 m4;
         m4.x = a; m4.y = b; m4.z = c; m4.w = a * a + b * b + c * c;
         sM[v] = m4;
     }
     for (int bq = tid; bq < VY * VZ; bq += bs) {
-        const R b = py[bq % VY], c = pz[bq / VY];
-        R4 y4;
-        y4.x = b; y4.y = c; y4.z = b * b + c * c; y4.w = R(0);
+        const float b = py[bq % VY], c = pz[bq / VY];
+        float4 y4;
+        y4.x = b; y4.y = c; y4.z = b * b + c * c; y4.w = 0.0f;
         sYZ[bq] = y4;
     }
     __syncthreads();
@@ -63,8 +60,8 @@ __global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __
     // compensated tree then has three levels, and each shuffle serves four
     // nodes.  Other sets: one warp per node, a table of all velocities.
     const bool vec4 = (QX2 & 3) == 0 && (QX2 & (QX2 - 1)) == 0 && QX2 <= 32 && V >= 32;
-    auto store = [&](int node, R a0, R a1, R a2, R a3, R a4, R c0, R c1, R c2, R c3, R c4) {
-        R* o = sums + (size_t)node * kSumStride;
+    auto store = [&](int node, float a0, float a1, float a2, float a3, float a4, float c0, float c1, float c2, float c3, float c4) {
+        float* o = sums + (size_t)node * kSumStride;
         o[0] = a0; o[1] = a1; o[2] = a2; o[3] = a3; o[4] = a4;
         o[8] = c0; o[9] = c1; o[10] = c2; o[11] = c3; o[12] = c4;
     };
@@ -72,20 +69,20 @@ __global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __
         const int sl = lane & 7;
         const int x0 = (4 * sl) % QX2;
         const int lg = __ffs(QX2) - 1;                   // 2Qx = 2^lg
-        const R pxa = sM[x0].x, pxb = sM[x0 + 1].x, pxc = sM[x0 + 2].x, pxd = sM[x0 + 3].x;
+        const float pxa = sM[x0].x, pxb = sM[x0 + 1].x, pxc = sM[x0 + 2].x, pxd = sM[x0 + 3].x;
         for (int nb = (blockIdx.x * nw + warp) * 4; nb < g.nnodes; nb += gridDim.x * nw * 4) {
             const int node = nb + (lane >> 3);
             // compensated per-lane sums (FP32 states)
-            R a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0, c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
+            float a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0, c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
             if (node < g.nnodes) {
                 const int ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0;
                 const InstDev& I = g.inst[ii];
-                const R4* f4 = reinterpret_cast<const R4*>(fs + (size_t)I.f_off + (size_t)(node - I.node_off) * V);
+                const float4* f4 = reinterpret_cast<const float4*>(fs + (size_t)I.f_off + (size_t)(node - I.node_off) * V);
 #pragma unroll 4
                 for (int q = sl; q < (V >> 2); q += 8) {
-                    const R4 x = f4[q];
-                    const R4 yz = sYZ[(q << 2) >> lg];
-                    const R sq = (x.x + x.y) + (x.z + x.w);
+                    const float4 x = f4[q];
+                    const float4 yz = sYZ[(q << 2) >> lg];
+                    const float sq = (x.x + x.y) + (x.z + x.w);
                     csum_add(a0, c0, sq);
                     csum_add(a1, c1, pxa * x.x + pxb * x.y + pxc * x.z + pxd * x.w);
                     csum_add(a2, c2, yz.x * sq);
@@ -94,10 +91,10 @@ __global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __
                 }
             }
             // compensated tree over the eight lanes of each node
-            auto tree8 = [](R& sa, R& ca) {
+            auto tree8 = [](float& sa, float& ca) {
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) {
-                    const R s2 = __shfl_xor_sync(0xffffffffu, sa, o), c2 = __shfl_xor_sync(0xffffffffu, ca, o);
+                    const float s2 = __shfl_xor_sync(0xffffffffu, sa, o), c2 = __shfl_xor_sync(0xffffffffu, ca, o);
                     csum_add(sa, ca, s2);
                     ca += c2;
                 }
@@ -110,12 +107,12 @@ __global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __
     for (int node = blockIdx.x * nw + warp; node < g.nnodes; node += gridDim.x * nw) {
         const int ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0;
         const InstDev& I = g.inst[ii];
-        const R* f = fs + (size_t)I.f_off + (size_t)(node - I.node_off) * V;
+        const float* f = fs + (size_t)I.f_off + (size_t)(node - I.node_off) * V;
         // compensated per-lane sums (FP32 states), compensated warp tree
-        R a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0, c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
+        float a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0, c0 = 0, c1 = 0, c2 = 0, c3 = 0, c4 = 0;
         for (int v = lane; v < V; v += 32) {
-            const R val = f[v];
-            const R4 mw = sM[v];
+            const float val = f[v];
+            const float4 mw = sM[v];
             csum_add(a0, c0, val);
             csum_add(a1, c1, mw.x * val);
             csum_add(a2, c2, mw.y * val);
@@ -127,8 +124,7 @@ __global__ void __launch_bounds__(256) sums_kernel(const GroupDev g, const R* __
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __restrict__ sums) {
+__global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const float* __restrict__ sums) {
     extern __shared__ __align__(16) double csm[];
     const int Nx = g.Nx, Ny = g.Ny, Nz = g.Nz;
     const int nrec = 5 * Nx + 1;
@@ -162,7 +158,7 @@ __global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __r
     const float2* sTxF = sTF;
     const float2* sTyF = sTxF + g.Qx * (Nx + 1);
     const float2* sTzF = sTyF + VY * (Ny + 1);
-    R* coef = static_cast<R*>(g.coef);
+    float* coef = static_cast<float*>(g.coef);
     const int nf = QX2 + VY + VZ;
     const int nbatches = (g.nnodes + 31) / 32;
     for (int bt = blockIdx.x * nw + warp; bt < nbatches; bt += gridDim.x * nw) {
@@ -174,7 +170,7 @@ __global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __r
             const int node = base + lane;
             const int ii = g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0;
             const double inv_Kn = g.inst[ii].inv_Kn;
-            const R* sm = sums + (size_t)node * kSumStride;
+            const float* sm = sums + (size_t)node * kSumStride;
             active = inv_Kn != 0.0;
             // n, u, T in FP64 from the compensated sums (one division)
             const double n = (double)sm[0] + (double)sm[8], in = 1.0 / n;
@@ -201,8 +197,8 @@ __global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __r
         //    so that the lanes of a warp follow the same path
         for (int t = lane; t < nb * QX2; t += 32) {          // n g_x
             const int k = t / QX2, o = t - k * QX2;
-            R* line = coef + (size_t)(base + k) * g.ncp;
-            if (sNT[2 * k + 1] == 0.0) { line[o] = R(0); continue; }
+            float* line = coef + (size_t)(base + k) * g.ncp;
+            if (sNT[2 * k + 1] == 0.0) { line[o] = 0.0f; continue; }
             const int kk = o % g.Qx, sg = o / g.Qx;
             if (df) {
                 const float2* Gs = sGF + k * ncoef + sg * (Nx + 1);
@@ -210,61 +206,61 @@ __global__ void __launch_bounds__(32) coef_kernel(const GroupDev g, const R* __r
                 float2 acc = df_mul(Tr[0], Gs[0]);
                 for (int l = 1; l <= Nx; ++l) acc = df_add(acc, df_mul(Tr[l], Gs[l]));
                 acc = df_mul(acc, sIn[k].n);
-                line[o] = (R)(acc.x + acc.y);
+                line[o] = acc.x + acc.y;
             } else {
                 const double* Gs = sG + k * ncoef + sg * (Nx + 1);
                 const double* Tr = sTx + kk * (Nx + 1);
                 double acc = 0.0;
                 for (int l = 0; l <= Nx; ++l) acc += Tr[l] * Gs[l];
-                line[o] = (R)(acc * sNT[2 * k]);
+                line[o] = (float)(acc * sNT[2 * k]);
             }
         }
         for (int t = lane; t < nb * VY; t += 32) {           // g_y
             const int k = t / VY, j = t - k * VY;
-            R* line = coef + (size_t)(base + k) * g.ncp + QX2;
-            if (sNT[2 * k + 1] == 0.0) { line[j] = R(0); continue; }
-            if (!g.Qy) { line[j] = R(1); continue; }
+            float* line = coef + (size_t)(base + k) * g.ncp + QX2;
+            if (sNT[2 * k + 1] == 0.0) { line[j] = 0.0f; continue; }
+            if (!g.Qy) { line[j] = 1.0f; continue; }
             if (df) {
                 const float2* Gy = sGF + k * ncoef + 2 * (Nx + 1);
                 const float2* Tr = sTyF + j * (Ny + 1);
                 float2 acc = df_mul(Tr[0], Gy[0]);
                 for (int l = 1; l <= Ny; ++l) acc = df_add(acc, df_mul(Tr[l], Gy[l]));
-                line[j] = (R)(acc.x + acc.y);
+                line[j] = acc.x + acc.y;
             } else {
                 const double* Gy = sG + k * ncoef + 2 * (Nx + 1);
                 const double* Tr = sTy + j * (Ny + 1);
                 double acc = 0.0;
                 for (int l = 0; l <= Ny; ++l) acc += Tr[l] * Gy[l];
-                line[j] = (R)acc;
+                line[j] = (float)acc;
             }
         }
         for (int t = lane; t < nb * VZ; t += 32) {           // g_z
             const int k = t / VZ, j = t - k * VZ;
-            R* line = coef + (size_t)(base + k) * g.ncp + QX2 + VY;
-            if (sNT[2 * k + 1] == 0.0) { line[j] = R(0); continue; }
-            if (!g.Qz) { line[j] = R(1); continue; }
+            float* line = coef + (size_t)(base + k) * g.ncp + QX2 + VY;
+            if (sNT[2 * k + 1] == 0.0) { line[j] = 0.0f; continue; }
+            if (!g.Qz) { line[j] = 1.0f; continue; }
             if (df) {
                 const float2* Gz = sGF + k * ncoef + 2 * (Nx + 1) + (Ny + 1);
                 const float2* Tr = sTzF + j * (Nz + 1);
                 float2 acc = df_mul(Tr[0], Gz[0]);
                 for (int l = 1; l <= Nz; ++l) acc = df_add(acc, df_mul(Tr[l], Gz[l]));
-                line[j] = (R)(acc.x + acc.y);
+                line[j] = acc.x + acc.y;
             } else {
                 const double* Gz = sG + k * ncoef + 2 * (Nx + 1) + (Ny + 1);
                 const double* Tr = sTz + j * (Nz + 1);
                 double acc = 0.0;
                 for (int l = 0; l <= Nz; ++l) acc += Tr[l] * Gz[l];
-                line[j] = (R)acc;
+                line[j] = (float)acc;
             }
         }
-        if (lane < nb) coef[(size_t)(base + lane) * g.ncp + nf] = (R)sNT[2 * lane + 1];   // 1/tau
+        if (lane < nb) coef[(size_t)(base + lane) * g.ncp + nf] = (float)sNT[2 * lane + 1];   // 1/tau
         if (g.has_field && lane < nb) {              // a = a_uniform + a_field(node)
             const int node = base + lane;
             const InstDev& I = g.inst[g.ninst > 1 ? find_slot(g.node_start, g.ninst, node) : 0];
-            R* fl = coef + (size_t)node * g.ncp + g.field_off;
-            fl[0] = (R)(I.ax + g.afield[3 * (size_t)node]);
-            fl[1] = (R)(I.ay + g.afield[3 * (size_t)node + 1]);
-            fl[2] = (R)(I.az + g.afield[3 * (size_t)node + 2]);
+            float* fl = coef + (size_t)node * g.ncp + g.field_off;
+            fl[0] = (float)(I.ax + g.afield[3 * (size_t)node]);
+            fl[1] = (float)(I.ay + g.afield[3 * (size_t)node + 1]);
+            fl[2] = (float)(I.az + g.afield[3 * (size_t)node + 2]);
         }
         __syncwarp();
     }
@@ -749,7 +745,7 @@ __global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, co
 }  // namespace
 
 cudaError_t prepare_node() {
-    cudaError_t e = cudaFuncSetAttribute(coef_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(coef_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(coef_df_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
@@ -757,7 +753,7 @@ cudaError_t prepare_node() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(coef_df_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(sums_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    return cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
 }
 
 int sm_count() {
@@ -800,9 +796,12 @@ cudaError_t launch_df_special(const double* z, int n, double* erf_out, double* e
 }
 
 // Whether the one-launch node pass (sums, factor lines and walls) takes this
-// FP32 group: rows of 8, 16 or 32 p_x values, the double-float lines.
+// FP32 group: rows of 8, 16 or 32 p_x values, the double-float lines, within the 48 KB
+// of shared memory that a launch has without asking (the sets that march need
+// 43.5 KB at most).
 bool node_fused_available(int precision, const GroupDev& g) {
-    return precision != HLB_FP64_ && g.use_df && max(g.Nx, max(g.Ny, g.Nz)) < 16 && (g.QX2 == 8 || g.QX2 == 16 || g.QX2 == 32);
+    return precision != HLB_FP64_ && g.use_df && max(g.Nx, max(g.Ny, g.Nz)) < 16 && (g.QX2 == 8 || g.QX2 == 16 || g.QX2 == 32) &&
+           node_smem<32>(g).bytes <= 47 * 1024;
 }
 
 // Nodes per CTA of the one-launch node pass.  With rows of 32 values (the longest
@@ -814,33 +813,19 @@ bool node_fused_available(int precision, const GroupDev& g) {
 static int node_nb(const GroupDev& g) { return g.QX2 == 32 && g.nnodes <= 64 * sm_count() ? 8 : 32; }
 
 template <int ADV, int LOWN>
-static cudaError_t node_df_launch(const GroupDev& g, const float* fs, cudaStream_t st, bool prepare) {
+static void node_df_launch(const GroupDev& g, const float* fs, cudaStream_t st) {
     const int NB = node_nb(g);
     const size_t smem = NB == 8 ? node_smem<8>(g).bytes : node_smem<32>(g).bytes;
-    if (prepare) {
-        // needed only above the 48 KB that a launch has without asking (setting
-        // an attribute loads the kernel, which a handle's creation would wait for)
-        if (smem <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(NB == 8 ? (const void*)node_df_kernel<ADV, LOWN, 8> : (const void*)node_df_kernel<ADV, LOWN, 32>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    }
     const int grid = g.nrows * g.wchunks + (g.nnodes + NB - 1) / NB;
     if (NB == 8) launch_dependent(g.pdl, node_df_kernel<ADV, LOWN, 8>, grid, kNodeT, smem, st, g, fs);
     else launch_dependent(g.pdl, node_df_kernel<ADV, LOWN, 32>, grid, kNodeT, smem, st, g, fs);
-    return cudaSuccess;
 }
-
-static cudaError_t node_df_dispatch(int adv, const GroupDev& g, const float* fs, cudaStream_t st, bool prepare) {
-    const bool low = g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12;
-    if (adv == HLB_WENO5_)
-        return low ? node_df_launch<HLB_WENO5_, 1>(g, fs, st, prepare) : node_df_launch<HLB_WENO5_, 0>(g, fs, st, prepare);
-    return low ? node_df_launch<HLB_UPWIND2_, 1>(g, fs, st, prepare) : node_df_launch<HLB_UPWIND2_, 0>(g, fs, st, prepare);
-}
-
-cudaError_t prepare_node_fused(int adv, const GroupDev& g) { return node_df_dispatch(adv, g, nullptr, nullptr, true); }
 
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
-    node_df_dispatch(adv, g, static_cast<const float*>(fs), st, false);
+    const bool low = g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12;
+    const float* f = static_cast<const float*>(fs);
+    if (adv == HLB_WENO5_) low ? node_df_launch<HLB_WENO5_, 1>(g, f, st) : node_df_launch<HLB_WENO5_, 0>(g, f, st);
+    else low ? node_df_launch<HLB_UPWIND2_, 1>(g, f, st) : node_df_launch<HLB_UPWIND2_, 0>(g, f, st);
 }
 
 // The FP64 node pass and walls (every FP64 group).
@@ -863,9 +848,9 @@ void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st
 // node's slot of g.sums), then the factor lines.
 void launch_node(const GroupDev& g, const void* fs, cudaStream_t st) {
     const size_t smem_a = 4 * (g.V + g.VY * g.VZ) * sizeof(float);
-    const int blocks_a = one_wave(reinterpret_cast<const void*>(&sums_kernel<float>), 256, smem_a, (g.nnodes + 7) / 8);
+    const int blocks_a = one_wave(reinterpret_cast<const void*>(&sums_kernel), 256, smem_a, (g.nnodes + 7) / 8);
     const int nrec = 5 * g.Nx + 1;
-    sums_kernel<float><<<blocks_a, 256, smem_a, st>>>(g, (const float*)fs, (float*)g.sums);
+    sums_kernel<<<blocks_a, 256, smem_a, st>>>(g, (const float*)fs, (float*)g.sums);
     const int nmax = max(g.Nx, max(g.Ny, g.Nz));
     if (g.use_df && nmax < 16) {
         const int nP = (g.Qx + 1) / 2 * (g.Nx + 1) + (g.VY + 1) / 2 * (g.Ny + 1) + (g.VZ + 1) / 2 * (g.Nz + 1);
@@ -878,7 +863,7 @@ void launch_node(const GroupDev& g, const void* fs, cudaStream_t st) {
         const int nT = g.Qx * (g.Nx + 1) + g.VY * (g.Ny + 1) + g.VZ * (g.Nz + 1);
         const int ncoef = 2 * (g.Nx + 1) + (g.Ny + 1) + (g.Nz + 1);
         const size_t smem_b = 8 * (nrec + nT) + 8 * (32 * ncoef + 64) + 32 * sizeof(NodeDF);
-        coef_kernel<float><<<(g.nnodes + 31) / 32, 32, smem_b, st>>>(g, (const float*)g.sums);
+        coef_kernel<<<(g.nnodes + 31) / 32, 32, smem_b, st>>>(g, (const float*)g.sums);
     }
 }
 
