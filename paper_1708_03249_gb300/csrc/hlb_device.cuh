@@ -614,8 +614,9 @@ __device__ __forceinline__ float wall_ghost2(float f0, float f1, float f2) {
 
 // Fluxes per unit velocity at NF consecutive faces, two independent rows at
 // once: face f lies between c[f + 2] and c[f + 3] of c[0 .. NF + 4] (cells in
-// ascending order), upwind for a positive (pos) or negative velocity.
-template <int ADV, int NF>
+// ascending order), upwind for a positive (pos) or negative velocity.  UNIFORM:
+// pos is the same over a warp, so that a branch beats the selects (upwind2).
+template <int ADV, int NF, bool UNIFORM = false>
 __device__ __forceinline__ void packed_faces(bool pos, const float2* c, float2* F) {
     if (ADV == HLB_WENO5_) {
         float2 u[NF + 4], r[NF];           // in upwind order
@@ -631,6 +632,14 @@ __device__ __forceinline__ void packed_faces(bool pos, const float2* c, float2* 
             weno5_faces2<NF>(u, r);
 #pragma unroll
             for (int f = 0; f < NF; ++f) F[f] = r[NF - 1 - f];
+        }
+    } else if (UNIFORM) {
+        if (pos) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) F[f] = upwind2_face2(c[f + 1], c[f + 2]);
+        } else {
+#pragma unroll
+            for (int f = 0; f < NF; ++f) F[f] = upwind2_face2(c[f + 4], c[f + 3]);
         }
     } else {
 #pragma unroll

@@ -155,15 +155,17 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
     // Copy `lane` of pair p (22 lanes: 12 halo rows, 4 head rows, 4 f^n rows,
     // 2 factor-line runs): source, bytes and destination in B; false if the
     // lane has none for this pair.
-    // Slabs of up to four warps take turns: pair p's copies are issued by warp p %
-    // (S / 32), so that each warp runs the issue code once in that many pairs
+    // One warp, or four with WENO-5, take turns: pair p's copies are issued by warp
+    // p % (S / 32), so that each warp runs the issue code once in that many pairs
     // (large channel, 16 x 8 slabs: 2.90 against 2.92 ms per stage with the
-    // copies spread over the warps).  With 16 warps the spread is the better one
-    // (32 x 16 slabs of the 256^2 box: 296 against 298 us): warps 0 and 1 take the
-    // halo rows of cells x0 and x0+1, warp 2 the head rows and factor lines, warp
-    // 3 the f^n rows.  Thread 0 registers each pair's byte count
+    // copies spread over the warps).  With upwind2, whose few instructions leave
+    // the issuing warp behind the others, and with 16 warps the spread is the
+    // better one (large channel, upwind2: 2.07 against 2.31 ms; 32 x 16 slabs of
+    // the 256^2 box: 296 against 298 us): warps 0 and 1 take the halo rows of
+    // cells x0 and x0+1, warp 2 the head rows and factor lines, warp 3 the f^n
+    // rows.  Thread 0 registers each pair's byte count
     // (arrive.expect_tx) before any warp can issue that pair's copies.
-    constexpr bool kTurns = S / 32 <= 4;
+    constexpr bool kTurns = S / 32 < 4 || (S / 32 == 4 && ADV == HLB_WENO5_);
     int my_copy = -1;
     if (kTurns) {
         my_copy = lane < 22 ? lane : -1;
@@ -344,7 +346,7 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
 #pragma unroll
         for (int k = 0; k < 3; ++k) col[5 + k] = __fmul2_rn(make_float2(B.halo[0][3 + k][vl], B.halo[1][3 + k][vl]), sv2);
         float2 Gy[3];
-        packed_faces<ADV, 3>(ypos, col, Gy);
+        packed_faces<ADV, 3, (32 / QX2 <= VY / 2)>(ypos, col, Gy);      // a warp's rows lie on one side of p_y = 0
         const float2 dy0 = __fmul2_rn(vys, fsub2(Gy[1], Gy[0]));   // row y0, cells x0, x0+1
         const float2 dy1 = __fmul2_rn(vys, fsub2(Gy[2], Gy[1]));   // row y0+1
         // shift the window by two cells
