@@ -719,7 +719,8 @@ hlb_status build_group(hlb_handle* h, Group& G) {
     // there (hlb_launch_count), not for speed.  us per step, one launch against
     // the three (GB300): 60 nodes of 32 velocities 36 / 69, 240 nodes 38 / 71, 1023
     // nodes 39 / 70; of 512 velocities 58 / 169, 69 / 178, 91 / 174.
-    G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && (G.TY == 1 || G.nnodes > 256);
+    G.node_fused = G.march_ok && hlb::node_fused_available(G.precision, G.dev) && hlb::node_fused_pays(G.dev) &&
+                   (G.TY == 1 || G.nnodes > 256);
     if (G.march_ok && G.precision == HLB_FP32 && !G.node_fused) HLB_CUDA(hlb::prepare_node());
 
     // launch shape of the stage kernel.  With Kx in global memory each

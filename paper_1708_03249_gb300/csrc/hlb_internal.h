@@ -196,6 +196,7 @@ void gauss_legendre_rule(int n, std::vector<double>& x, std::vector<double>& w);
 void launch_node(const GroupDev& g, const void* fs, cudaStream_t st);
 // The node pass and the walls in one launch, for the FP32 groups it takes.
 bool node_fused_available(int precision, const GroupDev& g);
+bool node_fused_pays(const GroupDev& g);
 int sm_count();          // of the current device when first called (152 if it cannot be asked)
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st);
 void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st);

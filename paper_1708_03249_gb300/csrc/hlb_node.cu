@@ -18,7 +18,7 @@ namespace {
 // ---------------------------------------------------------------------------
 // node kernels of the FP32 groups that node_df_kernel does not take (orders
 // above 15, rows that are not 8, 16 or 32 values, 2D groups of at most 256
-// nodes)
+// nodes, large groups of few velocities (node_fused_pays))
 // ---------------------------------------------------------------------------
 // Per-node equilibrium factors, in two passes with no block-wide barrier:
 //   sums_kernel   streams the stage input once (one warp per node) and writes
@@ -812,6 +812,22 @@ bool node_fused_available(int precision, const GroupDev& g) {
 // 171 / 183, 19456 379 / 347; order 8: 1216 nodes 38.5 / 36.8, 4864 46.5 / 45.2.
 static int node_nb(const GroupDev& g) { return g.QX2 == 32 && g.nnodes <= 64 * sm_count() ? 8 : 32; }
 
+// Orders at which the recurrences' start is in double-float too (LOWN).
+static bool node_low_order(const GroupDev& g) { return g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12; }
+
+// Whether the one-launch node pass is the faster one for a group that it can
+// take.  It hides the sums' latency behind the lines and saves two launches; the
+// separate kernels form the lines of 128 nodes per table load.  With few values
+// per node the lines are the work and the launches are nothing in a large group.
+// us per step, one launch against three (GB300): 32 x 1 velocities, order 7, 60000
+// nodes 129 / 157, 130000 301 / 295, 400000 862 / 754, 3000000 6151 / 4852; order 15,
+// 400000 1062 / 1157, 3000000 7593 / 7118; 16 x 8 velocities 400000 nodes 1192 /
+// 1208, 3000000 8542 / 8275; 8 x 4 407 / 437 at 300000, 3675 / 3616 at 3000000; from
+// 512 velocities on equal or faster at every size (16 x 8 x 8, 1000000 nodes, 15709 / 16013).
+bool node_fused_pays(const GroupDev& g) {
+    return g.V >= 512 || g.nnodes <= (g.QX2 == 32 && node_low_order(g) ? 1 << 17 : 1 << 19);
+}
+
 template <int ADV, int LOWN>
 static void node_df_launch(const GroupDev& g, const float* fs, cudaStream_t st) {
     const int NB = node_nb(g);
@@ -822,7 +838,7 @@ static void node_df_launch(const GroupDev& g, const float* fs, cudaStream_t st) 
 }
 
 void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
-    const bool low = g.Nx <= HLB_DF_SPECIAL_MAX_N && max(g.Ny, g.Nz) < 12;
+    const bool low = node_low_order(g);
     const float* f = static_cast<const float*>(fs);
     if (adv == HLB_WENO5_) low ? node_df_launch<HLB_WENO5_, 1>(g, f, st) : node_df_launch<HLB_WENO5_, 0>(g, f, st);
     else low ? node_df_launch<HLB_UPWIND2_, 1>(g, f, st) : node_df_launch<HLB_UPWIND2_, 0>(g, f, st);
