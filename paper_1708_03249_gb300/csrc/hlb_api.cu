@@ -122,7 +122,7 @@ struct Group {
     // items of a stage (per instance its node chunks, then its segments),
     // node chunks and segments per instance, resident CTAs
     bool persist_ok = false;
-    bool pdl = false;                        // dependent launches (a handle's only group, not a large one)
+    bool pdl = false;                        // dependent launches (dependent_pays)
     bool node_fused = false;                 // the node pass and the walls in one launch
     bool persist_auto = false;               // steps with it unless told otherwise (hlb_set_persistent)
     bool persist_use = true;                 // the autotuner's pick: persistent or per-stage launches
@@ -378,11 +378,35 @@ std::vector<hlb::Work> segment_list(const hlb_handle* h, const Group& G, int SX)
     return works;
 }
 
+// Whether the kernels of a step of group G are launched as dependents
+// (launch_dependent), which hides their launch and set-up.  The waiting CTAs hold
+// registers and shared memory, and the scheduler places them unevenly beside the
+// running ones: that costs more than it hides
+// - with several groups stepping side by side (37 channels in three groups 135
+//   against 123 us per step), and in a large group, where the launch is nothing
+//   (1024 x 512 x 1024 velocities 10.28 against 10.19 ms);
+// - in FP64, whose pipe two CTAs on one SM share, unless there are at most half
+//   as many marching CTAs as SMs, one CTA fits an SM, or a 1D group is large;
+// - with two FP32 CTAs per SM, in about one wave of segments that are not the shortest.
+// us per step, dependent against ordinary launches (GB300): FP64, 64 cells of 32
+// velocities 39 / 45, 100 cells of 512 173 / 199, 22000 of 32 308 / 315, but 2000 of 32
+// 74 / 56 and 50 x 50 of 32 105 / 74; FP32, 512 cells of 128 31 / 39, 60 x 40 of 32
+// 34 / 45, 317 x 203 of 128 260 / 271, the 256^2 box 1090 / 1109, but 100 x 100 cells of
+// 512 243 / 215, where 60 x 40 takes 82 / 90.
+bool dependent_pays(const hlb_handle* h, const Group& G, int nsm) {
+    if (h->groups.size() != 1 || G.nvalues > (1LL << 27)) return false;
+    const int per = hlb::march_ctas_per_sm(G.precision, G.QX2 * G.VY, G.TY);
+    if (G.precision == HLB_FP64) return G.TY == 1 && (per == 1 || 2 * G.nworks <= nsm || G.nnodes >= 10000);
+    return !(per == 2 && G.SX >= 8 && 10LL * G.nworks >= 19LL * nsm && 10LL * G.nworks <= 26LL * nsm);
+}
+
 // The per-stage marching launch's work list (one CTA per item).
 hlb_status set_segments(hlb_handle* h, Group& G, int SX) {
     G.SX = SX;
     const std::vector<hlb::Work> works = segment_list(h, G, SX);
     G.nworks = (int)works.size();
+    G.pdl = dependent_pays(h, G, hlb::sm_count());
+    G.dev.pdl = G.pdl ? 1 : 0;
     return upload(G.d_works, works);
 }
 
@@ -1008,15 +1032,6 @@ hlb_status hlb_create(const hlb_config* cfg, int ninst, void* cuda_stream, hlb_h
     for (auto& G : h->groups) {
         hlb_status s = build_group(h.get(), *G);
         if (s != HLB_OK) return s;
-        // Dependent launches hide the launch and set-up of a stage's kernels.  A
-        // waiting CTA holds its registers and shared memory: with several groups
-        // stepping side by side that costs more than it hides (37 channels in
-        // three groups 135 against 123 us per step), and in a large group the
-        // launch is nothing (1024 x 512 x 1024 velocities 10.28 against 10.19 ms);
-        // 64 cells of the FP64 channel take 48.2 against 51.3 us, 512 of the
-        // stretched one 31.3 against 39, the 256^2 box 1097 against 1114 (GB300).
-        G->pdl = h->groups.size() == 1 && G->nvalues <= (1LL << 27) && !G->npairs;
-        G->dev.pdl = G->pdl ? 1 : 0;
     }
     h->inst_node_off.resize(ninst);
     h->inst_value_off.resize(ninst);

@@ -13,9 +13,13 @@ constexpr double kSqrt2Pi = 2.5066282746310005024157652848110;
 
 // Programmatic dependent launch (launch_dependent, hlb_internal.h): a stage's
 // kernels follow one another in a stream, and each one's launch and set-up can
-// run while the one before it drains.  pdl_trigger lets the next kernel's CTAs
-// start once every CTA of this one has; pdl_wait returns when the kernels before
-// this one are complete and their writes visible, at once in an ordinary launch.
+// run while the one before it drains.  pdl_wait returns when the kernels before
+// this one are complete and their writes visible, at once in an ordinary launch;
+// pdl_trigger lets the next kernel's CTAs start once every CTA of this one has
+// called it.  It stands after the wait: one kernel waits behind the one that runs,
+// where a trigger at the start let whole steps pile up, whose waiting CTAs hold
+// the slots and leave the running kernel's unevenly placed (500 cells of 128 FP64
+// velocities 155 against 87 us per step, 5000 cells of 32 FP32 ones 32.8 against 28.2).
 // Nothing that an earlier kernel of the step writes may be read, and nothing in
 // global memory written, before pdl_wait.  (State pointers of such kernels are not
 // __restrict__: loads through them would count as invariant and could be

@@ -54,7 +54,6 @@ template <int ADV, int QX2, int VY, int FM, int FF, int SR = 0>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? 8 : (QX2 * VY <= 256 ? 4 : 2))))
 march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs,
               const float* fn, float* fo, int stage) {
-    pdl_trigger();
     constexpr int S = QX2 * VY;
     static_assert(S % 32 == 0, "the exchange barrier counts whole warps");
     constexpr int QX = QX2 / 2;
@@ -173,6 +172,7 @@ march1_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs,
     }
     __syncthreads();
     pdl_wait();                                             // from here on: the state, the walls, the factor lines
+    pdl_trigger();
     for (int p = 0; p < kLineDepth - 1; ++p) issue(p);
     const float nwl = (float)g.nw[(size_t)(I.row_off + row) * 2 + 0] * gwl;        // scaled emitted ghosts
     const float nwr = (float)g.nw[(size_t)(I.row_off + row) * 2 + 1] * gwr;

@@ -71,7 +71,6 @@ constexpr size_t march_smem_bytes() {
 template <typename R, int ADV, int QX2, int VY, int TY>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? (TY > 1 ? 3 : 4) : 1)))
 march_kernel(const GroupDev g, const Work* __restrict__ works, const R* fs, const R* fn, R* fo, int stage) {
-    pdl_trigger();
     constexpr int S = QX2 * VY;
     constexpr int QX = QX2 / 2;
     using Buf = StepBuf<R, QX2, VY, TY>;
@@ -159,6 +158,7 @@ march_kernel(const GroupDev g, const Work* __restrict__ works, const R* fs, cons
     }
     __syncthreads();
     pdl_wait();                                  // from here on: the state, the walls, the factor lines
+    pdl_trigger();
     if (t == 0)
         for (int xs = xa; xs < xa + kDepth - 1; ++xs) issue(xs);
 #pragma unroll

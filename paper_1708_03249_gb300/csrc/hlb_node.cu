@@ -437,10 +437,10 @@ __device__ __forceinline__ void node_sums(const float* fs, const float* __restri
 template <int ADV, int LOWN, int NB>
 __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const GroupDev g, const float* fs) {
     extern __shared__ __align__(16) unsigned char nsm[];
-    pdl_trigger();
     const int nwall = g.nrows * g.wchunks;
     if ((int)blockIdx.x < nwall) {
         pdl_wait();
+        pdl_trigger();
         wall_block<float, ADV>(g, fs, blockIdx.x, reinterpret_cast<double*>(nsm));
         return;
     }
@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
         sOff[tid] = g.inst[ii].f_off + (long long)(base + tid - g.inst[ii].node_off) * V;
     }
     pdl_wait();
+    pdl_trigger();
     __syncthreads();
     // 1. moment sums: 2Qx / 4 lanes per node, so that a lane's p_x never change
     // and step r of its loop is the row r of (jy, kz)
@@ -578,12 +579,12 @@ __device__ __forceinline__ void half_range_coefficients(const GroupDev& g, int r
 
 template <int ADV, int NB>
 __global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, const double* fs) {
-    pdl_trigger();
     extern __shared__ __align__(16) double dsm[];
     constexpr int LPN = kNode64T / NB;                        // lanes per node
     const int nwall = g.nrows * g.wchunks;
     if ((int)blockIdx.x < nwall) {
         pdl_wait();
+        pdl_trigger();
         wall_block<double, ADV>(g, fs, blockIdx.x, dsm);
         return;
     }
@@ -606,6 +607,7 @@ __global__ void __launch_bounds__(kNode64T) node_f64_kernel(const GroupDev g, co
         sRow[3 * r + 2] = py * py + pz * pz;
     }
     pdl_wait();
+    pdl_trigger();
     __syncthreads();
     // 1. moments: each lane its own p_x, weighted once per column
     {

@@ -64,7 +64,6 @@ template <int ADV, int QX2, int VY, int FM, int FF, int SR = 0>
 __global__ void __launch_bounds__(QX2 * VY, (QX2 * VY <= 32 ? 16 : (QX2 * VY <= 128 ? HLB_PAIR_MIN_BLOCKS : 2)))
 march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float* fs, const float* fn, float* fo,
                   int stage) {
-    pdl_trigger();
     constexpr int S = QX2 * VY;
     constexpr int QX = QX2 / 2;
     constexpr int SP = QX2 + 1;            // padded sF row: the K_x reads of a warp hit distinct banks
@@ -241,6 +240,7 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
     }
     __syncthreads();
     pdl_wait();                        // from here on: the state, the walls, the factor lines
+    pdl_trigger();
     for (int p = 0; p < kPairDepth - 1; ++p) issue(p);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
