@@ -655,7 +655,14 @@ hlb_status build_group(hlb_handle* h, Group& G) {
             const hlb_config& c = h->cfg[G.members[m]];
             if ((long long)c.nx * c.ny * G.V >= (1LL << 31) - (long long)G.V * 8) big = true;
         }
-        G.march_ok = !small_ny && !big && hlb::march_available(G.precision, G.adv, G.QX2, G.VY, G.TY);
+        // FP64 groups in 2D of at most 2^16 values keep the generic kernel, whose many
+        // small CTAs fill the SMs where the strips of two rows leave most of them
+        // idle.  us per step, generic against marching (GB300): 32 x 32 cells of 32
+        // velocities 54 / 61 (upwind2), 84 / 110 (WENO-5), without collisions 33 / 41
+        // and 67 / 94; 15 x 20 of 128 69 / 77, 103 / 129, 46 / 55, 84 / 111; but 60 x 40 of
+        // 32 76 / 72, 140 / 124, 43 / 44, 113 / 101 and 32 x 32 of 128 117 / 95, 241 / 197.
+        const bool few = G.precision == HLB_FP64 && two_d && G.nvalues <= (1LL << 16);
+        G.march_ok = !small_ny && !big && !few && hlb::march_available(G.precision, G.adv, G.QX2, G.VY, G.TY);
         if (G.march_ok) {
             // Segment length from N = cells per resident CTA (strips of TY
             // rows; CTAs per SM as compiled).  Small problems: one wave of the
