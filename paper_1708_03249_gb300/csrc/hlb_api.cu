@@ -396,7 +396,7 @@ std::vector<hlb::Work> segment_list(const hlb_handle* h, const Group& G, int SX)
 bool dependent_pays(const hlb_handle* h, const Group& G, int nsm) {
     if (h->groups.size() != 1 || G.nvalues > (1LL << 27)) return false;
     const int per = hlb::march_ctas_per_sm(G.precision, G.QX2 * G.VY, G.TY);
-    if (G.precision == HLB_FP64) return G.TY == 1 && (per == 1 || 2 * G.nworks <= nsm || G.nnodes >= 10000);
+    if (G.precision == HLB_FP64) return G.TY == 1 && (per == 1 || 2 * G.nworks <= nsm || G.nnodes >= 16384);
     return !(per == 2 && G.SX >= 8 && 10LL * G.nworks >= 19LL * nsm && 10LL * G.nworks <= 26LL * nsm);
 }
 

@@ -526,11 +526,15 @@ __global__ void __launch_bounds__(kNodeT, LOWN ? 8 : 7) node_df_kernel(const Gro
 // small group waits on one thread's chain and a large one on the pipe: the
 // roles of the recurrences run in different threads (p_x in warp 0, p_y and
 // p_z in warp 1), the dot products over the whole CTA; one node per CTA where
-// that leaves at most two CTAs per SM, eight otherwise.  Per
+// that leaves at most two CTAs per SM, sixteen, whose recurrences and short rows
+// fill the lanes of a warp, in groups of more than 16 nodes per SM, eight
+// between and in the order-200 sets, whose long rows want the lanes.  Per
 // stage (GB300): 5795 nodes of 128 velocities 30 us; 72 nodes of 400 velocities,
 // order 20, 14.7 us with one node per CTA, 47 with eight; the 64 nodes of the
 // FP64 channel (moments, lines and walls in three kernels before) take 9 of the
-// 17 us that a stage is now.
+// 17 us that a stage is now.  Sixteen against eight: 100000 nodes of 32 velocities
+// 158 / 277 us, of 128 259 / 371, 5000 of 32 19 / 24; 1200 of 128 18.5 / 16.7; 2400 of
+// order 200 463 / 423 (with the quadrature).
 // ---------------------------------------------------------------------------
 constexpr int kNode64T = 128;
 
@@ -847,18 +851,23 @@ void launch_node_fused(int adv, const GroupDev& g, const void* fs, cudaStream_t 
 }
 
 // The FP64 node pass and walls (every FP64 group).
-void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
-    const int NB = g.nnodes <= 2 * sm_count() ? 1 : 8;
+template <int ADV, int NB>
+static void node_f64_launch(const GroupDev& g, const double* fs, cudaStream_t st) {
     const int grid = g.nrows * g.wchunks + (g.nnodes + NB - 1) / NB;
-    const size_t smem = node64_smem(g, NB);
+    launch_dependent(g.pdl, node_f64_kernel<ADV, NB>, grid, kNode64T, node64_smem(g, NB), st, g, fs);
+}
+
+template <int ADV>
+static void node_f64_dispatch(const GroupDev& g, const double* fs, cudaStream_t st) {
+    if (g.nnodes <= 2 * sm_count()) node_f64_launch<ADV, 1>(g, fs, st);
+    else if (g.nnodes <= 16 * sm_count() || g.QX2 > 64) node_f64_launch<ADV, 8>(g, fs, st);
+    else node_f64_launch<ADV, 16>(g, fs, st);
+}
+
+void launch_node_f64(int adv, const GroupDev& g, const void* fs, cudaStream_t st) {
     const double* f = static_cast<const double*>(fs);
-    if (adv == HLB_WENO5_) {
-        if (NB == 1) launch_dependent(g.pdl, node_f64_kernel<HLB_WENO5_, 1>, grid, kNode64T, smem, st, g, f);
-        else launch_dependent(g.pdl, node_f64_kernel<HLB_WENO5_, 8>, grid, kNode64T, smem, st, g, f);
-    } else {
-        if (NB == 1) launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 1>, grid, kNode64T, smem, st, g, f);
-        else launch_dependent(g.pdl, node_f64_kernel<HLB_UPWIND2_, 8>, grid, kNode64T, smem, st, g, f);
-    }
+    if (adv == HLB_WENO5_) node_f64_dispatch<HLB_WENO5_>(g, f, st);
+    else node_f64_dispatch<HLB_UPWIND2_>(g, f, st);
 }
 
 // Node pass of a stage of the FP32 groups that the one-launch pass does not
