@@ -262,7 +262,8 @@ hlb_status hlb_set_state_dev(hlb_handle* h, const void* f_dev, size_t bytes);
  * group that runs them, times the three stage launches of one step for the
  * built-in x-segment length and for half, one, two and four times the present
  * one, rounded up to multiples of 6 cells from 12 on (CUDA events on the
- * handle's stream, one untimed round, three timed) and keeps the fastest; for
+ * handle's stream, one untimed round, three timed) and keeps the fastest, but
+ * the built-in one where whole steps with it are as fast; for
  * groups on the persistent kernel, whole persistent steps for segment items of
  * 24 to 264 cells, and of the built-in length where that is shorter, times one
  * or half the resident CTAs per SM.  The state is only read (the launches write the two scratch

@@ -1741,8 +1741,8 @@ hlb_status tune_persist(hlb_handle* h, Group& G, EventPair& ev, int* chosen, flo
 // back, so the state is kept.
 hlb_status time_per_stage_step(hlb_handle* h, Group& G, EventPair& ev, float* step_ms) {
     const int cur = G.cur, prev = G.prev;
-    const bool use = G.persist_use;
-    G.persist_use = false;
+    const bool use = G.persist_use, timed = h->time_kernels;
+    G.persist_use = h->time_kernels = false;
     for (int round = 0; round < 4; ++round) {
         if (round == 1) cudaEventRecord(ev.e0, h->stream);
         enqueue_group_step(h, G, h->stream);
@@ -1751,6 +1751,7 @@ hlb_status time_per_stage_step(hlb_handle* h, Group& G, EventPair& ev, float* st
     }
     cudaEventRecord(ev.e1, h->stream);
     G.persist_use = use;
+    h->time_kernels = timed;
     float ms = 0.0f;
     cudaError_t e = cudaEventSynchronize(ev.e1);
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev.e0, ev.e1);
@@ -1791,8 +1792,9 @@ hlb_status tune_group(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
 hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen) {
     // The built-in length, which is the shortest for groups of less than a wave,
     // and half, one, two and four times the present one as multiples of 6 cells
-    // from 12 on.  Stage kernels only, so that the node pass does not hide the
-    // difference.  us per step, tuned among the multiples of 6 alone against the
+    // from 12 on.  Stage kernels first, so that the node pass does not hide the
+    // difference; a length that beats the built-in one there has to do so over whole
+    // steps too (the launches overlap).  us per step, tuned among the multiples of 6 alone against the
     // built-in length (GB300): 95 x 61 cells of 128 FP64 velocities 1252 (12
     // cells) against 795 (4), 60 x 40 of 128 FP32 72.6 against 53.3, 512 cells of
     // 128 39.2 against 31.4.
@@ -1832,6 +1834,13 @@ hlb_status tune_group_stages(hlb_handle* h, Group& G, EventPair& ev, int* chosen
         if (e != cudaSuccess) { s = fail(HLB_ECUDA, std::string("autotune timing: ") + cudaGetErrorString(e)); break; }
         if (best_ms < 0.0f || ms < best_ms) { best_ms = ms; best = sx; }
         if (c < multiples && (best_timed_ms < 0.0f || ms < best_timed_ms)) { best_timed_ms = ms; best_timed = sx; }
+    }
+    if (s == HLB_OK && best != G.SX_builtin) {
+        float ms_builtin = 0.0f, ms_best = 0.0f;
+        if ((s = set_segments(h, G, G.SX_builtin)) == HLB_OK && (s = time_per_stage_step(h, G, ev, &ms_builtin)) == HLB_OK &&
+            (s = set_segments(h, G, best)) == HLB_OK && (s = time_per_stage_step(h, G, ev, &ms_best)) == HLB_OK &&
+            ms_builtin <= ms_best)
+            best = G.SX_builtin;
     }
     // the chosen length (the one before after an error), or no marching at all
     const hlb_status s2 = set_segments(h, G, s == HLB_OK ? best : base);
