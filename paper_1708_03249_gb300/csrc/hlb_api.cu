@@ -735,12 +735,12 @@ hlb_status build_group(hlb_handle* h, Group& G) {
             // the force term's form (set above): on the tensor cores where the
             // caller asked for it and the slab tiles into 16 x 8 x 8 blocks;
             // by default where 3xTF32 measured faster than the FMA loop on a
-            // GB300: the 1D kernel's 32 x 16 slabs (0.412 against 0.523 ms
+            // GB300: the 1D kernel's 32 x 16 slabs (0.385 against 0.495 ms
             // per stage, 131072 cells) and the 2D kernel's 16 x 8 slabs with
-            // upwind2 (2.06 against 2.39 ms, 1024 x 512 cells, 1024
+            // upwind2 (2.07 against 2.40 ms, 1024 x 512 cells, 1024
             // velocities); with WENO-5 the 2D kernel is issue-bound and the
-            // FMA loop is faster (3.43 against 3.64 ms; 32 x 16: 0.330
-            // against 0.347 ms)
+            // FMA loop is faster (2.90 against 3.14 ms; 32 x 16: 0.289
+            // against 0.315 ms)
             HLB_CUDA(hlb::prepare_march(G.precision, G.adv, G.QX2, G.VY, G.TY, G.force_form));
         }
     }
@@ -754,20 +754,19 @@ hlb_status build_group(hlb_handle* h, Group& G) {
                    (G.TY == 1 || G.nnodes > 256);
     if (G.march_ok && G.precision == HLB_FP32 && !G.node_fused) HLB_CUDA(hlb::prepare_node());
 
-    // launch shape of the stage kernel.  With Kx in global memory each
-    // velocity's force term is a 2Qx-term dot product (FP64), so the velocities
-    // of a node are split over several CTAs (the balanced split below); the
-    // CTAs of one node form its moments redundantly.
+    // launch shape of the generic stage kernel.  With Kx in global memory (the
+    // order-200 sets in 2D) each velocity's force term is a 2Qx-term dot product
+    // (FP64), so the velocities of a node are split over several CTAs; each
+    // reads the node's factor line.
     int per_sm = 1, dev = 0, nsm = 1;
     HLB_CUDA(cudaGetDevice(&dev));
     HLB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     G.vchunks = 1;
     auto block_of = [&](int vc) { return std::min(256, std::max(32, ((G.V + vc - 1) / vc + 31) / 32 * 32)); };
     if (G.d_KxT.p) {
-        // about 64 velocities per CTA at most, and enough CTAs for the two per
-        // SM the stage kernel is compiled for (measured against a split that
-        // minimised rounds times CTA size: 0.0927 against 0.0985 ms per stage
-        // launch on the eight-case order-200 handle)
+        // at least 64 velocities per CTA, and no more CTAs than the two per SM
+        // the kernel is compiled for.  us per stage, split against whole nodes
+        // (400 velocities, GB300): 12 x 3 cells 28 / 56, 24 x 3 41 / 56, 24 x 6 60 / 56
         const int by_size = (G.V + 63) / 64;
         const int by_fill = (2 * nsm + G.nnodes - 1) / G.nnodes;
         G.vchunks = std::max(1, std::min(by_size, by_fill));

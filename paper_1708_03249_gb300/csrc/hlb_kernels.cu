@@ -124,14 +124,13 @@ __device__ __forceinline__ void face_pair(const R* w, bool pos, R& Fp, R& Fm) {
 // ---------------------------------------------------------------------------
 // stage kernel
 // ---------------------------------------------------------------------------
-// CTAs per SM the generic stage kernel is compiled for (2: at most 128
-// registers per thread, so that two 256-thread CTAs fit an SM; on the order-200
-// set 0.0927 ms per stage launch against 0.0989 ms at 1, eight ballistic cases).
-#ifndef HLB_STAGE_MIN_BLOCKS
-#define HLB_STAGE_MIN_BLOCKS 2
-#endif
+// CTAs per SM the generic stage kernel is compiled for: two, at most 128
+// registers per thread.  us per stage against one (GB300): 24 x 6 cells of 400
+// FP64 velocities 60 / 78, 24 x 40 314 / 357; 64 x 64 of 1024 FP32 velocities with a
+// force along p_z 548 / 875.
+constexpr int kStageMinBlocks = 2;
 template <typename R, int ADV>
-__global__ void __launch_bounds__(256, HLB_STAGE_MIN_BLOCKS)
+__global__ void __launch_bounds__(256, kStageMinBlocks)
 stage_kernel(const GroupDev g, const R* __restrict__ fs, const R* __restrict__ fn,
              R* __restrict__ fo, int stage) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -615,7 +614,8 @@ wall_kernel(const GroupDev g, const R* __restrict__ fs) {
 // points while |u_x| <= 2 sqrt(T); beyond the end g h_l is below 1e-17 of its
 // maximum for l <= 31; 3.7e-15 of max |G| at order 20 against a 30-point rule on
 // panels of 0.1 sqrt(T) in extended precision, 3.8e-15 with 20 points on panels of
-// sqrt(T)), h_l(p) by the three-term recurrence of the orthonormal basis
+// sqrt(T); 2.6e-14 at orders 20 and 31 over T from 0.05 to 30 and |u_x| up to 5, the
+// rounding of the FP64 recurrence), h_l(p) by the three-term recurrence of the orthonormal basis
 // (forward evaluation at a point is stable).  The integration-by-parts
 // recurrence of node_coefficients carries its rounding (and that of its erf
 // and exp start) along a solution that grows about threefold per order:

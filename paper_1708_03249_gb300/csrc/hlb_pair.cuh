@@ -43,7 +43,7 @@ constexpr int kPairDepth = HLB_PAIR_DEPTH;   // pairs of cells in flight (copy b
 // f32x2 pairs in shared memory), or warp-level tensor-core products (3xTF32
 // or split-BF16, hlb_device.cuh) when both contractions tile into 16 x 8 x 8
 // blocks.  On the 1024 x 512 channel with 16 x 8 x 8 velocities the 3xTF32
-// form measured 3.74 ms per stage launch against 3.51 ms for the FMA loop (the
+// form measured 3.14 ms per stage launch against 2.90 ms for the FMA loop (the
 // fragment loads, splits and stores cost more issue slots than the packed
 // FMAs they replace); the library picks the form per velocity set.
 template <int QX2, int VY, int FM>
@@ -150,7 +150,7 @@ march_pair_kernel(const GroupDev g, const Work* __restrict__ works, const float*
     const int slab = kz * S;
     const uint32_t row_bytes = S * sizeof(float);
 
-    // producer (warp 0, one copy per lane): the inputs of pair p into buffer p % kPairDepth
+    // the copies of pair p go into buffer p % kPairDepth
     // Copy `lane` of pair p (22 lanes: 12 halo rows, 4 head rows, 4 f^n rows,
     // 2 factor-line runs): source, bytes and destination in B; false if the
     // lane has none for this pair.
