@@ -4,7 +4,6 @@ schemes, a collisionless group, a force field).  Tolerance of test_gpu_parity:
 1e-10 of max |f| up to order 8."""
 import math
 
-import numpy as np
 import pytest
 
 from paper_1708_03249_gb300 import workloads as W
